@@ -307,14 +307,15 @@ const char* fb_kernel_name(int kind);
  * dimension N. impl: 0 = automatic (tcgen05 when N % 128 == 0 and K % 64 == 0: the
  * 2-SM cta_group::2 kernel when N % 256 == 0, else the 1-SM kernel), 1 = force the
  * CUDA-core kernel, 2 = force the 1-SM tcgen05 kernel (same shape rules), 3 = the 2-SM
- * kernel over whole 256 x 256 tiles only, 4 = the 2-SM kernel with the stream-K split:
- * every SM pair takes an equal share of the (tile, 64-wide K block) units and tiles cut
- * between pairs are summed from fp32 partials in the model's workspace, in K order (so
- * the result does not depend on timing). impl 4 needs N % 256 == 0 and at least 4 K
- * blocks per SM pair (ceil(M / 256) * N / 256 * K / 64 >= 4 * pairs), else FB_ECUDA;
- * impl 0 takes the stream-K split only when K >= 96 * 64 and the whole 256 x 256 tiles
- * number fewer than the SM pairs that can be resident (e.g. 1560 x 1536 x 8960), whole
- * tiles otherwise. */
+ * kernel over whole tiles only (256 output features x T rows, T a multiple of 16 up to 256
+ * fitted to M), 4 = the 2-SM kernel with the stream-K split: every SM pair takes an equal
+ * share of the (256 x 256 tile, 64-wide K block) units and tiles cut between pairs are
+ * summed from fp32 partials in the model's workspace, in K order (so the result does not
+ * depend on timing). impl 4 needs N % 256 == 0 and at least 4 K blocks per SM pair
+ * (ceil(M / 256) * N / 256 * K / 64 >= 4 * pairs), else FB_ECUDA; impl 0 takes the
+ * stream-K split only when the 256 x 256 tiles fill at most 4 rounds of the resident SM
+ * pairs and leave at least 24 K blocks per pair idle in the last (e.g. 1560 x 1536 x 8960),
+ * whole tiles otherwise. */
 /* fb_set_op_repeat: fb_op_gemm / fb_op_attention launch their kernel n >= 1 times back
  * to back (default 1), for timing a kernel without a stream synchronisation per launch. */
 fb_status fb_set_op_repeat(fb_model* m, int n);

@@ -317,8 +317,9 @@ fb_status end_call(fb_model* m) {
 
 // ---- kernel wrappers with statistics ------------------------------------------------
 // impl: 0 automatic, 1 CUDA-core kernel, 2 the 1-SM tcgen05 kernel, 3 the 2-SM kernel
-// over whole tiles, 4 the 2-SM kernel with the stream-K split
-fb_status run_gemm(fb_model* m, const GemmArgs& g0, int impl = 0) {
+// over whole tiles, 4 the 2-SM kernel with the stream-K split. The model's own launches take
+// the tcgen05 kernels over whole tiles where the shape allows (3).
+fb_status run_gemm(fb_model* m, const GemmArgs& g0, int impl = 3) {
   GemmArgs g = g0;
   g.sk_ws = m->sk_ws;
   g.sk_ctr = m->sk_ctr;

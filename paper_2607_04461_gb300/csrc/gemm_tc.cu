@@ -42,18 +42,6 @@ struct TcCfg {
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/;
 };
 
-// Shared-memory matrix descriptor: K-major, 128-byte swizzle; 8-row core-matrix groups
-// are 1024 bytes apart (stride byte offset); leading byte offset unused for this layout.
-__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;                 // leading byte offset (16 B, ignored)
-  d |= (uint64_t)(1024 >> 4) << 32;       // stride byte offset
-  d |= (uint64_t)1 << 46;                 // descriptor version (tcgen05)
-  d |= (uint64_t)2 << 61;                 // layout: 128-byte swizzle
-  return d;
-}
-
 // Instruction descriptor, kind::f16: D fp32, A and B bf16, both K-major, M=128, N=BN.
 template <int BN>
 __device__ __forceinline__ uint32_t idesc_bf16() {
@@ -102,81 +90,78 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   const uint32_t tmem_base = *tmem_holder;
   // The weights do not depend on the previous kernel: the producer starts loading the W
   // tiles of its first tile's first stages before waiting for its predecessor.
-  const int pre = (warp == 0 && lane == 0 && (int)blockIdx.x < n_tiles)
-                      ? (nk < C::STAGES ? nk : C::STAGES) : 0;
-  for (int kb = 0; kb < pre; ++kb) {
-    uint8_t* sa = smem + kb * C::STAGE_BYTES;
-    mbar_expect_tx(&full[kb], C::STAGE_BYTES);
-    tma_load_2d(sa + C::A_BYTES, &tmW, &full[kb], kb * BK, ((int)blockIdx.x % n_nt) * BN);
-  }
+  const int pre = (int)blockIdx.x < n_tiles ? (nk < C::STAGES ? nk : C::STAGES) : 0;
+  if (warp == 0 && elect_one())
+    for (int kb = 0; kb < pre; ++kb) {
+      uint8_t* sa = smem + kb * C::STAGE_BYTES;
+      mbar_expect_tx(&full[kb], C::STAGE_BYTES);
+      tma_load_2d(sa + C::A_BYTES, &tmW, &full[kb], kb * BK, ((int)blockIdx.x % n_nt) * BN);
+    }
   griddep_wait();  // inputs written by the previous kernel are visible from here on
   griddep_launch();
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer ----------------
-      int stage = 0;
-      uint32_t phase = 0;
-      uint32_t issued[C::STAGES];
-#pragma unroll
-      for (int s = 0; s < C::STAGES; ++s) issued[s] = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-        const int m0 = (tile / n_nt) * BM, n0 = (tile % n_nt) * BN;
-        for (int kb = 0; kb < nk; ++kb) {
-          uint8_t* sa = smem + stage * C::STAGE_BYTES;
-          if (tile == (int)blockIdx.x && kb < pre) {
-            tma_load_2d(sa, &tmA, &full[stage], kb * BK, m0);  // W already requested
-          } else {
-            if (!mbar_wait(&empty[stage], phase ^ 1u, err)) { ok = false; break; }
+    // ---------------- TMA producer ----------------
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    int issued = 0;  // loads' K blocks so far
+    for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+      const int m0 = (tile / n_nt) * BM, n0 = (tile % n_nt) * BN;
+      for (int kb = 0; kb < nk; ++kb) {
+        uint8_t* sa = smem + stage * C::STAGE_BYTES;
+        const bool have_w = tile == (int)blockIdx.x && kb < pre;  // W already requested
+        if (!have_w && !mbar_wait_warp(&empty[stage], phase ^ 1u, err)) { ok = false; break; }
+        if (elect_one()) {
+          if (!have_w) {
             mbar_expect_tx(&full[stage], C::STAGE_BYTES);
-            tma_load_2d(sa, &tmA, &full[stage], kb * BK, m0);
             tma_load_2d(sa + C::A_BYTES, &tmW, &full[stage], kb * BK, n0);
           }
-          ++issued[stage];
-          if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+          tma_load_2d(sa, &tmA, &full[stage], kb * BK, m0);
         }
+        ++issued;
+        if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
       }
-      if (!ok) {
-        // Let this CTA's loads in flight land before the CTA exits.
-        for (int s = 0; s < C::STAGES; ++s)
-          if (issued[s]) {
-            const uint32_t a = smem_u32(&full[s]);
-            const uint64_t t0 = fb_globaltimer();
-            while (!mbar_try(a, (issued[s] - 1) & 1u) &&
-                   fb_globaltimer() - t0 < fb_wait_limit()) {
-            }
-          }
+    }
+    if (!ok && lane == 0) {
+      // Let this CTA's loads in flight land before the CTA exits: the last use of every
+      // stage so far (stage s's u-th use completes phase u - 1 of its barrier).
+      for (int s = 0; s < C::STAGES && s < issued; ++s) {
+        const int uses = (issued - s + C::STAGES - 1) / C::STAGES;
+        const uint32_t a = smem_u32(&full[s]);
+        const uint64_t t0 = fb_globaltimer();
+        while (!mbar_try(a, (uses - 1) & 1u) && fb_globaltimer() - t0 < fb_wait_limit()) {
+        }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      const uint32_t idesc = idesc_bf16<BN>();
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      int it = 0;
-      for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++it) {
-        const int acc = it & 1;
-        const uint32_t acc_phase = (it >> 1) & 1;
-        if (!mbar_wait(&tmem_empty[acc], acc_phase ^ 1u, err)) break;
+    // ---------------- MMA issuer ----------------
+    const uint32_t idesc = idesc_bf16<BN>();
+    const uint32_t ring_lo = desc_lo_k(smem_u32(smem));
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    int it = 0;
+    for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++it) {
+      const int acc = it & 1;
+      const uint32_t acc_phase = (it >> 1) & 1;
+      if (!mbar_wait_warp(&tmem_empty[acc], acc_phase ^ 1u, err)) break;
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + acc * BN;
+      for (int kb = 0; kb < nk; ++kb) {
+        if (!mbar_wait_warp(&full[stage], phase, err)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * BN;
-        for (int kb = 0; kb < nk; ++kb) {
-          if (!mbar_wait(&full[stage], phase, err)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t sa = smem_u32(smem + stage * C::STAGE_BYTES);
-          const uint64_t adesc = sdesc_sw128(sa), bdesc = sdesc_sw128(sa + C::A_BYTES);
+        const uint32_t alo = ring_lo + (uint32_t)stage * (C::STAGE_BYTES >> 4);
+        const uint32_t blo = alo + (C::A_BYTES >> 4);
+        if (elect_one()) {
+          // +32 bytes per K=16 step inside the swizzle row (encoded >> 4 -> +2)
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            // +32 bytes per K=16 step inside the swizzle row (encoded >> 4 -> +2)
-            tc_mma_f16(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, (kb | k) ? 1u : 0u);
-          }
+          for (int k = 0; k < BK / 16; ++k)
+            tc_mma_ss_lo(d_tmem, alo + 2 * k, blo + 2 * k, DESC_HI, idesc, (kb | k) ? 1u : 0u);
           tc_commit(&empty[stage]);
-          if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+          if (kb + 1 == nk) tc_commit(&tmem_full[acc]);
         }
-        if (ok) tc_commit(&tmem_full[acc]);
+        if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
       }
     }
   } else {
@@ -224,83 +209,45 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 }
 
 // ---- 2-SM variant -------------------------------------------------------------------
-// A cluster of two CTAs computes a 256 x 256 tile with tcgen05.mma.cta_group::2: CTA r
-// of the pair holds rows 128 r .. 128 r + 127 of the A tile and rows 128 r .. of the W
-// tile in its shared memory, and receives rows 128 r .. of the accumulator in its TMEM.
-// Per SM this moves 32 KB per K block instead of 48 KB for the same MMA work, so six
-// stages fit. The even CTA issues the MMAs; its "full" barriers count the TMA bytes of
-// both CTAs (the odd CTA's loads complete on them across the pair), its commits arrive on
-// the "empty" / "tmem_full" barriers of both CTAs, and both CTAs' epilogue warps release
-// an accumulator on its "tmem_empty" barrier.
-constexpr int C2_BN = 256;
-constexpr int C2_HALF_BYTES = 128 * BK * 2;          // 16 KB: 128 rows x 64 bf16
-constexpr int C2_STAGE_BYTES = 2 * C2_HALF_BYTES;    // this CTA's A rows + W rows
-constexpr int C2_TMEM_COLS = 2 * C2_BN;
-// Epilogues. bf16 outputs and the fp32 gated residual go through shared memory and TMA:
-// each epilogue warp owns two 32 x 32 tiles (bf16 64-byte rows with the 64-byte swizzle,
-// or fp32 128-byte rows with the 128-byte swizzle, so that one row per lane is read and
-// written at full shared-memory bandwidth), writes its results there and stores them with
-// a TMA bulk store that runs while it computes the next chunk; the fp32 residual tiles of
-// a chunk are loaded by TMA into the same tile, two chunks ahead, the first two before
-// the accumulator is ready. The residual + contribution epilogue (Delta) stages each
-// chunk in a [32][33] float tile per warp and moves whole 128-byte rows with plain loads
-// and stores. The epilogue space comes out of the operand ring where needed.
-constexpr int EPI_STAGE_FLOATS = 32 * 33;
+// A cluster of two CTAs computes a tile of 256 output features x T tokens (rows of A) with
+// tcgen05.mma.cta_group::2: the features are the MMA's M dimension (256, CTA r of the pair
+// holds features 128 r .. 128 r + 127 of the W tile and receives their accumulators in its
+// TMEM, one feature per lane, one token per column), the tokens its N dimension (any
+// multiple of 16 up to 256; CTA r holds T / 2 of the A rows). The even CTA issues the MMAs;
+// its "full" barriers count the TMA bytes of both CTAs (the odd CTA's loads complete on
+// them across the pair), its commits arrive on the "empty" / "tmem_full" barriers of both
+// CTAs, and both CTAs' epilogue warps release an accumulator on its "tmem_empty" barrier.
+//
+// T is a launch parameter (see choose_tile): with the tokens along N the split follows the
+// row count in steps of 16, so that few rows (one candidate's 1560) neither leave SM pairs
+// idle nor compute padding. Stages and barriers are laid out for T at run time.
+constexpr int C2_BN = 256;                           // output features of a tile
+constexpr int C2_W_BYTES = 128 * BK * 2;             // 16 KB: this CTA's 128 W rows x 64 bf16
+constexpr int C2_TMEM_COLS = 512;                    // two accumulators of up to 256 tokens
+constexpr int C2_MAX_STAGES = 8;
+constexpr int C2_SMEM_BYTES = 232448;                // all of an SM's shared memory
+// Epilogue tiles and operand ring per epilogue: each of the 8 epilogue warps owns NBUF tiles
+// of CHUNK tokens x 32 features, through which results leave by TMA store and (fp32 residual)
+// residual rows arrive by TMA load. A chunk costs its warp about 300 clocks of buffer wait,
+// proxy fence and store issue, so the bf16 epilogues take 32 tokens at a time; the fp32 ones
+// take 16, which leaves the operand ring its stages.
 template <int KIND>
 struct C2Cfg {
-  static constexpr bool TMA_EPI = KIND != EPI_RESID_DELTA;
-  static constexpr bool STAGED = KIND == EPI_RESID_DELTA;
-  static constexpr int STAGES = KIND == EPI_BF16 || KIND == EPI_GELU_BF16 ? 6 : 5;
-  static constexpr int TILE_BYTES = KIND == EPI_RESID ? 32 * 32 * 4 : 32 * 32 * 2;
-  static constexpr int EPI_BYTES = TMA_EPI ? 8 * 2 * TILE_BYTES : 8 * EPI_STAGE_FLOATS * 4;
-  static constexpr int SMEM_BYTES = STAGES * C2_STAGE_BYTES + EPI_BYTES + 1024 + 512;
+  static constexpr bool F32 = KIND == EPI_RESID || KIND == EPI_RESID_DELTA;
+  static constexpr int CHUNK = F32 ? 16 : 32;
+  static constexpr int NBUF = F32 ? 3 : 2;
+  static constexpr int TILE_BYTES = CHUNK * 32 * (F32 ? 4 : 2);
+  static constexpr int EPI_BYTES = 8 * NBUF * TILE_BYTES;
+  static constexpr int RING_BYTES = C2_SMEM_BYTES - 1024 /*align*/ - 512 /*barriers*/ - EPI_BYTES;
 };
-static_assert(C2Cfg<EPI_BF16>::SMEM_BYTES <= 232448 && C2Cfg<EPI_RESID>::SMEM_BYTES <= 232448 &&
-                  C2Cfg<EPI_RESID_DELTA>::SMEM_BYTES <= 232448,
-              "2-SM GEMM shared memory");
-
-// byte offset of row r, 16-byte column chunk q in a TMA tile of 128-byte rows (128-byte
-// swizzle: chunk bits 4-6 of the address XOR bits 7-9) or 64-byte rows (64-byte swizzle:
-// bits 4-5 XOR bits 7-8); tiles start on 1024-byte boundaries
-__device__ __forceinline__ uint32_t swz128(int r, int q) { return r * 128 + ((q ^ (r & 7)) << 4); }
-__device__ __forceinline__ uint32_t swz64(int r, int q) { return r * 64 + ((q ^ ((r >> 1) & 3)) << 4); }
-
-// Staged residual epilogue of one warp for one 32 x 32 chunk: rows row0..row0+31 (the
-// warp's TMEM lane quarter), columns col0..col0+31; acc holds the thread's row (lane).
-template <int KIND>
-__device__ __forceinline__ void epi_resid_staged(const GemmEpi& e, float* stg, int lane,
-                                                 int row0, int col0, int M, const float* acc) {
-#pragma unroll
-  for (int j = 0; j < 32; ++j) stg[lane * 33 + j] = acc[j];
-  __syncwarp();
-  const int col = col0 + lane;
-  const float g = e.gate ? e.gate[col] : 1.f;
-  const float b = e.bias ? e.bias[col] : 0.f;
-  // all 32 rows' loads in flight before the first store (one memory latency per chunk)
-  constexpr int NB = KIND == EPI_RESID_DELTA ? 16 : 32;  // Delta: 32 would spill
-#pragma unroll 1
-  for (int r0 = 0; r0 < 32; r0 += NB) {
-    float rv[NB], bv[NB];
-#pragma unroll
-    for (int q = 0; q < NB; ++q) {
-      const int row = row0 + r0 + q;
-      const size_t off = (size_t)row * e.ldo + col;
-      rv[q] = row < M ? e.resid[off] : 0.f;
-      if (KIND == EPI_RESID_DELTA) bv[q] = row < M ? e.base[off] : 0.f;
-    }
-#pragma unroll
-    for (int q = 0; q < NB; ++q) {
-      const int row = row0 + r0 + q;
-      if (row < M) {
-        const size_t off = (size_t)row * e.ldo + col;
-        const float o = rv[q] + g * (stg[(r0 + q) * 33 + lane] + b);
-        if (KIND == EPI_RESID_DELTA) e.delta[off] = __float2bfloat16_rn(o - bv[q]);
-        reinterpret_cast<float*>(e.out)[off] = o;
-      }
-    }
-  }
-  __syncwarp();
+__host__ __device__ __forceinline__ int c2_stages(int T, int ring_bytes) {
+  const int n = ring_bytes / (C2_W_BYTES + T / 2 * BK * 2);
+  return n < C2_MAX_STAGES ? n : C2_MAX_STAGES;
 }
+// Warps: 0 and 10 load (even and odd K blocks: one warp needs about 370 clocks from a free
+// stage to its two TMA loads, more than the MMAs of a narrow tile's K block take, 288 at
+// T = 144), 1 issues the MMAs, 2-9 run the epilogue.
+constexpr int C2_THREADS = 352;
 
 // ---- work split of the 2-SM kernel --------------------------------------------------
 // Data-parallel: cluster c computes whole tiles c, c + G, c + 2G, ... (G clusters).
@@ -351,7 +298,7 @@ __device__ __forceinline__ int sk_owner(long long u, long long U, int G) {
 }
 // Workspace slot of cluster c's segment of `tile`: 2c for the first segment of its range,
 // 2c + 1 for the last (a range meets at most two cut tiles). Per slot and CTA of the pair,
-// 8 epilogue warps x 4096 floats: [chunk 4][j/4 8][lane 32][4], 32 rows x 128 columns.
+// 8 epilogue warps x 4096 floats: the warp's chunks of CH tokens [chunk][j/4][lane 32][4].
 __device__ __forceinline__ float* sk_part(float* ws, int c, int tile, long long U, int G, int nk,
                                           int rank, int we) {
   const int first_tile = (int)(((long long)c * U / G) / nk);
@@ -359,35 +306,68 @@ __device__ __forceinline__ float* sk_part(float* ws, int c, int tile, long long 
   return ws + ((size_t)(slot * 2 + rank) * 8 + we) * 4096;
 }
 
+// ---- epilogue of the 2-SM kernel ----------------------------------------------------
+// A lane owns one output feature, so bias and gate are one register each, and a warp's
+// access to one token of a shared-memory tile or of global memory is one row of 32
+// consecutive features (128 bytes of fp32: no bank conflicts without a swizzle). A warp
+// takes every other chunk of the tile's tokens. The residual chunks load two ahead, the
+// first ones while the mainloop runs; the contribution epilogue (Delta) reads the base rows
+// into registers one chunk ahead and stores the contribution directly.
+
+// Two tokens' values (j, j + 1) of each lane's feature as one 4-byte store per lane: lanes
+// exchange with their neighbour, even lanes then hold two adjacent features of token j,
+// odd lanes of token j + 1 (64 contiguous bytes per token and warp).
+__device__ __forceinline__ uint32_t pair_pack_bf16(float v0, float v1, int lane) {
+  const float got = __shfl_xor_sync(0xffffffffu, (lane & 1) ? v0 : v1, 1);
+  return (lane & 1) ? pack_bf16x2(got, v1) : pack_bf16x2(v0, got);
+}
+
+// CH (16 or 32) TMEM columns of this warp's lanes, waited for
+template <int CH>
+__device__ __forceinline__ void tmem_ld_chunk(uint32_t taddr, uint32_t* r) {
+  if (CH == 32) {
+    tmem_ld32(taddr, r);
+    tmem_ld_wait();
+    reg_fence32(r);
+  } else {
+    tmem_ld16(taddr, r);
+    tmem_ld_wait();
+    reg_fence16(r);
+  }
+}
+
 template <int KIND>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
     gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                     const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmR,
-                    int M, int N, int K, GemmEpi epi, SkArgs sk, int* err) {
+                    int M, int N, int K, int T, GemmEpi epi, SkArgs sk, int* err) {
   using CC = C2Cfg<KIND>;
-  constexpr int C2_STAGES = CC::STAGES;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* epi_smem = smem + C2_STAGES * C2_STAGE_BYTES;
-  float* epi_stage = reinterpret_cast<float*>(epi_smem);
+  // (RING_BYTES and EPI_BYTES are multiples of 512: tiles and barriers stay aligned)
+  uint8_t* epi_smem = smem + CC::RING_BYTES;
   uint64_t* full = reinterpret_cast<uint64_t*>(epi_smem + CC::EPI_BYTES);
-  uint64_t* empty = full + C2_STAGES;
-  uint64_t* tmem_full = empty + C2_STAGES;
+  uint64_t* empty = full + C2_MAX_STAGES;
+  uint64_t* tmem_full = empty + C2_MAX_STAGES;
   uint64_t* tmem_empty = tmem_full + 2;
-  uint64_t* rload = tmem_empty + 2;  // residual tile loads: 2 per epilogue warp
-  uint64_t* pload = rload + 16;     // stream-K finisher: one partial prefetch per epilogue warp
-  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(pload + 8);
+  uint64_t* pload = tmem_empty + 2;  // stream-K finisher: one partial prefetch per epilogue warp
+  uint64_t* rload = pload + 8;       // residual tile loads: NBUF per epilogue warp
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(rload + 8 * 3);
+  uint32_t* gave_up = tmem_holder + 1;  // a role of this CTA gave up a wait
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const uint32_t rank = cluster_ctarank();
   const int cluster = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
-  const int n_mt = (M + 2 * BM - 1) / (2 * BM), n_nt = N / C2_BN, n_tiles = n_mt * n_nt;
+  const int n_mt = (M + T - 1) / T, n_nt = N / C2_BN, n_tiles = n_mt * n_nt;
   const int nk = K / BK;
+  const int stage_bytes = C2_W_BYTES + T / 2 * BK * 2;
+  const int stages = c2_stages(T, CC::RING_BYTES);
   bool failed = false;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < C2_STAGES; ++s) {
+    *gave_up = 0;
+    for (int s = 0; s < stages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -395,13 +375,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       mbar_init(&tmem_full[a], 1);
       mbar_init(&tmem_empty[a], 16);  // 8 epilogue warps x 2 CTAs
     }
-    for (int b = 0; b < 16; ++b) mbar_init(&rload[b], 1);
     for (int b = 0; b < 8; ++b) mbar_init(&pload[b], 1);
+    for (int b = 0; b < 8 * 3; ++b) mbar_init(&rload[b], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmW);
-    if (CC::TMA_EPI) tma_prefetch_desc(&tmO);
-    if (KIND == EPI_RESID) tma_prefetch_desc(&tmR);
+    tma_prefetch_desc(&tmO);
+    if (CC::F32) tma_prefetch_desc(&tmR);
   }
   if (warp == 1) tmem_alloc_cg2(tmem_holder, C2_TMEM_COLS);
   tc_fence_before();
@@ -411,56 +391,60 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
   const bool use_sk = sk.on != 0;
   const long long U = (long long)n_tiles * nk;
   // As in the 1-SM kernel: W tiles of the first segment's first stages before the wait.
-  Seg first{0, 0, 0};
   int pre = 0;
-  if (warp == 0 && lane == 0) {
+  if (warp == 0 || warp == 10) {
     WorkIter w0(use_sk, cluster, n_clusters, n_tiles, nk);
+    Seg first;
     if (w0.next(first)) {
       const int len = first.kb1 - first.kb0;
-      pre = len < C2_STAGES ? len : C2_STAGES;
+      pre = len < stages ? len : stages;
+      const int n0 = (first.tile % n_nt) * C2_BN + 128 * (int)rank;
+      if (warp == 0 && elect_one())
+        for (int i = 0; i < pre; ++i) {
+          if (rank == 0) mbar_expect_tx(&full[i], 2 * stage_bytes);
+          tma_load_2d_cg2(smem + i * stage_bytes, &tmW, mapa_shared(smem_u32(&full[i]), 0),
+                          (first.kb0 + i) * BK, n0);
+        }
     }
-  }
-  for (int i = 0; i < pre; ++i) {
-    uint8_t* sa = smem + i * C2_STAGE_BYTES;
-    if (rank == 0) mbar_expect_tx(&full[i], 2 * C2_STAGE_BYTES);
-    tma_load_2d_cg2(sa + C2_HALF_BYTES, &tmW, mapa_shared(smem_u32(&full[i]), 0),
-                    (first.kb0 + i) * BK, (first.tile % n_nt) * C2_BN + 128 * (int)rank);
   }
   griddep_wait();
   // Dependents may start once every CTA of this grid has passed here: with the stream-K
   // split all contributors are then resident, so a finisher's wait cannot be starved.
   griddep_launch();
 
-  if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer (both CTAs) ----------------
-      int stage = 0;
-      uint32_t phase = 0;
-      WorkIter wi(use_sk, cluster, n_clusters, n_tiles, nk);
-      Seg sg;
-      for (int it = 0; !failed && wi.next(sg); ++it) {
-        const int m0 = (sg.tile / n_nt) * 2 * BM, n0 = (sg.tile % n_nt) * C2_BN;
-        for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
-          uint8_t* sa = smem + stage * C2_STAGE_BYTES;
+  if (warp == 0 || warp == 10) {
+    // ---------------- TMA producers (both CTAs) ----------------
+    int stage = 0;
+    uint32_t phase = 0;
+    bool mine = warp == 0;  // K blocks alternate between the two warps
+    WorkIter wi(use_sk, cluster, n_clusters, n_tiles, nk);
+    Seg sg;
+    for (int it = 0; !failed && wi.next(sg); ++it) {
+      const int m0 = (sg.tile / n_nt) * T + T / 2 * (int)rank;
+      const int n0 = (sg.tile % n_nt) * C2_BN + 128 * (int)rank;
+      for (int kb = sg.kb0; kb < sg.kb1; ++kb, mine = !mine) {
+        if (mine) {
+          uint8_t* sw = smem + stage * stage_bytes;
           const uint32_t fb = mapa_shared(smem_u32(&full[stage]), 0);
-          if (it == 0 && kb - sg.kb0 < pre) {  // W already requested before the wait
-            tma_load_2d_cg2(sa, &tmA, fb, kb * BK, m0 + BM * (int)rank);
-            if (++stage == C2_STAGES) { stage = 0; phase ^= 1u; }
-            continue;
+          const bool have_w = it == 0 && kb - sg.kb0 < pre;  // requested before the wait
+          if (!have_w && !mbar_wait_warp(&empty[stage], phase ^ 1u, err)) { failed = true; break; }
+          if (elect_one()) {
+            if (!have_w) {
+              if (rank == 0) mbar_expect_tx(&full[stage], 2 * stage_bytes);
+              tma_load_2d_cg2(sw, &tmW, fb, kb * BK, n0);
+            }
+            tma_load_2d_cg2(sw + C2_W_BYTES, &tmA, fb, kb * BK, m0);
           }
-          if (!mbar_wait(&empty[stage], phase ^ 1u, err)) { failed = true; break; }
-          if (rank == 0) mbar_expect_tx(&full[stage], 2 * C2_STAGE_BYTES);
-          tma_load_2d_cg2(sa, &tmA, fb, kb * BK, m0 + BM * (int)rank);
-          tma_load_2d_cg2(sa + C2_HALF_BYTES, &tmW, fb, kb * BK, n0 + 128 * (int)rank);
-          if (++stage == C2_STAGES) { stage = 0; phase ^= 1u; }
         }
+        if (++stage == stages) { stage = 0; phase ^= 1u; }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       // ---------------- MMA issuer (even CTA) ----------------
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) |
-                             ((uint32_t)(C2_BN >> 3) << 17) | ((uint32_t)((2 * BM) >> 4) << 24);
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(T >> 3) << 17) |
+                             ((uint32_t)(C2_BN >> 4) << 24);
+      const uint32_t ring_lo = desc_lo_k(smem_u32(smem));
       int stage = 0;
       uint32_t phase = 0;
       WorkIter wi(use_sk, cluster, n_clusters, n_tiles, nk);
@@ -468,30 +452,37 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       for (int it = 0; !failed && wi.next(sg); ++it) {
         const int acc = it & 1;
         const uint32_t acc_phase = (it >> 1) & 1;
-        if (!mbar_wait(&tmem_empty[acc], acc_phase ^ 1u, err)) { failed = true; break; }
+        if (!mbar_wait_warp(&tmem_empty[acc], acc_phase ^ 1u, err)) { failed = true; break; }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * C2_BN;
+        const uint32_t d_tmem = tmem_base + acc * 256;
         for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
-          if (!mbar_wait(&full[stage], phase, err)) { failed = true; break; }
+          if (!mbar_wait_warp(&full[stage], phase, err)) { failed = true; break; }
           tc_fence_after();
-          const uint32_t sa = smem_u32(smem + stage * C2_STAGE_BYTES);
-          const uint64_t adesc = sdesc_sw128(sa), bdesc = sdesc_sw128(sa + C2_HALF_BYTES);
+          const uint32_t wlo = ring_lo + (uint32_t)(stage * (stage_bytes >> 4));
+          const uint32_t alo = wlo + (C2_W_BYTES >> 4);
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k)
-            tc_mma_f16_cg2(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc,
-                           (kb > sg.kb0 || k > 0) ? 1u : 0u);
-          tc_commit_mc(&empty[stage], 0x3);
-          if (++stage == C2_STAGES) { stage = 0; phase ^= 1u; }
+            for (int k = 0; k < BK / 16; ++k)
+              tc_mma_cg2_lo(d_tmem, wlo + 2 * k, alo + 2 * k, DESC_HI, idesc,
+                            (kb > sg.kb0 || k > 0) ? 1u : 0u);
+            tc_commit_mc(&empty[stage], 0x3);
+            if (kb + 1 == sg.kb1) tc_commit_mc(&tmem_full[acc], 0x3);
+          }
+          if (++stage == stages) { stage = 0; phase ^= 1u; }
         }
-        if (!failed) tc_commit_mc(&tmem_full[acc], 0x3);
       }
     }
   } else {
     // ---------------- epilogue (warps 2..9 of both CTAs) ----------------
+    // warp: features quarter * 32 .. + 31 of this CTA's 128 (its TMEM lanes), every other
+    // 16-token chunk of the tile
     const int quarter = warp & 3, half = (warp - 2) >> 2, we = warp - 2;
     const uint32_t te_remote = mapa_shared(smem_u32(&tmem_empty[0]), 0);
-    uint8_t* wtiles = epi_smem + we * 2 * CC::TILE_BYTES;  // this warp's two TMA tiles
-    uint32_t rl_phase = 0;                                 // bit b: parity of tile b's load
+    constexpr int NBUF = CC::NBUF, CH = CC::CHUNK;
+    const bool has_r = CC::F32 && epi.resid != nullptr;
+    uint8_t* wtiles = epi_smem + we * NBUF * CC::TILE_BYTES;
+    uint64_t* wload = rload + we * 3;
+    uint32_t rl_phase = 0;  // bit b: parity of tile b's next load
     WorkIter wi(use_sk, cluster, n_clusters, n_tiles, nk);
     Seg sg;
     for (int it = 0; wi.next(sg); ++it) {
@@ -499,50 +490,43 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
       const uint32_t acc_phase = (it >> 1) & 1;
       const int tile = sg.tile;
       const bool whole = sg.kb0 == 0 && sg.kb1 == nk;
-      const int m0 = (tile / n_nt) * 2 * BM, n0 = (tile % n_nt) * C2_BN;
-      const int prow = m0 + BM * (int)rank + quarter * 32 + lane;
-      const int row0 = m0 + BM * (int)rank + quarter * 32;
-      // residual chunk cc of this warp's rows into tile cc % 2 (one lane)
-      auto rload_issue = [&](int cc) {
-        const int b = cc & 1;
-        mbar_expect_tx(&rload[2 * we + b], CC::TILE_BYTES);
-        tma_load_2d(wtiles + b * CC::TILE_BYTES, &tmR, &rload[2 * we + b],
-                    n0 + (half * 4 + cc) * 32, row0);
-      };
-      // bias and gate of this warp's four chunks, one column per lane, requested before
-      // the accumulator is ready (the chunks broadcast them with shuffles)
-      const int ecol = n0 + half * 128 + lane;
-      const float eb0 = epi.bias ? __ldg(epi.bias + ecol) : 0.f;
-      const float eb1 = epi.bias ? __ldg(epi.bias + ecol + 32) : 0.f;
-      const float eb2 = epi.bias ? __ldg(epi.bias + ecol + 64) : 0.f;
-      const float eb3 = epi.bias ? __ldg(epi.bias + ecol + 96) : 0.f;
-      const bool has_gate = KIND == EPI_RESID && epi.gate;
-      const float eg0 = has_gate ? __ldg(epi.gate + ecol) : 1.f;
-      const float eg1 = has_gate ? __ldg(epi.gate + ecol + 32) : 1.f;
-      const float eg2 = has_gate ? __ldg(epi.gate + ecol + 64) : 1.f;
-      const float eg3 = has_gate ? __ldg(epi.gate + ecol + 96) : 1.f;
       // the cluster holding K blocks 0.. of a cut tile finishes it (see the work split)
-      const bool head = !whole && sg.kb0 == 0;
-      // tiles this cluster finishes: the first two residual chunks load during the mainloop
-      const bool has_r = KIND == EPI_RESID && epi.resid != nullptr;
-      const bool early = has_r && (whole || head) && row0 < M;
-      if (early) {
-        if (lane == 0) {
-          bulk_wait_read<0>();
-          rload_issue(0);
-          rload_issue(1);
+      const bool head = sg.kb0 == 0;
+      const int m0 = (tile / n_nt) * T;
+      const int f0 = (tile % n_nt) * C2_BN + 128 * (int)rank + quarter * 32;
+      const int nv = M - m0 < T ? M - m0 : T;  // valid tokens of the tile
+      // this warp's chunks: i = 0, 1, ... covers tokens (half + 2 i) * CH ..
+      const int ncht = (nv + CH - 1) / CH, nch = (ncht + 1 - half) / 2;
+      const size_t off0 = (size_t)(m0 + half * CH) * epi.ldo + f0 + lane;
+      const float bias = head && epi.bias ? __ldg(epi.bias + f0 + lane) : 0.f;
+      const float gate = CC::F32 && head && epi.gate ? __ldg(epi.gate + f0 + lane) : 1.f;
+      // residual chunk i into tile i % NBUF (one lane)
+      auto rload_issue = [&](int i) {
+        const int t = i % NBUF;
+        mbar_expect_tx(&wload[t], CC::TILE_BYTES);
+        tma_load_2d(wtiles + t * CC::TILE_BYTES, &tmR, &wload[t], f0, m0 + (half + 2 * i) * CH);
+      };
+      float bv[16];
+      auto load_base = [&](int i) {  // Delta: base rows of chunk i
+        const int left = nv - (half + 2 * i) * CH;  // tokens from this chunk to the tile's end
+        const float* p = epi.base + off0 + (size_t)i * 2 * CH * epi.ldo;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) bv[j] = j < left ? __ldcg(p + (size_t)j * epi.ldo) : 0.f;
+      };
+      if (head && nch > 0) {
+        if (elect_one()) {
+          bulk_wait_read<0>();  // the previous output tile's stores have left the tiles
+          if (has_r) rload_issue(0);
+          if (has_r && nch > 1) rload_issue(1);
         }
         __syncwarp();
+        if (KIND == EPI_RESID_DELTA) load_base(0);
       }
-      // Delta epilogue, short-K tiles only: the rows into L2 (over a long mainloop the
-      // streamed operands would evict them)
-      if (CC::STAGED && whole && nk <= 48 && prow < M)
-        epi_prefetch<KIND>(epi, prow, n0 + half * (C2_BN / 2), C2_BN / 2);
       const bool ok = mbar_wait(&tmem_full[acc], acc_phase, err);
       if (!__all_sync(0xffffffffu, ok)) { failed = true; break; }
       tc_fence_after();
-      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * C2_BN;
-      bool finish = whole;
+      const uint32_t taddr =
+          tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * 256 + half * CH;
       int c_lo = 0, n_c = 1;
       if (!whole) {
         c_lo = sk_owner((long long)tile * nk, U, n_clusters);
@@ -550,20 +534,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
         int* ctr = sk.ctr + ((size_t)c_lo * 2 + rank) * 8 + we;
         if (!head) {
           // a later part of a cut tile: publish this warp's partial and count in
-          float* part = sk_part(sk.ws, cluster, tile, U, n_clusters, nk, (int)rank, we);
+          float4* part = reinterpret_cast<float4*>(
+                             sk_part(sk.ws, cluster, tile, U, n_clusters, nk, (int)rank, we)) + lane;
 #pragma unroll 1
-          for (int cc = 0; cc < 4; ++cc) {
-            uint32_t r[32];
-            tmem_ld32(taddr + (half * 4 + cc) * 32, r);
-            tmem_ld_wait();
-            reg_fence32(r);
-            float4* dst = reinterpret_cast<float4*>(part + cc * 1024) + lane;
+          for (int i = 0; i < nch; ++i) {
+            uint32_t r[CH];
+            tmem_ld_chunk<CH>(taddr + i * 2 * CH, r);
 #pragma unroll
-            for (int j4 = 0; j4 < 8; ++j4)
-              dst[j4 * 32] = make_float4(__uint_as_float(r[4 * j4]),
-                                         __uint_as_float(r[4 * j4 + 1]),
-                                         __uint_as_float(r[4 * j4 + 2]),
-                                         __uint_as_float(r[4 * j4 + 3]));
+            for (int j4 = 0; j4 < CH / 4; ++j4)
+              part[(i * (CH / 4) + j4) * 32] = make_float4(
+                  __uint_as_float(r[4 * j4]), __uint_as_float(r[4 * j4 + 1]),
+                  __uint_as_float(r[4 * j4 + 2]), __uint_as_float(r[4 * j4 + 3]));
           }
           __threadfence();
           __syncwarp();
@@ -591,162 +572,111 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
           ok2 = __shfl_sync(0xffffffffu, ok2, 0);
           if (!ok2) { failed = true; break; }
           __threadfence();
-          // The next contributor's partial (16 KB for this warp) into this warp's part of
-          // the operand ring, idle now: a head segment is the last of the cluster's range,
-          // so every MMA that read the ring has completed and no load follows. One bulk
-          // copy instead of a round trip per chunk below. Only for rows the chunk loop
-          // handles: that loop waits for the copy before the CTA can leave.
-          if (lane == 0 && row0 < M) {
-            fence_proxy_async_global();
-            mbar_expect_tx(&pload[we], 16384);
-            bulk_load_1d(smem + we * 16384,
-                         sk_part(sk.ws, c_lo + 1, tile, U, n_clusters, nk, (int)rank, we), 16384,
-                         &pload[we]);
+          // The next contributor's partial (up to 16 KB for this warp) into this warp's
+          // part of the operand ring, idle now: a head segment is the last of the
+          // cluster's range, so every MMA that read the ring has completed and no load
+          // follows. One bulk copy instead of a round trip per chunk below, which waits
+          // for it before the CTA can leave.
+          if (nch > 0) {
+            if (lane == 0) {
+              fence_proxy_async_global();
+              mbar_expect_tx(&pload[we], nch * CH * 128);
+              bulk_load_1d(smem + we * 16384,
+                           sk_part(sk.ws, c_lo + 1, tile, U, n_clusters, nk, (int)rank, we),
+                           nch * CH * 128, &pload[we]);
+            }
+            __syncwarp();
+            const bool pok = mbar_wait(&pload[we], 0, err);
+            if (!__all_sync(0xffffffffu, pok)) { failed = true; break; }
           }
-          __syncwarp();
-          finish = true;
         }
       }
-      if (finish && row0 < M) {
-        if (has_r && !early) {
-          if (lane == 0) {
-            bulk_wait_read<0>();
-            for (int cc = 0; cc < 2; ++cc) rload_issue(cc);
-          }
-          __syncwarp();
-        }
-#pragma unroll 1
-        for (int cc = 0; cc < 4; ++cc) {
-          const int c = half * 4 + cc;
-          float v[32];
-          if (whole) {
-            uint32_t r[32];
-            tmem_ld32(taddr + c * 32, r);
-            tmem_ld_wait();
-            reg_fence32(r);
+      if (head) {
+        // the chunk's sums: this cluster's accumulators, for a cut tile plus the other
+        // contributors' partials in K order (this cluster's is the first), the next one's
+        // from the copy in shared memory
+        auto chunk_sums = [&](int i, float* v) {
+          uint32_t r[CH];
+          tmem_ld_chunk<CH>(taddr + i * 2 * CH, r);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-          } else {
-            // the contributors' partials summed in K order, this cluster's from TMEM, the
-            // next one's from the copy in shared memory (waited for once, at chunk 0)
-            if (cc == 0) {
-              const bool pok = mbar_wait(&pload[we], 0, err);
-              if (!__all_sync(0xffffffffu, pok)) { failed = true; break; }
-            }
+          for (int j = 0; j < CH; ++j) v[j] = __uint_as_float(r[j]);
+          for (int q = 1; q < n_c; ++q) {
+            const float4* src =
+                reinterpret_cast<const float4*>(
+                    q == 1 ? reinterpret_cast<const float*>(smem + we * 16384)
+                           : sk_part(sk.ws, c_lo + q, tile, U, n_clusters, nk, (int)rank, we)) +
+                i * (CH * 8) + lane;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = 0.f;
-#pragma unroll 1
-            for (int q = 0; q < n_c; ++q) {
-              const int cq = c_lo + q;
-              if (cq == cluster) {
-                uint32_t r[32];
-                tmem_ld32(taddr + c * 32, r);
-                tmem_ld_wait();
-                reg_fence32(r);
-#pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] += __uint_as_float(r[j]);
-              } else if (cq == c_lo + 1) {  // shared memory: generic loads
-                const float4* src = reinterpret_cast<const float4*>(
-                                        reinterpret_cast<const float*>(smem + we * 16384) +
-                                        cc * 1024) + lane;
-#pragma unroll
-                for (int j4 = 0; j4 < 8; ++j4) {
-                  const float4 f = src[j4 * 32];
-                  v[4 * j4] += f.x;
-                  v[4 * j4 + 1] += f.y;
-                  v[4 * j4 + 2] += f.z;
-                  v[4 * j4 + 3] += f.w;
-                }
-              } else {
-                const float4* src = reinterpret_cast<const float4*>(
-                                        sk_part(sk.ws, cq, tile, U, n_clusters, nk, (int)rank, we) +
-                                        cc * 1024) + lane;
-#pragma unroll
-                for (int j4 = 0; j4 < 8; ++j4) {
-                  const float4 f = __ldcg(src + j4 * 32);
-                  v[4 * j4] += f.x;
-                  v[4 * j4 + 1] += f.y;
-                  v[4 * j4 + 2] += f.z;
-                  v[4 * j4 + 3] += f.w;
-                }
-              }
+            for (int j4 = 0; j4 < CH / 4; ++j4) {
+              const float4 f = q == 1 ? src[j4 * 32] : __ldcg(src + j4 * 32);
+              v[4 * j4] += f.x;
+              v[4 * j4 + 1] += f.y;
+              v[4 * j4 + 2] += f.z;
+              v[4 * j4 + 3] += f.w;
             }
           }
-          const int col0 = n0 + c * 32;
-          if (CC::STAGED) {
-            epi_resid_staged<KIND>(epi, epi_stage + we * EPI_STAGE_FLOATS, lane, row0, col0, M, v);
-            continue;
-          }
-          const int b = cc & 1;
+        };
+#pragma unroll 1
+        for (int i = 0; i < nch; ++i) {
+          float v[CH];
+          chunk_sums(i, v);
+          const int b = i % NBUF;
           uint8_t* tile_b = wtiles + b * CC::TILE_BYTES;
-          // this chunk's bias / gate (lane j holds column j; see eb / eg)
-          const float bl = cc == 0 ? eb0 : cc == 1 ? eb1 : cc == 2 ? eb2 : eb3;
-          const float gl = cc == 0 ? eg0 : cc == 1 ? eg1 : cc == 2 ? eg2 : eg3;
-          if (KIND == EPI_RESID) {
-            float4 rr[8];
+          if (CC::F32) {
+            float* tf = reinterpret_cast<float*>(tile_b) + lane;
             if (has_r) {
-              const bool lok = mbar_wait(&rload[2 * we + b], (rl_phase >> b) & 1u, err);
+              const bool lok = mbar_wait(&wload[b], (rl_phase >> b) & 1u, err);
               rl_phase ^= 1u << b;
               if (!__all_sync(0xffffffffu, lok)) { failed = true; break; }
-              // all eight residual loads first: a load after a store to the same tile
-              // would otherwise wait for it
 #pragma unroll
-              for (int j4 = 0; j4 < 8; ++j4)
-                rr[j4] = *reinterpret_cast<const float4*>(tile_b + swz128(lane, j4));
+              for (int j = 0; j < CH; ++j) v[j] = tf[j * 32] + gate * (v[j] + bias);
+              // tile (i + 2) % 3 was stored from one chunk ago: free for chunk i + 2
+              if (i + 2 < nch && elect_one()) {
+                bulk_wait_read<0>();
+                rload_issue(i + 2);
+              }
             } else {
-              // no residual: only the store issued from this tile two chunks ago must
-              // have left shared memory
-              if (lane == 0) bulk_wait_read<1>();
+              // no residual: the store from this tile three chunks ago has been read
+              if (elect_one()) bulk_wait_read<2>();
               __syncwarp();
 #pragma unroll
-              for (int j4 = 0; j4 < 8; ++j4) rr[j4] = make_float4(0.f, 0.f, 0.f, 0.f);
+              for (int j = 0; j < CH; ++j) v[j] = gate * (v[j] + bias);
             }
 #pragma unroll
-            for (int j4 = 0; j4 < 8; ++j4) {
-              float bb[4], gg[4];
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                bb[q] = __shfl_sync(0xffffffffu, bl, 4 * j4 + q);
-                gg[q] = __shfl_sync(0xffffffffu, gl, 4 * j4 + q);
-              }
-              rr[j4].x += gg[0] * (v[4 * j4] + bb[0]);
-              rr[j4].y += gg[1] * (v[4 * j4 + 1] + bb[1]);
-              rr[j4].z += gg[2] * (v[4 * j4 + 2] + bb[2]);
-              rr[j4].w += gg[3] * (v[4 * j4 + 3] + bb[3]);
-            }
-#pragma unroll
-            for (int j4 = 0; j4 < 8; ++j4)
-              *reinterpret_cast<float4*>(tile_b + swz128(lane, j4)) = rr[j4];
+            for (int j = 0; j < CH; ++j) tf[j * 32] = v[j];
           } else {
-            // the store issued from this tile two chunks ago has left shared memory (the
-            // one outstanding group allowed is the other tile's, one chunk ago)
-            if (lane == 0) bulk_wait_read<1>();
+            // the store from this tile two chunks ago has left shared memory
+            if (elect_one()) bulk_wait_read<1>();
             __syncwarp();
-            // bias by shuffle; GELU on packed fp32 pairs
+            uint32_t* tw = reinterpret_cast<uint32_t*>(tile_b) + (lane & 1) * 16 + (lane >> 1);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              uint32_t w[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                float y0 = v[8 * q + 2 * i] + __shfl_sync(0xffffffffu, bl, 8 * q + 2 * i);
-                float y1 = v[8 * q + 2 * i + 1] + __shfl_sync(0xffffffffu, bl, 8 * q + 2 * i + 1);
-                if (KIND == EPI_GELU_BF16) gelu_tanh_f2(y0, y1);
-                w[i] = pack_bf16x2(y0, y1);
-              }
-              *reinterpret_cast<uint4*>(tile_b + swz64(lane, q)) = make_uint4(w[0], w[1], w[2], w[3]);
+            for (int j = 0; j < CH; j += 2) {
+              float y0 = v[j] + bias, y1 = v[j + 1] + bias;
+              if (KIND == EPI_GELU_BF16) gelu_tanh_f2(y0, y1);
+              tw[j * 16] = pair_pack_bf16(y0, y1, lane);
             }
           }
           fence_proxy_async_smem();
           __syncwarp();
-          if (lane == 0) {
-            tma_store_2d(&tmO, smem_u32(tile_b), col0, row0);
+          if (elect_one()) {
+            // boxes of 16 tokens; a second one past the tile's end belongs to the next tile
+            const int t0 = (half + 2 * i) * CH;
+            tma_store_2d(&tmO, smem_u32(tile_b), f0, m0 + t0);
+            if (CH == 32 && t0 + 16 < nv)
+              tma_store_2d(&tmO, smem_u32(tile_b) + CC::TILE_BYTES / 2, f0, m0 + t0 + 16);
             bulk_commit();
-            if (has_r && cc + 2 < 4) {
-              bulk_wait_read<0>();  // the tile is free again: next residual chunk into it
-              rload_issue(cc + 2);
-            }
           }
-          __syncwarp();
+          if (KIND == EPI_RESID_DELTA) {
+            const int left = nv - (half + 2 * i) * CH;
+            bf16* dl = epi.delta + off0 + (size_t)i * 2 * CH * epi.ldo - lane + (lane & ~1) +
+                       (size_t)(lane & 1) * epi.ldo;
+#pragma unroll
+            for (int j = 0; j < CH; j += 2) {
+              const uint32_t w = pair_pack_bf16(v[j] - bv[j], v[j + 1] - bv[j + 1], lane);
+              if (j + (lane & 1) < left) *reinterpret_cast<uint32_t*>(dl + (size_t)j * epi.ldo) = w;
+            }
+            if (i + 1 < nch) load_base(i + 1);
+          }
         }
         if (failed) break;
       }
@@ -756,15 +686,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1)
     }
   }
 
-  if (CC::TMA_EPI && warp >= 2 && lane == 0) bulk_wait<0>();  // own TMA stores complete
-  if (failed || *(volatile int*)err != 0) {
+  // own TMA stores complete (one lane issued them all)
+  if (warp >= 2 && warp < 10 && elect_one()) bulk_wait<0>();
+  if (failed) *gave_up = 1;
+  tc_fence_before();
+  cluster_sync();
+  if (*gave_up != 0) {
     // After a timeout, give TMA loads that may still be in flight time to land before
-    // the shared memory they target is released (they complete within microseconds).
+    // the shared memory they target is released (they complete within microseconds). A CTA
+    // with loads in flight has unfinished tiles, so its own epilogue gave up too.
     const uint64_t t0 = fb_globaltimer();
     while (fb_globaltimer() - t0 < 100000ull) __nanosleep(1000);
   }
-  tc_fence_before();
-  cluster_sync();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc_cg2(tmem_base, C2_TMEM_COLS);
@@ -828,39 +761,50 @@ cudaError_t dispatch_kind(const GemmArgs& g, int* err, int num_sms, cudaStream_t
   return cudaErrorInvalidValue;
 }
 
-// 2-D map over an epilogue matrix [rows][cols] (row stride ld elements) with 32 x 32
-// boxes: fp32 with the 128-byte swizzle, bf16 with the 64-byte swizzle.
+// 2-D map over an epilogue matrix [rows][cols] (row stride ld elements) with 16 x 32 boxes
 bool make_epi_map(CUtensorMap* map, const void* ptr, bool f32, int rows, int cols, int ld) {
   auto enc = get_encode();
   if (!enc) return false;
   const size_t es = f32 ? 4 : 2;
   cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)ld * es};
-  cuuint32_t box[2] = {32, 32};
+  cuuint32_t box[2] = {32, 16};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = enc(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
                    2, const_cast<void*>(ptr), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   f32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
 
+// Token width T of the 2-SM kernel's tiles on mc SM pairs: the multiple of 16 with the least
+// estimated time in SM clocks. A K block's operands, 128 W rows and T / 2 token rows of 128
+// bytes per SM, arrive at about 64 bytes per clock and SM, 256 + T clocks, which is also the
+// MMAs' time (2 T) at T = 256 and more than it below; 313 clocks is the loading and issuing
+// threads' time per K block (163 ns at 64 to 160 tokens x 1536 x 8960). As many rounds as the
+// fullest pair has tiles, each its mainloop or, if that is longer, the epilogue (about 16
+// clocks per token) that runs beside it, and the last round's epilogue. Measured (us, chosen
+// T first): 1560 x 4608 x 1536 18.3 at T = 208 (20.4 at 256, 19.8 at 160), 1560 x 8960 x 1536
+// 29.7 at 208 (32.0 at 256), 1560 x 1536 x 1536 with residual 11.4 at 144 (14.9 at 256),
+// 1560 x 1536 x 8960 32.3 at 144 (46.2 at 256), 4096 x 1536 x 1536 18.8 at 176 (22.3 at 256),
+// 49920 x 1536 x 1536 185 at 256 (197 at 208).
+int choose_tile(int M, int N, int nk, int mc) {
+  int best_T = 256;
+  double best = 0;
+  for (int T = 256; T >= 16; T -= 16) {
+    const long tiles = (long)((M + T - 1) / T) * (N / C2_BN), rounds = (tiles + mc - 1) / mc;
+    const double main = (double)nk * (256 + T > 313 ? 256 + T : 313), epilogue = 16.0 * T + 400;
+    const double est = rounds * (main > epilogue ? main : epilogue) + epilogue;
+    if (best == 0 || est < best) {
+      best = est;
+      best_T = T;
+    }
+  }
+  return best_T;
+}
+
 template <int KIND>
 cudaError_t launch2(const GemmArgs& g, int* err, int num_sms, cudaStream_t st) {
-  CUtensorMap ma, mw, mo, mr;
-  memset(&mo, 0, sizeof(mo));
-  memset(&mr, 0, sizeof(mr));
-  if (!make_map(&ma, g.A, g.M, g.K, g.lda, BM) || !make_map(&mw, g.W, g.N, g.K, g.ldw, 128))
-    return cudaErrorInvalidValue;
-  if (C2Cfg<KIND>::TMA_EPI &&
-      !make_epi_map(&mo, g.epi.out, KIND == EPI_RESID, g.M, g.N, g.epi.ldo))
-    return cudaErrorInvalidValue;
-  mr = CUtensorMap{};  // unused without a residual
-  if (KIND == EPI_RESID && g.epi.resid &&
-      !make_epi_map(&mr, g.epi.resid, true, g.M, g.N, g.epi.ldo))
-    return cudaErrorInvalidValue;
-  constexpr int C2_SMEM_BYTES = C2Cfg<KIND>::SMEM_BYTES;
   cudaError_t e = cudaFuncSetAttribute(gemm_tc2_kernel<KIND>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, C2_SMEM_BYTES);
   if (e != cudaSuccess) return e;
@@ -871,7 +815,7 @@ cudaError_t launch2(const GemmArgs& g, int* err, int num_sms, cudaStream_t st) {
   if (occ == 0) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(num_sms, 1, 1);
-    cfg.blockDim = dim3(NUM_THREADS, 1, 1);
+    cfg.blockDim = dim3(C2_THREADS, 1, 1);
     cfg.dynamicSmemBytes = C2_SMEM_BYTES;
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, gemm_tc2_kernel<KIND>, &cfg) != cudaSuccess || n < 1) {
@@ -882,35 +826,36 @@ cudaError_t launch2(const GemmArgs& g, int* err, int num_sms, cudaStream_t st) {
     occ_clusters[KIND].store(n, std::memory_order_relaxed);
   }
   const int mc = occ < num_sms / 2 ? occ : num_sms / 2;
-  const int tiles = ((g.M + 2 * BM - 1) / (2 * BM)) * (g.N / C2_BN);
   const int nk = g.K / BK;
-  SkArgs sk{0, g.sk_ws, g.sk_ctr};
-  // Stream-K automatically only for a few rounds of tiles (<= 4) whose last round leaves
-  // at least 24 K blocks' worth of work per pair idle ((rounds - tiles / pairs) * nk >=
-  // 24), with A and W together within half of L2. There the idle pairs' share of the K
-  // loop outweighs writing and summing the partials of cut tiles. Measured on all 76
-  // pairs: 1560 x 1536 x 8960 gains (43.2 vs 47.9 us); a short K (1560 x 1536 x 1536:
-  // 22.9 vs 15.8 us) and 1560 x 8960 x 1536 (3.2 rounds: 41.4 vs 37.6 us) lose. The
-  // contiguous unit ranges spread each round over far-apart tiles, so operands larger
-  // than L2 are read several times: 8192 x 1536 x 8960 (2.5 rounds, A 147 MB) took 203
-  // us and 1.07 GB of DRAM reads against 156 us and 0.34 GB over whole tiles. On a
-  // partition of 20 pairs the 1560 x 1536 x 8960 shape's 42 tiles take 3 rounds, the
-  // last 90 % empty.
-  const long long U = (long long)tiles * nk;
-  const bool sk_ok = g.sk_ws && g.sk_ctr && mc <= g.sk_clusters && U >= 4LL * mc;
-  const int rounds = (tiles + mc - 1) / mc;
+  // Stream-K automatically (sk_mode 0, the single-op calls) only for a few rounds of
+  // 256 x 256 tiles (<= 4) whose last round leaves at least 24 K blocks' worth of work per
+  // pair idle ((rounds - tiles / pairs) * nk >= 24), with A and W together within half of
+  // L2: the cut tiles' partials are written and summed at a cost that a short K does not
+  // repay, and the contiguous unit ranges spread each round over far-apart tiles, so
+  // operands larger than L2 are read several times. The block's own launches use whole
+  // tiles (sk_mode 1): with the tile width fitted to the rows they are faster there
+  // (1560 x 1536 x 8960 on 76 pairs: 32.3 us over 66 tiles of T = 144, 43.0 us cut).
+  const long tiles256 = (long)((g.M + 255) / 256) * (g.N / C2_BN);
+  const long rounds256 = (tiles256 + mc - 1) / mc;
   const double operand_bytes = 2.0 * ((double)g.M + g.N) * g.K;
-  const bool sk_pays = rounds <= 4 && ((long long)rounds * mc - tiles) * nk >= 24LL * mc &&
+  const bool sk_ok =
+      g.sk_ws && g.sk_ctr && mc <= g.sk_clusters && tiles256 * (long long)nk >= 4LL * mc;
+  const bool sk_pays = rounds256 <= 4 && (rounds256 * mc - tiles256) * nk >= 24LL * mc &&
                        operand_bytes <= 64.0 * 1024 * 1024;
-  if (g.sk_mode == 2) {
-    if (!sk_ok) return cudaErrorInvalidValue;
-    sk.on = 1;
-  } else if (g.sk_mode == 0 && sk_ok && sk_pays) {
-    sk.on = 1;
-  }
+  if (g.sk_mode == 2 && !sk_ok) return cudaErrorInvalidValue;
+  SkArgs sk{g.sk_mode == 2 || (g.sk_mode == 0 && sk_ok && sk_pays) ? 1 : 0, g.sk_ws, g.sk_ctr};
+  // stream-K keeps T = 256: fewer tiles to cut and shorter K ranges to sum
+  const int T = sk.on ? 256 : choose_tile(g.M, g.N, nk, mc);
+  const int tiles = (g.M + T - 1) / T * (g.N / C2_BN);
+  CUtensorMap ma, mw, mo, mr{};  // mr: unused without a residual
+  if (!make_map(&ma, g.A, g.M, g.K, g.lda, T / 2) || !make_map(&mw, g.W, g.N, g.K, g.ldw, 128) ||
+      !make_epi_map(&mo, g.epi.out, C2Cfg<KIND>::F32, g.M, g.N, g.epi.ldo) ||
+      (C2Cfg<KIND>::F32 && g.epi.resid &&
+       !make_epi_map(&mr, g.epi.resid, true, g.M, g.N, g.epi.ldo)))
+    return cudaErrorInvalidValue;
   const int clusters = sk.on ? mc : (tiles < mc ? tiles : mc);
-  return launch_k(gemm_tc2_kernel<KIND>, dim3(2 * clusters), dim3(NUM_THREADS), C2_SMEM_BYTES, st,
-                  ma, mw, mo, mr, g.M, g.N, g.K, g.epi, sk, err);
+  return launch_k(gemm_tc2_kernel<KIND>, dim3(2 * clusters), dim3(C2_THREADS), C2_SMEM_BYTES, st,
+                  ma, mw, mo, mr, g.M, g.N, g.K, T, g.epi, sk, err);
 }
 
 cudaError_t dispatch2(const GemmArgs& g, int* err, int num_sms, cudaStream_t st) {
@@ -937,7 +882,7 @@ cudaError_t gemm_tc_set_wait_limit(unsigned long long ns) { return fb_set_wait_l
 
 cudaError_t gemm_tc(const GemmArgs& g, int* err, int num_sms, cudaStream_t st, bool force_1sm) {
   if (!gemm_tc_supported(g)) return cudaErrorInvalidValue;
-  // 2-SM 256 x 256 tiles whenever N allows; otherwise 1-SM 128 x BN tiles, BN = 256
+  // 2-SM tiles of 256 features x T tokens whenever N allows; otherwise 1-SM 128 x BN tiles, BN = 256
   // when that still gives every SM a tile.
   if (g.N % C2_BN == 0 && !force_1sm && num_sms >= 2) return dispatch2(g, err, num_sms, st);
   if (g.sk_mode == 2) return cudaErrorInvalidValue;  // stream-K exists in the 2-SM kernel only

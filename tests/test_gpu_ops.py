@@ -59,6 +59,40 @@ def test_gemm_tc_2sm_ragged_rows(model, M):
     _gemm_case(model, M, 512, 128, 0, impl=0)
 
 
+@pytest.mark.parametrize("M,N,K", [
+    (5, 256, 64),        # fewer rows than the narrowest tile, one K block
+    (100, 2304, 192),    # one token tile per feature tile, a ragged last chunk
+    (700, 1536, 320),    # narrow tiles, 5 K blocks (both loading warps, uneven)
+    (1560, 1536, 128),   # 11 token tiles, the last one partial
+    (1560, 4608, 640),   # two rounds
+    (2049, 512, 1536),   # one row in the last tile
+])
+@pytest.mark.parametrize("epi", [0, 1, 2, 3])
+def test_gemm_2sm_tile_widths(model, M, N, K, epi):
+    """The 2-SM kernel fits its tiles' token width to M: every width class, ragged last
+    tiles and chunks, against the fp64 product; rows past M stay untouched."""
+    A = randn((M, K), 71)
+    W = randn((N, K), 72, scale=K ** -0.5)
+    bias, gate = randn((N,), 73, dtype=torch.float32), randn((N,), 74, dtype=torch.float32)
+    resid = randn((M, N), 75, dtype=torch.float32) if epi >= 2 else None
+    base = randn((M, N), 76, dtype=torch.float32) if epi == 3 else None
+    out = torch.full((M + 32, N), 7.0, dtype=torch.float32 if epi >= 2 else torch.bfloat16,
+                     device="cuda")
+    delta = torch.full((M + 32, N), 7.0, dtype=torch.bfloat16, device="cuda")
+    fb.fb_op_gemm(model.handle, M, N, K, A, W, bias, epi, out, resid,
+                  gate if epi >= 2 else None, base, delta if epi == 3 else None, 3)
+    torch.cuda.synchronize()
+    assert torch.all(out[M:] == 7.0) and torch.all(delta[M:] == 7.0)
+    y = O.linear(f64(A), f64(W), f64(bias))
+    if epi < 2:
+        assert rel_max(f64(out[:M]), O.gelu_tanh(y) if epi else y) <= 1e-2   # bf16 output
+    else:
+        want = f64(resid) + f64(gate) * y
+        assert rel_max(f64(out[:M]), want) <= 1e-4
+        if epi == 3:
+            assert rel_max(f64(delta[:M]), want - f64(base)) <= 1e-2
+
+
 # Stream-K shapes: the refine pass's one-candidate projections (1560 rows), a few tiles
 # over a long K (13 pairs per tile), and two tiles over K = 9728 (about 38 pairs each).
 SK_SHAPES = [(1560, 1536, 1536), (1560, 1536, 8960), (1560, 8960, 1536), (1560, 4608, 1536),
