@@ -243,45 +243,45 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TB >> 3) << 17) |
-                               ((uint32_t)(TB >> 4) << 24);
-      const uint32_t idesc_pv = idesc_s | (1u << 16);  // B (V) is MN-major
-      const uint32_t dhi = DESC_HI;
-      const uint32_t q_lo = desc_lo_k(smem_u32(Qs)), p_lo = desc_lo_k(smem_u32(Ps));
-      const uint32_t k_lo = desc_lo_k(smem_u32(Ks)), v_lo = desc_lo_mn(smem_u32(Vs), SUB);
-      auto issue_s = [&](int j) {
-        const uint32_t ka = k_lo + (j % KSLOT) * (K_BYTES >> 4);
-        if (j + 1 < n_kv || last_nch == 4) {
+    // ---------------- MMA issuer ----------------
+    const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TB >> 3) << 17) |
+                             ((uint32_t)(TB >> 4) << 24);
+    const uint32_t idesc_pv = idesc_s | (1u << 16);  // B (V) is MN-major
+    const uint32_t dhi = DESC_HI;
+    const uint32_t q_lo = desc_lo_k(smem_u32(Qs)), p_lo = desc_lo_k(smem_u32(Ps));
+    const uint32_t k_lo = desc_lo_k(smem_u32(Ks)), v_lo = desc_lo_mn(smem_u32(Vs), SUB);
+    auto issue_s = [&](int j) {
+      const uint32_t ka = k_lo + (j % KSLOT) * (K_BYTES >> 4);
+      if (j + 1 < n_kv || last_nch == 4) {
 #pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint32_t off = ((kk >> 2) * SUB + (kk & 3) * 32) >> 4;
-            tc_mma_ss_lo(tmem + (j & 1) * TB, q_lo + off, ka + off, dhi, idesc_s, kk ? 1u : 0u);
-          }
-        } else {
-          const uint32_t idesc = idesc_keys(idesc_s, last_nch);
-#pragma unroll 1
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint32_t off = ((kk >> 2) * SUB + (kk & 3) * 32) >> 4;
-            tc_mma_ss_lo(tmem + (j & 1) * TB, q_lo + off, ka + off, dhi, idesc, kk ? 1u : 0u);
-          }
+        for (int kk = 0; kk < 8; ++kk) {
+          const uint32_t off = ((kk >> 2) * SUB + (kk & 3) * 32) >> 4;
+          tc_mma_ss_lo(tmem + (j & 1) * TB, q_lo + off, ka + off, dhi, idesc_s, kk ? 1u : 0u);
         }
-        tc_commit(&s_full[j & 1]);
-      };
-      if (mbar_wait(q_full, 0, err) && mbar_wait(&k_full[0], 0, err)) {
-        tc_fence_after();
-        issue_s(0);
-        for (int j = 0; j < n_kv; ++j) {
-          if (j + 1 < n_kv) {
-            if (!mbar_wait(&k_full[(j + 1) % KSLOT], ((j + 1) / KSLOT) & 1, err)) { failed = true; break; }
-            tc_fence_after();
-            issue_s(j + 1);
-          }
-          if (!mbar_wait(p_full, j & 1, err)) { failed = true; break; }
-          if (!mbar_wait(&v_full[j & 1], (j >> 1) & 1, err)) { failed = true; break; }
+      } else {
+        const uint32_t idesc = idesc_keys(idesc_s, last_nch);
+#pragma unroll 1
+        for (int kk = 0; kk < 8; ++kk) {
+          const uint32_t off = ((kk >> 2) * SUB + (kk & 3) * 32) >> 4;
+          tc_mma_ss_lo(tmem + (j & 1) * TB, q_lo + off, ka + off, dhi, idesc, kk ? 1u : 0u);
+        }
+      }
+      tc_commit(&s_full[j & 1]);
+    };
+    if (mbar_wait_warp(q_full, 0, err) && mbar_wait_warp(&k_full[0], 0, err)) {
+      tc_fence_after();
+      if (elect_one()) issue_s(0);
+      for (int j = 0; j < n_kv; ++j) {
+        if (j + 1 < n_kv) {
+          if (!mbar_wait_warp(&k_full[(j + 1) % KSLOT], ((j + 1) / KSLOT) & 1, err)) { failed = true; break; }
           tc_fence_after();
-          const uint32_t va = v_lo + (j & 1) * (V_BYTES >> 4);
+          if (elect_one()) issue_s(j + 1);
+        }
+        if (!mbar_wait_warp(p_full, j & 1, err)) { failed = true; break; }
+        if (!mbar_wait_warp(&v_full[j & 1], (j >> 1) & 1, err)) { failed = true; break; }
+        tc_fence_after();
+        const uint32_t va = v_lo + (j & 1) * (V_BYTES >> 4);
+        if (elect_one()) {
           if (j + 1 < n_kv || last_nch == 4) {
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) {
@@ -299,9 +299,9 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
           tc_commit(o_done);
         }
-      } else {
-        failed = true;
       }
+    } else {
+      failed = true;
     }
   } else {
     // ---------------- softmax (warps 2..5), one query row per thread ----------------
@@ -408,12 +408,11 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   }
 
-  if (failed || *(volatile int*)err != 0) {
-    const uint64_t t0 = fb_globaltimer();  // let in-flight TMA loads land
+  tc_fence_before();
+  if (__syncthreads_or(failed)) {  // a role gave up: loads in flight land before the CTA exits
+    const uint64_t t0 = fb_globaltimer();
     while (fb_globaltimer() - t0 < 100000ull) __nanosleep(1000);
   }
-  tc_fence_before();
-  __syncthreads();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, TMEM_COLS);
@@ -857,94 +856,97 @@ __global__ void __launch_bounds__(THREADS2, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TB >> 3) << 17) |
-                               ((uint32_t)(TB >> 4) << 24);
-      const uint32_t idesc_pv = idesc_s | (1u << 16);
-      const int last_nch = (p.Lkv - (n_kv - 1) * TB + 31) >> 5;
-      // descriptor lower words of the Q buffers, K slot 0 and V slot 0 (the other slots lie
-      // K_BYTES / V_BYTES further on)
-      const uint32_t dhi = DESC_HI;
-      const uint32_t q_lo[2] = {desc_lo_k(smem_u32(Qs)), desc_lo_k(smem_u32(Qs + Q_BYTES))};
-      const uint32_t k_lo = desc_lo_k(smem_u32(Ks)), v_lo = desc_lo_mn(smem_u32(Vs), SUB);
-      uint32_t kb = 0, vb = 0, pc[2] = {0u, 0u};  // K, V tiles and P tiles (per group) consumed
-      bool ok = true;
-      int it = 0;
-      // S_g of key tile j (K ring slot of tile kb + j); the last group's S of a tile frees
-      // its K slot, and of the last tile also the Q buffer
-      auto issue_s = [&](int g, int j, int ng) {
-        const uint32_t kt = kb + j;
-        const uint32_t ka = k_lo + (kt % KS) * (K_BYTES >> 4);
-        const uint32_t qg = q_lo[g];
-        if (j + 1 < n_kv || last_nch == 4) {
+    const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TB >> 3) << 17) |
+                             ((uint32_t)(TB >> 4) << 24);
+    const uint32_t idesc_pv = idesc_s | (1u << 16);
+    const int last_nch = (p.Lkv - (n_kv - 1) * TB + 31) >> 5;
+    // descriptor lower words of the Q buffers, K slot 0 and V slot 0 (the other slots lie
+    // K_BYTES / V_BYTES further on)
+    const uint32_t dhi = DESC_HI;
+    const uint32_t q_lo[2] = {desc_lo_k(smem_u32(Qs)), desc_lo_k(smem_u32(Qs + Q_BYTES))};
+    const uint32_t k_lo = desc_lo_k(smem_u32(Ks)), v_lo = desc_lo_mn(smem_u32(Vs), SUB);
+    uint32_t kb = 0, vb = 0, pc[2] = {0u, 0u};  // K, V tiles and P tiles (per group) consumed
+    bool ok = true;
+    int it = 0;
+    // S_g of key tile j (K ring slot of tile kb + j); the last group's S of a tile frees
+    // its K slot, and of the last tile also the Q buffer
+    auto issue_s = [&](int g, int j) {
+      const uint32_t kt = kb + j;
+      const uint32_t ka = k_lo + (kt % KS) * (K_BYTES >> 4);
+      const uint32_t qg = q_lo[g];
+      if (j + 1 < n_kv || last_nch == 4) {
 #pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint32_t off = ((kk >> 2) * SUB + (kk & 3) * 32) >> 4;
-            tc_mma_ss_lo(tmem + g * TB, qg + off, ka + off, dhi, idesc_s, kk ? 1u : 0u);
-          }
-        } else {
-          const uint32_t idesc = idesc_keys(idesc_s, last_nch);
+        for (int kk = 0; kk < 8; ++kk) {
+          const uint32_t off = ((kk >> 2) * SUB + (kk & 3) * 32) >> 4;
+          tc_mma_ss_lo(tmem + g * TB, qg + off, ka + off, dhi, idesc_s, kk ? 1u : 0u);
+        }
+      } else {
+        const uint32_t idesc = idesc_keys(idesc_s, last_nch);
 #pragma unroll 1
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint32_t off = ((kk >> 2) * SUB + (kk & 3) * 32) >> 4;
-            tc_mma_ss_lo(tmem + g * TB, qg + off, ka + off, dhi, idesc, kk ? 1u : 0u);
-          }
+        for (int kk = 0; kk < 8; ++kk) {
+          const uint32_t off = ((kk >> 2) * SUB + (kk & 3) * 32) >> 4;
+          tc_mma_ss_lo(tmem + g * TB, qg + off, ka + off, dhi, idesc, kk ? 1u : 0u);
         }
-        tc_commit(&s_full[g]);
-      };
-      auto issue_pv = [&](int g, int j) {
-        const uint32_t va = v_lo + ((vb + j) & 1) * (V_BYTES >> 4);
-        if (j + 1 < n_kv || last_nch == 4) {
-#pragma unroll
-          for (int kk = 0; kk < 8; ++kk)
-            tc_mma_ts_lo(tmem + O_COL + g * TB, tmem + g * TB + kk * 8, va + kk * (2048 >> 4),
-                         dhi, idesc_pv, (j | kk) ? 1u : 0u);
-        } else {
-#pragma unroll 1
-          for (int kk = 0; kk < 2 * last_nch; ++kk)
-            tc_mma_ts_lo(tmem + O_COL + g * TB, tmem + g * TB + kk * 8, va + kk * (2048 >> 4),
-                         dhi, idesc_pv, (j | kk) ? 1u : 0u);
-        }
-      };
-      for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++it) {
-        const int qb = item % nqb;
-        const int ng = qb * 2 * TB + TB < p.Lq ? 2 : 1;
-        if (!(ok = mbar_wait(q_full, it & 1, err))) break;
-        if (!(ok = mbar_wait(&k_full[kb % KS], (kb / KS) & 1, err))) break;
-        tc_fence_after();
-        for (int g = 0; g < ng; ++g) issue_s(g, 0, ng);
-        for (int j = 0; j < n_kv && ok; ++j) {
-          const bool more = j + 1 < n_kv;
-          const uint32_t vt = vb + j;
-          // this step's V and next step's K tiles first: they are normally there already,
-          // and these waits then overlap the tensor pipe's last instructions of the
-          // previous batch instead of following the softmax's hand-off (the pipe holds
-          // about one instruction, so every wait between batches is idle pipe time)
-          if (!(ok = mbar_wait(&v_full[vt & 1], (vt >> 1) & 1, err))) break;
-          if (more) {
-            const uint32_t kt = kb + j + 1;
-            if (!(ok = mbar_wait(&k_full[kt % KS], (kt / KS) & 1, err))) break;
-          }
-          if (!(ok = mbar_wait(&p_full[0], pc[0]++ & 1, err))) break;
-          tc_fence_after();
-          issue_pv(0, j);
-          // a group's O rows are complete with its last PV: its epilogue may start while
-          // the other group's last PV runs
-          if (!more) tc_commit(&o_done[0]);
-          if (more) issue_s(0, j + 1, ng);
-          if (ng == 1) continue;
-          if (!(ok = mbar_wait(&p_full[1], pc[1]++ & 1, err))) break;
-          tc_fence_after();
-          issue_pv(1, j);
-          if (!more) tc_commit(&o_done[1]);
-          if (more) issue_s(1, j + 1, ng);
-        }
-        if (!ok) break;
-        kb += n_kv;
-        vb += n_kv;
       }
-      failed = !ok;
+      tc_commit(&s_full[g]);
+    };
+    auto issue_pv = [&](int g, int j) {
+      const uint32_t va = v_lo + ((vb + j) & 1) * (V_BYTES >> 4);
+      if (j + 1 < n_kv || last_nch == 4) {
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk)
+          tc_mma_ts_lo(tmem + O_COL + g * TB, tmem + g * TB + kk * 8, va + kk * (2048 >> 4),
+                       dhi, idesc_pv, (j | kk) ? 1u : 0u);
+      } else {
+#pragma unroll 1
+        for (int kk = 0; kk < 2 * last_nch; ++kk)
+          tc_mma_ts_lo(tmem + O_COL + g * TB, tmem + g * TB + kk * 8, va + kk * (2048 >> 4),
+                       dhi, idesc_pv, (j | kk) ? 1u : 0u);
+      }
+    };
+    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++it) {
+      const int qb = item % nqb;
+      const int ng = qb * 2 * TB + TB < p.Lq ? 2 : 1;
+      if (!(ok = mbar_wait_warp(q_full, it & 1, err))) break;
+      if (!(ok = mbar_wait_warp(&k_full[kb % KS], (kb / KS) & 1, err))) break;
+      tc_fence_after();
+      if (elect_one())
+        for (int g = 0; g < ng; ++g) issue_s(g, 0);
+      for (int j = 0; j < n_kv && ok; ++j) {
+        const bool more = j + 1 < n_kv;
+        const uint32_t vt = vb + j;
+        // this step's V and next step's K tiles first: they are normally there already,
+        // and these waits then overlap the tensor pipe's last instructions of the
+        // previous batch instead of following the softmax's hand-off (the pipe holds
+        // about one instruction, so every wait between batches is idle pipe time)
+        if (!(ok = mbar_wait_warp(&v_full[vt & 1], (vt >> 1) & 1, err))) break;
+        if (more) {
+          const uint32_t kt = kb + j + 1;
+          if (!(ok = mbar_wait_warp(&k_full[kt % KS], (kt / KS) & 1, err))) break;
+        }
+        if (!(ok = mbar_wait_warp(&p_full[0], pc[0]++ & 1, err))) break;
+        tc_fence_after();
+        // a group's O rows are complete with its last PV: its epilogue may start while
+        // the other group's last PV runs
+        if (elect_one()) {
+          issue_pv(0, j);
+          if (more) issue_s(0, j + 1);
+          else tc_commit(&o_done[0]);
+        }
+        if (ng == 1) continue;
+        if (!(ok = mbar_wait_warp(&p_full[1], pc[1]++ & 1, err))) break;
+        tc_fence_after();
+        if (elect_one()) {
+          issue_pv(1, j);
+          if (more) issue_s(1, j + 1);
+          else tc_commit(&o_done[1]);
+        }
+      }
+      if (!ok) break;
+      kb += n_kv;
+      vb += n_kv;
     }
+    failed = !ok;
   } else {
     // ---------------- softmax groups: warps 2-5 -> tile A, warps 6-9 -> tile B ----------
     const int g = (warp - 2) >> 2;
@@ -1101,12 +1103,11 @@ __global__ void __launch_bounds__(THREADS2, 1)
     }
   }
 
-  if (failed || *(volatile int*)err != 0) {
+  tc_fence_before();
+  if (__syncthreads_or(failed)) {  // a role gave up: loads in flight land before the CTA exits
     const uint64_t t0 = fb_globaltimer();
     while (fb_globaltimer() - t0 < 100000ull) __nanosleep(1000);
   }
-  tc_fence_before();
-  __syncthreads();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, TMEM_COLS);
