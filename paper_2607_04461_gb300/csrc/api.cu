@@ -200,6 +200,10 @@ struct fb_model {
   float* sk_ws = nullptr;
   int* sk_ctr = nullptr;
   int sk_clusters = 0;
+  // workspace of the attention's key split: partials and flags per CTA (zero between
+  // launches; reset after a device error)
+  float* attn_ws = nullptr;
+  int* attn_flags = nullptr;
   // statistics
   unsigned timing_mask = 0;
   int op_repeat = 1;
@@ -302,10 +306,12 @@ fb_status end_call(fb_model* m) {
   CK(cudaMemcpyAsync(m->herr, m->derr, sizeof(int), cudaMemcpyDeviceToHost, m->st));
   CK(cudaStreamSynchronize(m->st));
   collect_timings(m);
-  if (*m->herr != 0 && m->sk_ctr) {
-    // a kernel that gave up may have left stream-K counters counted in
+  if (*m->herr != 0 && m->sk_ctr && m->attn_flags) {
+    // a kernel that gave up may have left stream-K counters counted in or flags raised
     fb_stream_op_not_kernel();
     CK(cudaMemsetAsync(m->sk_ctr, 0, (size_t)m->sk_clusters * SK_CTR_PER_CLUSTER * sizeof(int),
+                       m->st));
+    CK(cudaMemsetAsync(m->attn_flags, 0, (size_t)m->dev_sms * ATTN_FLAGS_PER_CTA * sizeof(int),
                        m->st));
     CK(cudaStreamSynchronize(m->st));
   }
@@ -358,6 +364,9 @@ fb_status run_attn(fb_model* m, const AttnArgs& a0, int kind, int impl = 0) {
   AttnArgs a = a0;
   a.tc_variant = impl >= 2 ? impl - 1 : 0;
   a.sms = m->num_sms;
+  a.ws = m->attn_ws;
+  a.flags = m->attn_flags;
+  a.ws_ctas = m->dev_sms;
   const double flops = 4.0 * a.batch * a.heads * (double)a.Lq * a.Lkv * a.head_dim;
   const double kvb = (a.kv_batch_rows ? a.batch : 1) * 2.0 * a.Lkv * a.heads * a.head_dim * 2;
   const double bytes = 2.0 * a.batch * a.Lq * (double)a.heads * a.head_dim * 2 + kvb;
@@ -1038,10 +1047,14 @@ fb_status fb_init_model(const fb_cfg* cfg, const float* weights_host, fb_model**
   m->dev_sms = m->num_sms;
   m->sk_clusters = m->num_sms / 2;
   if ((s = dalloc_t(m, &m->sk_ws, (size_t)m->sk_clusters * SK_WS_FLOATS_PER_CLUSTER)) ||
-      (s = dalloc_t(m, &m->sk_ctr, (size_t)m->sk_clusters * SK_CTR_PER_CLUSTER)))
+      (s = dalloc_t(m, &m->sk_ctr, (size_t)m->sk_clusters * SK_CTR_PER_CLUSTER)) ||
+      (s = dalloc_t(m, &m->attn_ws, (size_t)m->dev_sms * ATTN_WS_FLOATS_PER_CTA)) ||
+      (s = dalloc_t(m, &m->attn_flags, (size_t)m->dev_sms * ATTN_FLAGS_PER_CTA)))
     return bail(s);
   if (cudaMemset(m->sk_ctr, 0, (size_t)m->sk_clusters * SK_CTR_PER_CLUSTER * sizeof(int)) !=
-      cudaSuccess)
+          cudaSuccess ||
+      cudaMemset(m->attn_flags, 0, (size_t)m->dev_sms * ATTN_FLAGS_PER_CTA * sizeof(int)) !=
+          cudaSuccess)
     return bail(fail(FB_ECUDA, "cudaMemset failed"));
   if (m->PD % 64 == 0 && D % 128 == 0) {
     const size_t PDs = m->PD;

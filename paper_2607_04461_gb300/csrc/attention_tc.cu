@@ -23,6 +23,8 @@
 // All waits are bounded; on a timeout the kernel records the error and drains.
 #include <cudaTypedefs.h>
 
+#include <cmath>
+
 #include "kernels.h"
 
 namespace {
@@ -45,7 +47,15 @@ struct Params {
   int ldo;
   float scale_log2;
   int* err;
-  int batch, heads;  // the persistent kernel's item count
+  int batch, heads;
+  // the persistent kernel's work split (see SplitPlan)
+  int n_full_qb;     // 256-query items per head with both query tiles in range
+  int n_full, n_items;         // such items in all, items in all
+  unsigned div_qb, div_heads;  // ceil(2^32 / n_full_qb), ceil(2^32 / heads): see div_by
+  int split;         // != 0: the items from `rounds` full rounds on are cut into equal shares
+  int rounds;
+  float* ws;         // per CTA: 8 warps x ATTN_WS_WARP floats (a cut item's partial)
+  int* flags;        // per CTA and warp: 1 = its partial is in ws (0 between launches)
 };
 
 // Operand layouts (descriptors from desc_lo_k / desc_lo_mn): Q, K and P are K-major with
@@ -736,23 +746,265 @@ __global__ void __launch_bounds__(THREADS2, 1)
 }
 
 // ---- persistent 256-query kernel ----------------------------------------------------
-// attn_tc2_kernel's computation with at most one CTA per SM, each looping over items
-// (batch b, head h, query-tile pair qb), qb fastest so that the CTAs running at the same
-// time share their K/V tiles in L2. Per CTA the work of consecutive items overlaps:
-//  * the producer loads the next item's Q as soon as the current item's last S MMAs are
+// attn_tc2_kernel's computation with at most one CTA per SM, each working through segments:
+// whole items (batch b, head h, query-tile pair qb) and, where whole items would leave SMs
+// idle in the last round, parts of the key range of one item. Items are numbered with the
+// pairs of two query tiles first (qb fastest, so that the CTAs running at the same time
+// share their K/V tiles in L2), then the items of a last single tile. Per CTA the work of
+// consecutive segments overlaps:
+//  * the producer loads the next segment's Q as soon as the current one's last S MMAs are
 //    done (q_empty) and carries on through the K/V rings, whose slots and phases count
-//    across items; the slots are released by a softmax thread that has seen a tile's last
+//    across segments; the slots are released by a softmax thread that has seen a tile's last
 //    S MMAs done, so the MMA issuer commits only what the softmax groups wait for (each
 //    tcgen05.commit holds up the issuing thread while softmax warps share its SM
 //    sub-partition);
-//  * the MMA issuer starts the next item's S MMAs right after the current item's last PV
+//  * the MMA issuer starts the next segment's S MMAs right after the current one's last PV
 //    (the tensor pipe runs in order, so S_g overwrites P_g only after PV_g has read it);
-//  * each softmax group stores its O rows (o_done, one phase per item of the group) while
+//  * each softmax group stores its O rows (o_done, one phase per segment of the group) while
 //    those S MMAs run, each thread its row in 32-byte stores (whole sectors); its first P
-//    of the next item is announced only after those TMEM reads, so the first PV of the
-//    next item (accumulate = 0) cannot overwrite O early.
+//    of the next segment is announced only after those TMEM reads, so the first PV of the
+//    next segment (accumulate = 0) cannot overwrite O early.
 // Group B has no work in items whose second query tile lies past Lq; the issuer and the
 // group count the phases of their own barriers.
+//
+// Work split. G CTAs; `rounds` full rounds of items (CTA c: items c, c + G, ...), then, with
+// p.split, the rest as G contiguous ranges of equal cost over the (item, 128-key step) units:
+// 4 per step of an item with two query tiles, 3 with one (measured about 0.75). An item cut
+// between CTAs c_lo .. c_hi is finished by c_hi, the others leave the group's unnormalised O
+// rows, row maxima and sums (fp32) in the workspace; c_hi adds them in CTA order, so the
+// result does not depend on timing. A CTA works on the part that it contributes first and
+// finishes another's item last, so the finisher's wait is normally over before it begins;
+// and it waits only for CTAs of lower index, which started before it.
+constexpr int ATTN_WS_WARP = 32 * 128 + 64;  // O rows [chunk 4][4-column group 8][lane][4], (m, l)
+static_assert(8 * ATTN_WS_WARP == ATTN_WS_FLOATS_PER_CTA && 8 == ATTN_FLAGS_PER_CTA, "attention workspace");
+
+enum { SEG_WHOLE = 0, SEG_PART = 1, SEG_FINISH = 2 };
+struct Seg {
+  int item, j0, j1, kind;  // key tiles j0 .. j1 - 1 of the item
+};
+// One CTA's segments in order: a contributed part, whole items of the full rounds, whole
+// items of its range, the tail of an item that it finishes.
+struct SplitPlan {
+  int part_item, part_j0, part_j1;  // part_j1 == 0: none
+  int whole_first, n_whole;
+  int tail_item, tail_j0;           // tail_item < 0: none
+  int c_lo;                         // first contributor of tail_item
+};
+// The split region's unit arithmetic.
+struct SplitUnits {
+  int n_kv, n_full, n_items, r0;    // r0: first item of the region
+  unsigned full_units, units;       // (units x G fits 32 bits: plan_split)
+  __device__ SplitUnits(const Params& p, int n_kv_, int G) : n_kv(n_kv_) {
+    n_full = p.n_full;
+    n_items = p.n_items;
+    r0 = p.rounds * G;              // <= n_full
+    full_units = (unsigned)(n_full - r0) * 4 * n_kv;
+    units = full_units + (unsigned)(n_items - n_full) * 3 * n_kv;
+  }
+  // where CTA c's range begins
+  __device__ void at(unsigned c, unsigned G, int& item, int& j) const {
+    const unsigned u = c * units / G;
+    if (u >= units) {
+      item = n_items;
+      j = 0;
+    } else if (u < full_units) {
+      item = r0 + (int)(u / (4u * n_kv));
+      j = (int)(u % (4u * n_kv)) / 4;
+    } else {
+      item = n_full + (int)((u - full_units) / (3u * n_kv));
+      j = (int)((u - full_units) % (3u * n_kv)) / 3;
+    }
+  }
+};
+__device__ void make_split_plan(const Params& p, int n_kv, int G, int c, SplitPlan* pl) {
+  const SplitUnits su(p, n_kv, G);
+  pl->part_j1 = 0;
+  pl->n_whole = 0;
+  pl->tail_item = -1;
+  int i0, j0, i1, j1;
+  su.at(c, G, i0, j0);
+  su.at(c + 1, G, i1, j1);
+  if (i0 == i1) {                   // inside one item, which another CTA finishes
+    pl->part_item = i0;
+    pl->part_j0 = j0;
+    pl->part_j1 = j1 > j0 ? j1 : 0;
+    return;
+  }
+  if (j0 > 0) {
+    pl->tail_item = i0;
+    pl->tail_j0 = j0;
+    // the contributors are the CTAs before this one down to the first whose range reaches
+    // the item's first key tile (a share is more than a step, so each holds some of it,
+    // except one whose range ends within the item's first step)
+    int lo = c, ilo = i0, jlo = j0;
+    while (ilo == i0 && jlo > 0) {
+      --lo;
+      su.at(lo, G, ilo, jlo);
+    }
+    pl->c_lo = lo;
+  }
+  pl->whole_first = j0 > 0 ? i0 + 1 : i0;
+  pl->n_whole = i1 - pl->whole_first;
+  pl->part_item = i1;
+  pl->part_j0 = 0;
+  pl->part_j1 = j1;
+}
+// Segment s of the CTA; false past the last.
+template <bool SPLIT>
+__device__ __forceinline__ bool get_seg(const Params& p, const SplitPlan& pl, int s, int n_kv,
+                                        Seg& g) {
+  g.j0 = 0;
+  g.j1 = n_kv;
+  g.kind = SEG_WHOLE;
+  if (!SPLIT) {
+    g.item = (int)blockIdx.x + s * (int)gridDim.x;
+    return g.item < p.n_items;
+  }
+  if (pl.part_j1) {
+    if (s == 0) {
+      g = Seg{pl.part_item, pl.part_j0, pl.part_j1, SEG_PART};
+      return true;
+    }
+    --s;
+  }
+  if (s < p.rounds) {
+    g.item = (int)blockIdx.x + s * (int)gridDim.x;
+    return true;
+  }
+  s -= p.rounds;
+  if (s < pl.n_whole) {
+    g.item = pl.whole_first + s;
+    return true;
+  }
+  if (s > pl.n_whole || pl.tail_item < 0) return false;
+  g = Seg{pl.tail_item, pl.tail_j0, n_kv, SEG_FINISH};
+  return true;
+}
+// Waits (bounded, as mbar_wait) until another CTA has raised its flag.
+__device__ __forceinline__ bool wait_flag(int* flag, int* err) {
+  const uint64_t t0 = fb_globaltimer();
+  while (*(volatile int*)flag == 0) {
+    if (*(volatile int*)err != 0) return false;
+    if (fb_globaltimer() - t0 > fb_wait_limit()) {
+      atomicExch(err, FB_DEVERR_WAIT_TIMEOUT);
+      return false;
+    }
+    __nanosleep(64);
+  }
+  return true;
+}
+// Whole warp: makes its earlier stores visible and sets the flag.
+__device__ __forceinline__ void raise_flag(int* flag, int lane) {
+  __threadfence();
+  __syncwarp();
+  if (lane == 0) atomicExch(flag, 1);
+}
+// The finisher of a cut item waits for the parts of CTAs c_lo .. blockIdx.x - 1 (this warp's
+// rows: flags by lane), updates the row's maximum m and sum l with theirs, in CTA order, and
+// returns in a_own the factor of the rows that it has in TMEM itself. False if a wait gave up.
+__device__ __forceinline__ bool join_parts(const Params& p, int c_lo, int ww, int lane, float& m,
+                                           float& l, float& a_own, int* err) {
+  const int n = (int)blockIdx.x - c_lo;
+  int* flags = p.flags + (size_t)c_lo * 8 + ww;
+  bool ok = true;
+  for (int i = lane; i < n && ok; i += 32) ok = wait_flag(flags + i * 8, err);
+  if (!__all_sync(0xffffffffu, ok)) return false;
+  __threadfence();
+  for (int i = lane; i < n; i += 32) flags[i * 8] = 0;  // free for the next launch
+  const float* part = p.ws + ((size_t)c_lo * 8 + ww) * ATTN_WS_WARP;
+  float m_all = m;
+#pragma unroll 4
+  for (int i = 0; i < n; ++i)
+    m_all = fmaxf(m_all, __ldcg(part + (size_t)i * 8 * ATTN_WS_WARP + 4096 + 2 * lane));
+  a_own = ex2(m - m_all);
+  l *= a_own;
+  m = m_all;
+#pragma unroll 4
+  for (int i = 0; i < n; ++i) {
+    const float2 ml = __ldcg(
+        reinterpret_cast<const float2*>(part + (size_t)i * 8 * ATTN_WS_WARP + 4096) + lane);
+    l += ml.y * ex2(ml.x - m_all);
+  }
+  return true;
+}
+// Adds 64 columns (half 0 or 1) of the parts' rows, scaled to the maximum m, to f in CTA order.
+// A part's 16 loads are in flight together.
+__device__ __forceinline__ void add_parts(const Params& p, int c_lo, int ww, int lane, float m,
+                                          int half, float4* f) {
+  const float* part = p.ws + ((size_t)c_lo * 8 + ww) * ATTN_WS_WARP;
+#pragma unroll 1
+  for (int c = c_lo; c < (int)blockIdx.x; ++c, part += 8 * ATTN_WS_WARP) {
+    const float a = ex2(__ldcg(part + 4096 + 2 * lane) - m);
+    float4 v[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+      v[q] = __ldcg(reinterpret_cast<const float4*>(part) + (half * 16 + q) * 32 + lane);
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      f[q].x += a * v[q].x;
+      f[q].y += a * v[q].y;
+      f[q].z += a * v[q].z;
+      f[q].w += a * v[q].w;
+    }
+  }
+}
+// x / d by the rounded-up reciprocal ceil(2^32 / d): exact while x d < 2^32 (plan_split
+// checks the largest item number); d = 1 has no 32-bit reciprocal and is passed as 0
+__device__ __forceinline__ int div_by(int x, unsigned recip) {
+  return recip ? (int)__umulhi((unsigned)x, recip) : x;
+}
+// item -> query-tile pair qb, head h, batch b, groups with work
+__device__ __forceinline__ int decode_item(const Params& p, int item, int& qb, int& h, int& b) {
+  const bool full = item < p.n_full;
+  int bh = item - p.n_full;
+  qb = p.n_full_qb;
+  if (full) {
+    bh = div_by(item, p.div_qb);
+    qb = item - bh * p.n_full_qb;
+  }
+  b = div_by(bh, p.div_heads);
+  h = bh - b * p.heads;
+  return full ? 2 : 1;
+}
+
+// One O row: 32 columns at a time, scaled by inv and rounded to bf16, in 32-byte stores (whole
+// sectors) where the rows are 32-byte aligned.
+struct ORow {
+  bf16* row;
+  bool in, st32;
+  __device__ __forceinline__ ORow(const Params& p, int item, int q) {
+    int qb, h, b;
+    decode_item(p, item, qb, h, b);
+    const int qrow = qb * 2 * TB + q;
+    in = qrow < p.Lq;
+    row = p.O + (size_t)(b * p.Lq + qrow) * p.ldo + h * 128;
+    st32 = ((reinterpret_cast<uintptr_t>(p.O) & 31) | (p.ldo & 15)) == 0;
+  }
+  __device__ __forceinline__ void store32(int c, const uint32_t* u, float inv) const {
+    if (!in) return;
+    if (st32) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        uint32_t w[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          w[i] = pack_bf16x2(__uint_as_float(u[q * 16 + 2 * i]) * inv,
+                             __uint_as_float(u[q * 16 + 2 * i + 1]) * inv);
+        store_b32x8(row + c * 32 + q * 16, w);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(u[q * 8 + i]) * inv;
+        store_bf16x8(row + c * 32 + q * 8, v);
+      }
+    }
+  }
+};
+
+template <bool SPLIT>
 __global__ void __launch_bounds__(THREADS2, 1)
     attn_tc2p_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                      const __grid_constant__ CUtensorMap tmV, Params p) {
@@ -777,11 +1029,11 @@ __global__ void __launch_bounds__(THREADS2, 1)
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int n_kv = (p.Lkv + TB - 1) / TB;
-  const int nqb = (p.Lq + 2 * TB - 1) / (2 * TB);
-  const int n_items = nqb * p.heads * p.batch;
+  __shared__ SplitPlan plan;
   int* err = p.err;
   bool failed = false;
 
+  if (SPLIT && threadIdx.x == 64) make_split_plan(p, n_kv, gridDim.x, blockIdx.x, &plan);
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
     mbar_init(q_empty, 1);
@@ -812,18 +1064,18 @@ __global__ void __launch_bounds__(THREADS2, 1)
     // ---------------- TMA producers: lane 0 Q and K, lane 1 V ----------------
     if (lane == 0) {
       uint32_t kt = 0;  // K tiles loaded by this CTA
-      int it = 0;
-      for (int item = blockIdx.x; item < n_items && !failed; item += gridDim.x, ++it) {
-        const int qb = item % nqb, bh = item / nqb, h = bh % p.heads, b = bh / p.heads;
+      Seg sg;
+      for (int it = 0; !failed && get_seg<SPLIT>(p, plan, it, n_kv, sg); ++it) {
+        int qb, h, b;
+        const int ng = decode_item(p, sg.item, qb, h, b);
         const int xq = h * 128, q_row0 = b * p.Lq + qb * 2 * TB, kv_row0 = b * p.kv_batch_rows;
-        const int ng = qb * 2 * TB + TB < p.Lq ? 2 : 1;
         if (!mbar_wait(q_empty, (it & 1) ^ 1u, err)) { failed = true; break; }
         mbar_expect_tx(q_full, ng * Q_BYTES);
         for (int g = 0; g < ng; ++g) {
           tma_load_2d(Qs + g * Q_BYTES, &tmQ, q_full, xq, q_row0 + g * TB);
           tma_load_2d(Qs + g * Q_BYTES + SUB, &tmQ, q_full, xq + 64, q_row0 + g * TB);
         }
-        for (int j = 0; j < n_kv; ++j, ++kt) {
+        for (int j = sg.j0; j < sg.j1; ++j, ++kt) {
           const int s = kt % KS;
           if (!mbar_wait(&k_empty[s], ((kt / KS) & 1) ^ 1u, err)) { failed = true; break; }
           uint8_t* st = Ks + s * K_BYTES;
@@ -835,10 +1087,12 @@ __global__ void __launch_bounds__(THREADS2, 1)
       }
     } else if (lane == 1) {
       uint32_t vt = 0;  // V tiles loaded by this CTA
-      for (int item = blockIdx.x; item < n_items && !failed; item += gridDim.x) {
-        const int bh = item / nqb, h = bh % p.heads, b = bh / p.heads;
+      Seg sg;
+      for (int it = 0; !failed && get_seg<SPLIT>(p, plan, it, n_kv, sg); ++it) {
+        int qb, h, b;
+        decode_item(p, sg.item, qb, h, b);
         const int xq = h * 128, kv_row0 = b * p.kv_batch_rows;
-        for (int j = 0; j < n_kv; ++j, ++vt) {
+        for (int j = sg.j0; j < sg.j1; ++j, ++vt) {
           const int s = vt & 1;
           // slot s last held tile vt - 2; its PV MMAs are done once the S MMAs of tile
           // vt - 1 are (the issuer issues those after them): the K slot release of tile
@@ -865,16 +1119,17 @@ __global__ void __launch_bounds__(THREADS2, 1)
     const uint32_t dhi = DESC_HI;
     const uint32_t q_lo[2] = {desc_lo_k(smem_u32(Qs)), desc_lo_k(smem_u32(Qs + Q_BYTES))};
     const uint32_t k_lo = desc_lo_k(smem_u32(Ks)), v_lo = desc_lo_mn(smem_u32(Vs), SUB);
-    uint32_t kb = 0, vb = 0, pc[2] = {0u, 0u};  // K, V tiles and P tiles (per group) consumed
+    // Everything the MMAs' operands depend on is counted under warp-uniform control flow (the
+    // segment's bounds, read from shared memory, only enter votes).
+    uint32_t ks = 0, kph = 0;           // K ring slot and phase of the current key tile
+    uint32_t vt = 0;                    // V tiles consumed (slot vt & 1)
+    uint32_t pph[2] = {0u, 0u};         // P phases per group
     bool ok = true;
-    int it = 0;
-    // S_g of key tile j (K ring slot of tile kb + j); the last group's S of a tile frees
-    // its K slot, and of the last tile also the Q buffer
-    auto issue_s = [&](int g, int j) {
-      const uint32_t kt = kb + j;
-      const uint32_t ka = k_lo + (kt % KS) * (K_BYTES >> 4);
+    // S_g of the key tile in K slot `slot`; `last`: the last key tile (its real keys only)
+    auto issue_s = [&](int g, uint32_t slot, bool last) {
+      const uint32_t ka = k_lo + slot * (K_BYTES >> 4);
       const uint32_t qg = q_lo[g];
-      if (j + 1 < n_kv || last_nch == 4) {
+      if (!last || last_nch == 4) {
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk) {
           const uint32_t off = ((kk >> 2) * SUB + (kk & 3) * 32) >> 4;
@@ -890,61 +1145,70 @@ __global__ void __launch_bounds__(THREADS2, 1)
       }
       tc_commit(&s_full[g]);
     };
-    auto issue_pv = [&](int g, int j) {
-      const uint32_t va = v_lo + ((vb + j) & 1) * (V_BYTES >> 4);
-      if (j + 1 < n_kv || last_nch == 4) {
+    auto issue_pv = [&](int g, uint32_t acc, bool last) {
+      const uint32_t va = v_lo + (vt & 1) * (V_BYTES >> 4);
+      if (!last || last_nch == 4) {
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)
           tc_mma_ts_lo(tmem + O_COL + g * TB, tmem + g * TB + kk * 8, va + kk * (2048 >> 4),
-                       dhi, idesc_pv, (j | kk) ? 1u : 0u);
+                       dhi, idesc_pv, kk ? 1u : acc);
       } else {
 #pragma unroll 1
         for (int kk = 0; kk < 2 * last_nch; ++kk)
           tc_mma_ts_lo(tmem + O_COL + g * TB, tmem + g * TB + kk * 8, va + kk * (2048 >> 4),
-                       dhi, idesc_pv, (j | kk) ? 1u : 0u);
+                       dhi, idesc_pv, kk ? 1u : acc);
       }
     };
-    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++it) {
-      const int qb = item % nqb;
-      const int ng = qb * 2 * TB + TB < p.Lq ? 2 : 1;
+    for (int it = 0; ok; ++it) {
+      Seg sg;
+      if (!__all_sync(0xffffffffu, get_seg<SPLIT>(p, plan, it, n_kv, sg))) break;
+      const bool two = __all_sync(0xffffffffu, sg.item < p.n_full);  // both query tiles
+      int j = sg.j0;
+      bool last = __all_sync(0xffffffffu, j + 1 == n_kv);
       if (!(ok = mbar_wait_warp(q_full, it & 1, err))) break;
-      if (!(ok = mbar_wait_warp(&k_full[kb % KS], (kb / KS) & 1, err))) break;
+      if (!(ok = mbar_wait_warp(&k_full[ks], kph, err))) break;
       tc_fence_after();
-      if (elect_one())
-        for (int g = 0; g < ng; ++g) issue_s(g, 0);
-      for (int j = 0; j < n_kv && ok; ++j) {
-        const bool more = j + 1 < n_kv;
-        const uint32_t vt = vb + j;
+      if (elect_one()) {
+        issue_s(0, ks, last);
+        if (two) issue_s(1, ks, last);
+      }
+      uint32_t acc = 0;
+      for (bool more = true; more; acc = 1) {
+        ++j;
+        more = __all_sync(0xffffffffu, j < sg.j1);
+        const bool next_last = __all_sync(0xffffffffu, j + 1 == n_kv);
+        const uint32_t ks1 = ks + 1 == KS ? 0 : ks + 1, kph1 = ks + 1 == KS ? kph ^ 1u : kph;
         // this step's V and next step's K tiles first: they are normally there already,
         // and these waits then overlap the tensor pipe's last instructions of the
         // previous batch instead of following the softmax's hand-off (the pipe holds
         // about one instruction, so every wait between batches is idle pipe time)
         if (!(ok = mbar_wait_warp(&v_full[vt & 1], (vt >> 1) & 1, err))) break;
-        if (more) {
-          const uint32_t kt = kb + j + 1;
-          if (!(ok = mbar_wait_warp(&k_full[kt % KS], (kt / KS) & 1, err))) break;
-        }
-        if (!(ok = mbar_wait_warp(&p_full[0], pc[0]++ & 1, err))) break;
+        if (more && !(ok = mbar_wait_warp(&k_full[ks1], kph1, err))) break;
+        if (!(ok = mbar_wait_warp(&p_full[0], pph[0], err))) break;
+        pph[0] ^= 1u;
         tc_fence_after();
         // a group's O rows are complete with its last PV: its epilogue may start while
         // the other group's last PV runs
         if (elect_one()) {
-          issue_pv(0, j);
-          if (more) issue_s(0, j + 1);
+          issue_pv(0, acc, last);
+          if (more) issue_s(0, ks1, next_last);
           else tc_commit(&o_done[0]);
         }
-        if (ng == 1) continue;
-        if (!(ok = mbar_wait_warp(&p_full[1], pc[1]++ & 1, err))) break;
-        tc_fence_after();
-        if (elect_one()) {
-          issue_pv(1, j);
-          if (more) issue_s(1, j + 1);
-          else tc_commit(&o_done[1]);
+        if (two) {
+          if (!(ok = mbar_wait_warp(&p_full[1], pph[1], err))) break;
+          pph[1] ^= 1u;
+          tc_fence_after();
+          if (elect_one()) {
+            issue_pv(1, acc, last);
+            if (more) issue_s(1, ks1, next_last);
+            else tc_commit(&o_done[1]);
+          }
         }
+        ks = ks1;
+        kph = kph1;
+        ++vt;
+        last = next_last;
       }
-      if (!ok) break;
-      kb += n_kv;
-      vb += n_kv;
     }
     failed = !ok;
   } else {
@@ -954,24 +1218,45 @@ __global__ void __launch_bounds__(THREADS2, 1)
     const int r = quarter * 32 + lane;
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
     const uint32_t s_col = g * TB, o_col = O_COL + g * TB;
-    uint32_t cnt = 0;   // items this group has worked on
-    uint32_t kbase = 0;  // K tiles of the CTA's earlier items (numbered as the producer does)
+    uint32_t cnt = 0;  // segments this group has worked on
+    uint32_t sc = 0;   // S tiles this group has seen
+    uint32_t kt = 0;   // K tiles of the CTA so far (numbered as the producer does)
     // the group whose S MMAs come last in a key tile (B, or A where B has no work) releases
-    // the tile's K slot, and at the item's last tile the Q buffer, once its S is done: the
+    // the tile's K slot, and at the segment's last tile the Q buffer, once its S is done: the
     // issuer's S MMAs of a tile follow its PV MMAs of the tile before, so this also frees
     // that tile's V slot
     const bool lead = (warp & 3) == 2 && lane == 0;  // one thread per group
-    for (int item = blockIdx.x; item < n_items && !failed; item += gridDim.x, kbase += n_kv) {
-      const int qb = item % nqb;
-      if (qb * 2 * TB + g * TB >= p.Lq) continue;  // this tile lies past Lq: no work
-      const bool last_group = g == 1 || qb * 2 * TB + TB >= p.Lq;
-      float m_used = -INFINITY, l = 0.f;
-      for (int j = 0; j < n_kv; ++j) {
-        const bool ok = mbar_wait(&s_full[g], (cnt * (uint32_t)n_kv + j) & 1, err);
+    bool flag_due = false;  // this group's part is stored, its flag not yet raised
+    auto raise_due = [&] {
+      if (flag_due) raise_flag(p.flags + blockIdx.x * 8 + warp - 2, lane);
+      flag_due = false;
+    };
+    float m_used = -INFINITY, l = 0.f;  // the row's maximum and sum in the current segment
+    bool finish = false;                // the last segment completes an item cut between CTAs
+    for (int it = 0;; ++it) {
+      int j, j_end;
+      bool last_group;
+      {
+        Seg sg;
+        if (!get_seg<SPLIT>(p, plan, it, n_kv, sg)) break;
+        const int ng = sg.item < p.n_full ? 2 : 1;
+        if (g >= ng) {  // this tile lies past Lq: no work
+          kt += sg.j1 - sg.j0;
+          if (SPLIT) raise_due();
+          continue;
+        }
+        j = sg.j0;
+        j_end = sg.j1;
+        last_group = g == ng - 1;
+      }
+      m_used = -INFINITY;
+      l = 0.f;
+      for (; j < j_end; ++j, ++sc, ++kt) {
+        const bool ok = mbar_wait(&s_full[g], sc & 1, err);
         if (!__all_sync(0xffffffffu, ok)) { failed = true; break; }
         if (lead && last_group) {
-          mbar_arrive(&k_empty[(kbase + j) % KS]);
-          if (j == n_kv - 1) mbar_arrive(q_empty);
+          mbar_arrive(&k_empty[kt % KS]);
+          if (j == j_end - 1) mbar_arrive(q_empty);
         }
         tc_fence_after();
         float s[128];
@@ -992,7 +1277,7 @@ __global__ void __launch_bounds__(THREADS2, 1)
             if (i >= valid) s[i] = -INFINITY;
         }
         const float mx = rowmax128(s) * p.scale_log2;
-        if (j == 0) {
+        if (m_used == -INFINITY) {  // the segment's first tile
           m_used = mx;
         } else if (__any_sync(0xffffffffu, mx > m_used + 8.f)) {
           const float m_new = fmaxf(m_used, mx);
@@ -1059,47 +1344,78 @@ __global__ void __launch_bounds__(THREADS2, 1)
         if (lane == 0) mbar_arrive(&p_full[g]);
       }
       if (failed) break;
-      // the item's O rows: PV_g of its last key tile done
+      Seg sg;
+      get_seg<SPLIT>(p, plan, it, n_kv, sg);
+      if (SPLIT) raise_due();
+      // the segment's O rows: PV_g of its last key tile done
       const bool ok = mbar_wait(&o_done[g], cnt & 1, err);
       if (!__all_sync(0xffffffffu, ok)) { failed = true; break; }
       tc_fence_after();
-      const int bh = item / nqb, h = bh % p.heads, b = bh / p.heads;
-      {
-        const float inv = 1.f / l;
-        const int qrow = qb * 2 * TB + g * TB + r;
-        bf16* orow = p.O + (size_t)(b * p.Lq + qrow) * p.ldo + h * 128;
-        // 32-byte stores (whole sectors) where the rows are 32-byte aligned
-        const bool st32 = ((reinterpret_cast<uintptr_t>(p.O) & 31) | (p.ldo & 15)) == 0;
+      if (SPLIT && sg.kind == SEG_PART) {
+        // publish the rows, maxima and sums; the flag goes up after the next segment's last
+        // key tile (its stores have then long been performed), or after the last segment
+        float* part = p.ws + ((size_t)blockIdx.x * 8 + warp - 2) * ATTN_WS_WARP;
 #pragma unroll 1
         for (int c = 0; c < 4; ++c) {
           uint32_t u[32];
           tmem_ld32(lane_base + o_col + c * 32, u);
           tmem_ld_wait();
           reg_fence32(u);
-          if (qrow < p.Lq) {
-            if (st32) {
 #pragma unroll
-              for (int q = 0; q < 2; ++q) {
-                uint32_t w[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                  w[i] = pack_bf16x2(__uint_as_float(u[q * 16 + 2 * i]) * inv,
-                                     __uint_as_float(u[q * 16 + 2 * i + 1]) * inv);
-                store_b32x8(orow + c * 32 + q * 16, w);
-              }
-            } else {
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                float v[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(u[q * 8 + i]) * inv;
-                store_bf16x8(orow + c * 32 + q * 8, v);
-              }
-            }
-          }
+          for (int q = 0; q < 8; ++q)
+            reinterpret_cast<float4*>(part)[(c * 8 + q) * 32 + lane] =
+                make_float4(__uint_as_float(u[4 * q]), __uint_as_float(u[4 * q + 1]),
+                            __uint_as_float(u[4 * q + 2]), __uint_as_float(u[4 * q + 3]));
+        }
+        reinterpret_cast<float2*>(part + 4096)[lane] = make_float2(m_used, l);
+        flag_due = true;
+      } else if (SPLIT && sg.kind == SEG_FINISH) {  // always the CTA's last segment
+        finish = true;
+        break;
+      } else {
+        const ORow out(p, sg.item, g * TB + r);
+        const float inv = 1.f / l;
+#pragma unroll 1
+        for (int c = 0; c < 4; ++c) {
+          uint32_t u[32];
+          tmem_ld32(lane_base + o_col + c * 32, u);
+          tmem_ld_wait();
+          reg_fence32(u);
+          out.store32(c, u, inv);
         }
       }
       ++cnt;
+    }
+    if (SPLIT && !failed) raise_due();
+    float a_own = 1.f;
+    if (SPLIT && finish) {
+      if (!join_parts(p, plan.c_lo, warp - 2, lane, m_used, l, a_own, err)) {
+        failed = true;
+        finish = false;
+      }
+    }
+    if (SPLIT && finish) {
+      const ORow out(p, plan.tail_item, g * TB + r);
+      const float inv = 1.f / l;
+#pragma unroll 1
+      for (int half = 0; half < 2; ++half) {
+        float4 f[16];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          uint32_t u[32];
+          tmem_ld32(lane_base + o_col + half * 64 + c * 32, u);
+          tmem_ld_wait();
+          reg_fence32(u);
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            f[c * 8 + q] = make_float4(
+                __uint_as_float(u[4 * q]) * a_own, __uint_as_float(u[4 * q + 1]) * a_own,
+                __uint_as_float(u[4 * q + 2]) * a_own, __uint_as_float(u[4 * q + 3]) * a_own);
+        }
+        add_parts(p, plan.c_lo, warp - 2, lane, m_used, half, f);
+        out.store32(half * 2, reinterpret_cast<const uint32_t*>(f), inv);
+        out.store32(half * 2 + 1, reinterpret_cast<const uint32_t*>(f + 8), inv);
+      }
     }
   }
 
@@ -1156,6 +1472,50 @@ bool map_o(CUtensorMap* m, const bf16* ptr, int batch, int Lq, int cols, int ld)
              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Chooses the persistent kernel's split and grid. Times in 128-key steps of a 256-query item
+// (1.45-1.55 us): whole items take their rounds; with the split every CTA takes an equal share,
+// its steps are about 5 % longer (the ranges share less K / V, the loop keeps more registers),
+// and storing, waiting for and adding the parts of cut items takes about 4.5 steps and one
+// more per part. Measured (us, whole items / split): 1 x 1560 x 12 heads 23.4 / 25.5, 2 x 1560
+// 40.8 / 35.2, 4 x 1560 60.9 / 57.8, 8 x 1560 103.3 / 102.7, 16 x 1560 186.9 / 202.9, 1 x 4096
+// 93.8 / 71.8, 4 x 4096 279.7 / 258.6, 1 x 1560 on 40 SMs 58.3 / 51.4, cross-attention (4 key
+// tiles) 4 x 1560 23.9 / 27.5.
+int plan_split(const AttnArgs& a, int sms, long items, Params* p) {
+  const int n_kv = (a.Lkv + TB - 1) / TB;
+  const long bh = (long)a.heads * a.batch;
+  p->n_full_qb = (a.Lq + TB - 1) / (2 * TB);
+  const long n_full = p->n_full_qb * bh, lone = items - n_full;
+  p->n_full = (int)n_full;
+  p->n_items = (int)items;
+  auto recip = [](int d) { return d > 1 ? (unsigned)((0x100000000ull + d - 1) / d) : 0u; };
+  p->div_qb = recip(p->n_full_qb);
+  p->div_heads = recip(a.heads);
+  p->ws = a.ws;
+  p->flags = a.flags;
+  p->split = 0;
+  p->rounds = 0;
+  const int grid = (int)(items < sms ? items : sms);
+  if (!a.ws || !a.flags || sms > a.ws_ctas) return grid;
+  // full rounds of two-tile items but one, so that every CTA's share of the rest is at least
+  // about one item and an item is cut in few parts
+  const double total = (4.0 * n_full + 3.0 * lone) * n_kv / 4;  // steps
+  long rounds = (long)(total / sms / n_kv) - 1;
+  if (rounds > n_full / sms) rounds = n_full / sms;
+  if (rounds < 0) rounds = 0;
+  const double rest = total - (double)rounds * sms * n_kv;
+  long G = sms;
+  if (rounds == 0 && rest / G < 3) G = (long)(rest / 3);  // at least 3 steps per CTA
+  if (G < 1) G = 1;
+  const double share = rest / G, parts = std::ceil(n_kv / share) + 1;
+  const double t_split = 1.05 * (rounds * n_kv + share) + 4.5 + parts;
+  const double t_whole = (double)((items + sms - 1) / sms) * n_kv;
+  // (the split's 32-bit unit arithmetic: see SplitUnits)
+  if (G <= 1 || t_split >= 0.98 * t_whole || total * 4 * sms > 4e9) return grid;
+  p->split = 1;
+  p->rounds = (int)rounds;
+  return (int)G;
+}
+
 }  // namespace
 
 cudaError_t attention_tc_set_wait_limit(unsigned long long ns) {
@@ -1201,20 +1561,21 @@ cudaError_t attention_tc(const AttnArgs& a, int* err, cudaStream_t st) {
   // 3. The shorter 128-query CTAs remain only where the 256-query form saves no waves
   // (both fit one wave, or Lq <= 128).
   const long ctas1 = (long)((a.Lq + TB - 1) / TB) * a.heads * a.batch;
-  const long ctas2 = (long)((a.Lq + 2 * TB - 1) / (2 * TB)) * a.heads * a.batch;
+  const long nqb = (a.Lq + 2 * TB - 1) / (2 * TB), ctas2 = nqb * a.heads * a.batch;
   const long w1 = (ctas1 + sms - 1) / sms, w2 = (ctas2 + sms - 1) / sms;
   const bool two = a.tc_variant >= 2 || (a.tc_variant == 0 && 4 * w1 >= 5 * w2);
   // 256-query items run in the persistent kernel (one CTA per SM looping over them, or one
   // item per CTA when they fit one wave: its MMA issue and slot releases are the leaner
   // ones, 1 x 1560 queries x 12 heads 25.8 -> 24.5 us); tc_variant 2 keeps the one-item
   // kernel
-  const bool persistent = a.tc_variant >= 3 || (two && a.tc_variant == 0);
+  const bool persistent = (a.tc_variant >= 3 || (two && a.tc_variant == 0)) &&
+                          ctas2 * (a.heads > nqb ? a.heads : nqb) < (1ll << 32);  // see div_by
   if (persistent) {
-    auto kern = attn_tc2p_kernel;
+    const int grid = plan_split(a, sms, ctas2, &p);
+    auto kern = p.split ? attn_tc2p_kernel<true> : attn_tc2p_kernel<false>;
     cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES);
     if (e != cudaSuccess) return e;
-    const int grid = (int)(ctas2 < sms ? ctas2 : sms);
     e = launch_k(kern, dim3(grid), dim3(THREADS2), SMEM2_BYTES, st, mq, mk, mv, p);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();

@@ -48,7 +48,14 @@ struct AttnArgs {
   int tc_variant;          // tcgen05 kernel: 0 automatic, 1 128-query CTAs, 2 256-query CTAs,
                            // 3 the persistent 256-query kernel
   int sms;                 // SMs the launch may use (its choice of CTA size); 0: the device's
+  // Workspace of the persistent kernel's split (null: whole items only): room for ws_ctas
+  // CTAs, and as many flag groups that start at zero and are left at zero.
+  float* ws;
+  int* flags;
+  int ws_ctas;
 };
+constexpr size_t ATTN_WS_FLOATS_PER_CTA = 8 * (32 * 128 + 64);
+constexpr int ATTN_FLAGS_PER_CTA = 8;
 // mma.sync (warp-level) kernel: head_dim 64 or 128.
 cudaError_t attention(const AttnArgs& a, cudaStream_t st);
 // tcgen05/TMEM kernel: head_dim 128, 16-byte aligned rows.

@@ -313,6 +313,40 @@ def test_attention(model, batch, Lq, Lkv, heads, dh, shared, impl):
         assert np.abs(got - want.reshape(Lq, D)).mean() <= 2e-3
 
 
+@pytest.mark.parametrize("batch,Lq,Lkv,heads,shared", [
+    (1, 1100, 2000, 40, False),   # single-tile items among the cut ones, 2.3 rounds of items
+    (3, 900, 1300, 14, False),    # 1.1 rounds: every item cut, ragged keys
+    (2, 1200, 1700, 19, True),    # shared K/V, 1.25 rounds
+    (5, 4096, 512, 12, True),     # four key tiles: not cut
+])
+def test_attention_key_split(model, batch, Lq, Lkv, heads, shared):
+    """Items whose key range is cut between CTAs (equal shares per SM): against the fp64
+    oracle on sampled heads, and bit for bit the same on a second and third call (the parts
+    are added in CTA order; the flags are back at zero)."""
+    D = heads * 128
+    q = randn((batch * Lq, D), 81)
+    k = randn(((1 if shared else batch) * Lkv, D), 82)
+    v = randn(((1 if shared else batch) * Lkv, D), 83)
+    outs = []
+    for _ in range(3):
+        o = torch.empty((batch * Lq, D), dtype=torch.bfloat16, device="cuda")
+        fb.fb_op_attention(model.handle, q, D, k, D, v, D, o, D, batch, Lq, Lkv,
+                           0 if shared else Lkv, heads, 128)
+        outs.append(o)
+    torch.cuda.synchronize()
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+    for b in range(batch):
+        kb = 0 if shared else b
+        for hd in sorted({0, heads // 2, heads - 1}):
+            c = slice(hd * 128, (hd + 1) * 128)
+            want = O.attention(f64(q[b * Lq:(b + 1) * Lq, c])[:, None],
+                               f64(k[kb * Lkv:(kb + 1) * Lkv, c])[:, None],
+                               f64(v[kb * Lkv:(kb + 1) * Lkv, c])[:, None]).reshape(Lq, 128)
+            got = f64(outs[0][b * Lq:(b + 1) * Lq, c])
+            assert rel_max(got, want) <= 2e-2
+            assert np.abs(got - want).mean() <= 2e-3
+
+
 def test_attention_strided_qkv(model):
     """Self-attention reading q, k, v from one packed [rows][3D] buffer."""
     batch, L, heads, dh = 2, 97, 2, 128
