@@ -68,12 +68,12 @@ cudaError_t attention_tc_set_wait_limit(unsigned long long ns);
 // out[r][:] = bf16(LN(x[r][:]) * (mul_base + mul[:]) + add[:]), x fp32 [rows][D].
 cudaError_t ln_mod(const float* x, bf16* out, int rows, int D, float eps, float mul_base,
                    const float* mul, const float* add, cudaStream_t st);
-// In place on bf16 rows: x[r][col0 + :D] = RMSNorm(.) * w, then (if rope != null) RoPE
-// with table rope[(r % tokens)][head_dim/2] of (cos, sin) per adjacent pair.
-// Two segments (col0, w0) and (col1, w1) when nseg == 2.
-cudaError_t qk_norm_rope(bf16* x, int rows, int ld, int D, int nseg, int col0, const float* w0,
-                         int col1, const float* w1, float eps, const float2* rope,
-                         int tokens, int head_dim, cudaStream_t st);
+// In place on bf16 rows, for each segment s < nseg (at most 65535): x[r][s dcol + :D] =
+// RMSNorm(.) * w0[s dw + :], then (if rope != null) RoPE with table rope[(r % tokens)]
+// [head_dim/2] of (cos, sin) per adjacent pair.
+cudaError_t qk_norm_rope(bf16* x, int rows, int ld, int D, int nseg, int dcol, const float* w0,
+                         ptrdiff_t dw, float eps, const float2* rope, int tokens, int head_dim,
+                         cudaStream_t st);
 // h[i] += sum_t coef[t] * anchor_t[i] over n_elems fp32 elements (bf16 anchors).
 #define FB_PROXY_MAX_TERMS 64
 struct ProxyTerms {

@@ -102,9 +102,8 @@ __device__ __forceinline__ void store_bf16x4(bf16* p, const float* v) {
 
 template <int THREADS, int VPT, int ROWS>
 __global__ void __launch_bounds__(THREADS * ROWS) qk_norm_rope_kernel(
-    bf16* __restrict__ x, int rows, int ld, int D, int col0, const float* __restrict__ w0,
-    int col1, const float* __restrict__ w1, float eps, const float2* __restrict__ rope,
-    int tokens, int head_dim) {
+    bf16* __restrict__ x, int rows, int ld, int D, int dcol, const float* __restrict__ w0,
+    ptrdiff_t dw, float eps, const float2* __restrict__ rope, int tokens, int head_dim) {
   static_assert(ROWS == 1 || THREADS == 32, "several rows per block need one warp per row");
   griddep_wait();
   griddep_launch();
@@ -113,9 +112,8 @@ __global__ void __launch_bounds__(THREADS * ROWS) qk_norm_rope_kernel(
   if (row >= (size_t)rows) return;
   const int tid = threadIdx.x % THREADS;
   const int seg = blockIdx.y;
-  const int col0s = seg ? col1 : col0;
-  const float* w = seg ? w1 : w0;
-  bf16* xr = x + row * ld + col0s;
+  const float* w = w0 + seg * dw;
+  bf16* xr = x + row * ld + (size_t)seg * dcol;
   float v[VPT][4];
   float ss = 0.f;
 #pragma unroll
@@ -146,12 +144,12 @@ __global__ void __launch_bounds__(THREADS * ROWS) qk_norm_rope_kernel(
 }
 
 template <int THREADS, int VPT, int ROWS = 1>
-cudaError_t qkn_launch(bf16* x, int rows, int ld, int D, int nseg, int col0, const float* w0,
-                       int col1, const float* w1, float eps, const float2* rope, int tokens,
-                       int head_dim, cudaStream_t st) {
+cudaError_t qkn_launch(bf16* x, int rows, int ld, int D, int nseg, int dcol, const float* w0,
+                       ptrdiff_t dw, float eps, const float2* rope, int tokens, int head_dim,
+                       cudaStream_t st) {
   dim3 grid((rows + ROWS - 1) / ROWS, nseg);
   return launch_k(qk_norm_rope_kernel<THREADS, VPT, ROWS>, grid, dim3(THREADS * ROWS), 0, st, x,
-                  rows, ld, D, col0, w0, col1, w1, eps, rope, tokens, head_dim);
+                  rows, ld, D, dcol, w0, dw, eps, rope, tokens, head_dim);
 }
 
 // ---------------------------------------------------------------------------------
@@ -458,12 +456,12 @@ cudaError_t ln_mod(const float* x, bf16* out, int rows, int D, float eps, float 
   return cudaErrorInvalidValue;
 }
 
-cudaError_t qk_norm_rope(bf16* x, int rows, int ld, int D, int nseg, int col0, const float* w0,
-                         int col1, const float* w1, float eps, const float2* rope, int tokens,
-                         int head_dim, cudaStream_t st) {
+cudaError_t qk_norm_rope(bf16* x, int rows, int ld, int D, int nseg, int dcol, const float* w0,
+                         ptrdiff_t dw, float eps, const float2* rope, int tokens, int head_dim,
+                         cudaStream_t st) {
   if (rows == 0) return cudaSuccess;
 #define QKN(T, V, ...) \
-  qkn_launch<T, V, ##__VA_ARGS__>(x, rows, ld, D, nseg, col0, w0, col1, w1, eps, rope, tokens, head_dim, st)
+  qkn_launch<T, V, ##__VA_ARGS__>(x, rows, ld, D, nseg, dcol, w0, dw, eps, rope, tokens, head_dim, st)
   switch (D) {  // threads * 4 * VPT == D
     case 128: return QKN(32, 1);
     case 256: return QKN(64, 1);
