@@ -175,7 +175,8 @@ struct fb_model {
   float* noise = nullptr;   // device copy of host SDE draws, grown on demand
   size_t noise_elems = 0;
   bool text_ready = false;
-  float *emb = nullptr, *th1 = nullptr, *temb = nullptr, *mod = nullptr, *modl = nullptr,
+  // conditioning, FB_COND_STEPS rows each (tembs: SiLU(temb))
+  float *emb = nullptr, *th1 = nullptr, *temb = nullptr, *tembs = nullptr, *mod = nullptr, *modl = nullptr,
         *hmod = nullptr;
   float2* rope = nullptr;
   float* zbuf = nullptr;
@@ -422,30 +423,36 @@ fb_status encode_text(fb_model* m, const float* ctx, bf16* kv_dst) {
   return FB_OK;
 }
 
-// ---- per-step conditioning: temb, mod, per-layer modulation, head modulation ---------
-// have_emb: m->emb already holds the sinusoid of t (written by the previous step's
-// Euler kernel)
-fb_status time_embed(fb_model* m, float t, bool have_emb = false) {
+// ---- conditioning: temb, mod, per-layer modulation, head modulation -------------------
+// for the ns <= FB_COND_STEPS timesteps t[0 .. ns - 1] (one row each of the buffers). The
+// sampler takes a chunk of steps at a time: five launches per chunk instead of per step, the
+// weights (28 MB of modulation at dim 1536) read once per chunk.
+fb_status time_embed(fb_model* m, const float* t, int ns) {
   const fb_cfg& c = m->c;
   const int D = c.dim;
-  KTimer k(m, FB_K_SMALL, 2.0 * D * (c.freq_dim + D + 6.0 * D),
-           2.0 * D * (c.freq_dim + D + 6.0 * D), have_emb ? 4 : 5);
-  if (!have_emb) CK(timestep_sincos(t, c.freq_dim, m->emb, m->st));
-  CK(gemv(m->time_w1, m->time_b1, m->emb, m->th1, D, c.freq_dim, 0, 1, m->st));
-  CK(gemv(m->time_w2, m->time_b2, m->th1, m->temb, D, D, 0, 0, m->st));
-  CK(gemv(m->mod_w, m->mod_b, m->temb, m->mod, 6 * D, D, 1, 0, m->st));
-  CK(mod_prepare(m->mod, m->tables, c.depth, D, m->modl, m->head_table, m->temb, m->hmod, m->st));
+  CondSteps ts{};
+  for (int i = 0; i < ns; ++i) ts.t[i] = t[i];
+  KTimer k(m, FB_K_SMALL, 2.0 * ns * D * (c.freq_dim + D + 6.0 * D),
+           2.0 * D * (c.freq_dim + D + 6.0 * D), 5);
+  CK(timestep_sincos(ts, ns, c.freq_dim, m->emb, m->st));
+  CK(gemv(m->time_w1, m->time_b1, m->emb, nullptr, m->th1, D, c.freq_dim, ns, m->st));
+  CK(gemv(m->time_w2, m->time_b2, m->th1, m->temb, m->tembs, D, D, ns, m->st));
+  CK(gemv(m->mod_w, m->mod_b, m->tembs, m->mod, nullptr, 6 * D, D, ns, m->st));
+  CK(mod_prepare(m->mod, m->tables, c.depth, D, ns, m->modl, m->head_table, m->temb, m->hmod,
+                 m->st));
   return FB_OK;
 }
 
 // ---- one block B_l (Eq. 7) on h = hA (rows M), optional contribution write ----------
 // n: candidates (rows n*P). n_uncond > 0: the last n_uncond candidates are the
-// unconditional rows of guidance and attend to the unconditional text context.
-fb_status block_forward(fb_model* m, int l, float* h, int n, bf16* delta, int n_uncond = 0) {
+// unconditional rows of guidance and attend to the unconditional text context. cond: the
+// timestep's row of the conditioning buffers.
+fb_status block_forward(fb_model* m, int l, float* h, int n, bf16* delta, int n_uncond = 0,
+                        int cond = 0) {
   const fb_cfg& c = m->c;
   const int D = c.dim, M = n * m->P;
   const Layer& w = m->L[l];
-  const float* md = m->modl + (size_t)l * 6 * D;
+  const float* md = m->modl + ((size_t)cond * c.depth + l) * 6 * D;
   const float *s1 = md, *c1 = md + D, *g1 = md + 2 * D, *s2 = md + 3 * D, *c2 = md + 4 * D,
               *g2 = md + 5 * D;
   float* hB = m->hB;
@@ -709,13 +716,14 @@ fb_status sample(fb_model* m, float* z, int n, const float* sched, int S, const 
   CKS(ensure_anchors(m, need));
   const int M = nr * m->P;
   const size_t zn = (size_t)n * c.latent_c * c.latent_h * c.latent_w;
-  // with the tensor-core head, each step's Euler kernel also writes the next step's
-  // sinusoidal embedding and patch rows (step 0 computes its own)
+  // with the tensor-core head, each step's Euler kernel also writes the next step's patch
+  // rows (step 0 computes its own)
   const bool fused_next = m->vbuf && m->patch_a;
   for (int k = 0; k < S; ++k) {
     const float t = sched[k], t1 = sched[k + 1];
     const bool from_prev = fused_next && k > 0;
-    CKS(time_embed(m, t, from_prev));
+    const int cond = k % FB_COND_STEPS;
+    if (cond == 0) CKS(time_embed(m, sched + k, std::min(S - k, FB_COND_STEPS)));
     for (int u = 0; u < (so.guided ? 2 : 1); ++u) {
       float* hu = m->hA + (size_t)u * n * m->P * c.dim;
       const bool rows_ready = from_prev || u > 0;
@@ -738,7 +746,7 @@ fb_status sample(fb_model* m, float* z, int n, const float* sched, int S, const 
       if (a.type == 0) {
         bf16* d = a.slot >= 0 ? m->anchors + (size_t)a.slot * slot_elems : nullptr;
         CKS(wait_slot(m, a.slot, slot_elems));
-        CKS(block_forward(m, a.layer, m->hA, nr, d, so.guided ? n : 0));
+        CKS(block_forward(m, a.layer, m->hA, nr, d, so.guided ? n : 0, cond));
       } else {
         for (size_t i0 = 0; i0 < a.terms.size(); i0 += FB_PROXY_MAX_TERMS) {
           ProxyTerms pt{};
@@ -753,7 +761,8 @@ fb_status sample(fb_model* m, float* z, int n, const float* sched, int S, const 
         }
       }
     }
-    CKS(run_ln(m, m->hA, m->act, M, 1.f, m->hmod + c.dim, m->hmod));
+    const float* hmod = m->hmod + (size_t)cond * 2 * c.dim;
+    CKS(run_ln(m, m->hA, m->act, M, 1.f, hmod + c.dim, hmod));
     {
       HeadStep hs{};
       hs.dt = t1 - t;
@@ -777,9 +786,6 @@ fb_status sample(fb_model* m, float* z, int n, const float* sched, int S, const 
         CK(gemm_tc(g, m->derr, m->num_sms, m->st));
         if (k + 1 < S && m->patch_a) {
           hs.patch_next = m->patch_a;
-          hs.emb_next = m->emb;
-          hs.t_next = t1;
-          hs.freq_dim = c.freq_dim;
         }
         CK(euler_step(m->vbuf, m->npad, n, c.latent_c, c.latent_h, c.latent_w, c.patch, hs, z,
                       m->st));
@@ -1055,9 +1061,13 @@ fb_status fb_init_model(const fb_cfg* cfg, const float* weights_host, fb_model**
       (s = dalloc_t(m, &m->ctx_h, (size_t)c.text_len * D)) ||
       (s = dalloc_t(m, &m->ctx_p, (size_t)c.text_len * D)) ||
       (s = dalloc_t(m, &m->kvctx, (size_t)c.depth * c.text_len * 2 * D)) ||
-      (s = dalloc_t(m, &m->emb, (size_t)c.freq_dim)) || (s = dalloc_t(m, &m->th1, D)) ||
-      (s = dalloc_t(m, &m->temb, D)) || (s = dalloc_t(m, &m->mod, 6 * D)) ||
-      (s = dalloc_t(m, &m->modl, (size_t)c.depth * 6 * D)) || (s = dalloc_t(m, &m->hmod, 2 * D)) ||
+      (s = dalloc_t(m, &m->emb, (size_t)FB_COND_STEPS * c.freq_dim)) ||
+      (s = dalloc_t(m, &m->th1, FB_COND_STEPS * D)) ||
+      (s = dalloc_t(m, &m->temb, FB_COND_STEPS * D)) ||
+      (s = dalloc_t(m, &m->tembs, FB_COND_STEPS * D)) ||
+      (s = dalloc_t(m, &m->mod, FB_COND_STEPS * 6 * D)) ||
+      (s = dalloc_t(m, &m->modl, (size_t)FB_COND_STEPS * c.depth * 6 * D)) ||
+      (s = dalloc_t(m, &m->hmod, FB_COND_STEPS * 2 * D)) ||
       (s = dalloc_t(m, &m->rope, (size_t)m->P * c.head_dim / 2)) ||
       (s = dalloc_t(m, &m->zbuf, zn)) || (s = dalloc_t(m, &m->derr, 1)))
     return bail(s);
@@ -1295,7 +1305,7 @@ fb_status fb_block_forward(fb_model* m, int layer, float* h, int n, float t) {
   if (n == 0) return FB_OK;
   if (!is_device_ptr(h)) return fail(FB_EINVAL, "h must be device memory");
   CKS(begin_call(m));
-  CKS(time_embed(m, t));
+  CKS(time_embed(m, &t, 1));
   CKS(block_forward(m, layer, h, n, nullptr));
   return end_call(m);
 }

@@ -359,7 +359,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const uint32_t rank = cluster_ctarank();
   const int cluster = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
-  const int n_mt = (M + T - 1) / T, n_nt = N / C2_BN, n_tiles = n_mt * n_nt;
+  const int n_mt = (M + T - 1) / T, n_nt = (N + C2_BN - 1) / C2_BN, n_tiles = n_mt * n_nt;
   const int nk = K / BK;
   const int stage_bytes = C2_W_BYTES + T / 2 * BK * 2;
   const int stages = c2_stages(T, CC::RING_BYTES);
@@ -496,10 +496,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
       const int f0 = (tile % n_nt) * C2_BN + 128 * (int)rank + quarter * 32;
       const int nv = M - m0 < T ? M - m0 : T;  // valid tokens of the tile
       // this warp's chunks: i = 0, 1, ... covers tokens (half + 2 i) * CH ..
-      const int ncht = (nv + CH - 1) / CH, nch = (ncht + 1 - half) / 2;
+      // (none if its features lie past N, a multiple of 128)
+      const int ncht = (nv + CH - 1) / CH, nch = f0 < N ? (ncht + 1 - half) / 2 : 0;
       const size_t off0 = (size_t)(m0 + half * CH) * epi.ldo + f0 + lane;
-      const float bias = head && epi.bias ? __ldg(epi.bias + f0 + lane) : 0.f;
-      const float gate = CC::F32 && head && epi.gate ? __ldg(epi.gate + f0 + lane) : 1.f;
+      const float bias = nch && head && epi.bias ? __ldg(epi.bias + f0 + lane) : 0.f;
+      const float gate = CC::F32 && nch && head && epi.gate ? __ldg(epi.gate + f0 + lane) : 1.f;
       // residual chunk i into tile i % NBUF (one lane)
       auto rload_issue = [&](int i) {
         const int t = i % NBUF;
@@ -792,7 +793,8 @@ int choose_tile(int M, int N, int nk, int mc) {
   int best_T = 256;
   double best = 0;
   for (int T = 256; T >= 16; T -= 16) {
-    const long tiles = (long)((M + T - 1) / T) * (N / C2_BN), rounds = (tiles + mc - 1) / mc;
+    const long tiles = (long)((M + T - 1) / T) * ((N + C2_BN - 1) / C2_BN);
+    const long rounds = (tiles + mc - 1) / mc;
     const double main = (double)nk * (256 + T > 313 ? 256 + T : 313), epilogue = 16.0 * T + 400;
     const double est = rounds * (main > epilogue ? main : epilogue) + epilogue;
     if (best == 0 || est < best) {
@@ -839,14 +841,14 @@ cudaError_t launch2(const GemmArgs& g, int* err, int num_sms, cudaStream_t st) {
   const long rounds256 = (tiles256 + mc - 1) / mc;
   const double operand_bytes = 2.0 * ((double)g.M + g.N) * g.K;
   const bool sk_ok =
-      g.sk_ws && g.sk_ctr && mc <= g.sk_clusters && tiles256 * (long long)nk >= 4LL * mc;
+      g.N % C2_BN == 0 && g.sk_ws && g.sk_ctr && mc <= g.sk_clusters && tiles256 * (long long)nk >= 4LL * mc;
   const bool sk_pays = rounds256 <= 4 && (rounds256 * mc - tiles256) * nk >= 24LL * mc &&
                        operand_bytes <= 64.0 * 1024 * 1024;
   if (g.sk_mode == 2 && !sk_ok) return cudaErrorInvalidValue;
   SkArgs sk{g.sk_mode == 2 || (g.sk_mode == 0 && sk_ok && sk_pays) ? 1 : 0, g.sk_ws, g.sk_ctr};
   // stream-K keeps T = 256: fewer tiles to cut and shorter K ranges to sum
   const int T = sk.on ? 256 : choose_tile(g.M, g.N, nk, mc);
-  const int tiles = (g.M + T - 1) / T * (g.N / C2_BN);
+  const int tiles = (g.M + T - 1) / T * ((g.N + C2_BN - 1) / C2_BN);
   CUtensorMap ma, mw, mo, mr{};  // mr: unused without a residual
   if (!make_map(&ma, g.A, g.M, g.K, g.lda, T / 2) || !make_map(&mw, g.W, g.N, g.K, g.ldw, 128) ||
       !make_epi_map(&mo, g.epi.out, C2Cfg<KIND>::F32, g.M, g.N, g.epi.ldo) ||
@@ -882,9 +884,13 @@ cudaError_t gemm_tc_set_wait_limit(unsigned long long ns) { return fb_set_wait_l
 
 cudaError_t gemm_tc(const GemmArgs& g, int* err, int num_sms, cudaStream_t st, bool force_1sm) {
   if (!gemm_tc_supported(g)) return cudaErrorInvalidValue;
-  // 2-SM tiles of 256 features x T tokens whenever N allows; otherwise 1-SM 128 x BN tiles, BN = 256
-  // when that still gives every SM a tile.
-  if (g.N % C2_BN == 0 && !force_1sm && num_sms >= 2) return dispatch2(g, err, num_sms, st);
+  // 2-SM tiles of 256 features x T tokens; where N leaves half of the last feature tile empty
+  // (N % 256 == 128) only past one 128-row tile, where T spreads the rows over more SMs than
+  // the 1-SM kernel's 128 x BN tiles (BN = 256 when that still gives every SM a tile): the
+  // head's 1560 x 128 x 1536 took 13 SMs and 13.3 us there.
+  const bool half_tile = g.N % C2_BN != 0;
+  if (!force_1sm && num_sms >= 2 && (!half_tile || (g.M > BM && g.sk_mode != 2)))
+    return dispatch2(g, err, num_sms, st);
   if (g.sk_mode == 2) return cudaErrorInvalidValue;  // stream-K exists in the 2-SM kernel only
   const int mt = (g.M + BM - 1) / BM;
   if (g.N % 256 == 0 && mt * (g.N / 256) >= num_sms) return dispatch_kind<256>(g, err, num_sms, st);

@@ -93,13 +93,9 @@ struct HeadStep {
   float dt, t, w, sde_c, nscale;
   int uncond_rows;        // 0: no guidance
   const float* noise;     // null: ODE step
-  // euler_step only: the next step's conditioning, written from the updated z (null: last
-  // step). patch_next: bf16 patch rows (as patchify writes them); emb_next: the sinusoidal
-  // embedding of t_next (as timestep_sincos writes it, freq_dim entries).
+  // euler_step only: the next step's bf16 patch rows of the updated z, as patchify writes
+  // them (null: last step)
   bf16* patch_next;
-  float* emb_next;
-  float t_next;
-  int freq_dim;
 };
 cudaError_t head_euler(const bf16* a, int n, int C, int H, int W, int p, const bf16* Wh,
                        const float* bh, int D, const HeadStep& hs, float* z, cudaStream_t st);
@@ -109,19 +105,22 @@ cudaError_t patchify(const float* z, int n, int C, int H, int W, int p, bf16* ou
                      cudaStream_t st);
 // The guidance combination and step of head_euler, with v[row][o] (fp32, leading dimension
 // ldv >= C p p) the head output a Wh^T + bh computed by the tensor-core GEMM; with
-// hs.patch_next / hs.emb_next also the next step's patch rows and timestep embedding
-// (C p p % 8 == 0).
+// hs.patch_next also the next step's patch rows (C p p % 8 == 0).
 cudaError_t euler_step(const float* v, int ldv, int n, int C, int H, int W, int p,
                        const HeadStep& hs, float* z, cudaStream_t st);
-// y[o] = act_out(b[o] + sum_k W[o][k] act_in(x[k])), act: 0 none, 1 SiLU.
-cudaError_t gemv(const bf16* W, const float* b, const float* x, float* y, int O, int K,
-                 int act_in, int act_out, cudaStream_t st);
-// emb = [cos(1000 t f_k), sin(1000 t f_k)], f_k = 10000^(-k/half).
-cudaError_t timestep_sincos(float t, int dim, float* emb, cudaStream_t st);
-// modl[l][j][:] = mod[j][:] + table_l[j][:] (6 rows, all layers); head[j] = htab[j] + temb.
-cudaError_t mod_prepare(const float* mod, const float* tables, int L, int D,
-                        float* modl, const float* htab, const float* temb, float* head_mod,
-                        cudaStream_t st);
+// Conditioning for ns <= FB_COND_STEPS timesteps at once (their vectors are rows).
+#define FB_COND_STEPS 8
+struct CondSteps {
+  float t[FB_COND_STEPS];
+};
+// y[s][o] = b[o] + sum_k W[o][k] x[s][k] and ysilu[s][o] = SiLU of it (either may be null).
+cudaError_t gemv(const bf16* W, const float* b, const float* x, float* y, float* ysilu, int O,
+                 int K, int ns, cudaStream_t st);
+// emb[s] = [cos(1000 t_s f_k), sin(1000 t_s f_k)], f_k = 10000^(-k/half).
+cudaError_t timestep_sincos(const CondSteps& ts, int ns, int dim, float* emb, cudaStream_t st);
+// modl[s][l][j][:] = mod[s][j][:] + table_l[j][:] (6 rows, all layers); head[s][j] = htab[j] + temb[s].
+cudaError_t mod_prepare(const float* mod, const float* tables, int L, int D, int ns, float* modl,
+                        const float* htab, const float* temb, float* head_mod, cudaStream_t st);
 cudaError_t f32_to_bf16(const float* x, bf16* y, size_t n, cudaStream_t st);
 
 // ---- measurement probe ----------------------------------------------------------------

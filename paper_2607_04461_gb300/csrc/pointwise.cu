@@ -9,7 +9,8 @@
 //               z += (t' - t) v of dx = v dt, fused (CUDA cores, any C p p).
 //  patchify     z -> bf16 patch rows, the A operand of the tensor-core patch embedding.
 //  euler_step   the step of head_euler from the tensor-core head GEMM's output.
-//  gemv, timestep_sincos, mod_prepare, f32_to_bf16: per-step conditioning, conversions.
+//  gemv, timestep_sincos, mod_prepare, f32_to_bf16: conditioning (a chunk of timesteps at a
+//               time), conversions.
 #include "kernels.h"
 
 namespace {
@@ -243,56 +244,55 @@ __global__ void __launch_bounds__(256) patchify_kernel(const float* __restrict__
 }
 
 // euler_step: the guidance combination and the ODE / SDE step of head_euler, from the
-// head output v[row][o] (bias included) of the tensor-core head GEMM, fused with the next
-// step's conditioning inputs: the bf16 patch rows of the updated z (the A operand of the
-// next patch embedding) and the sinusoidal embedding of the next t. One block per token
-// row (p latent rows) of one candidate: threads walk the latent in memory order (each
-// element reads output o = (ch, y % p, x % p) of token x / p), then the updated values
-// leave through a shared-memory tile [token][o] as whole 16-byte patch-row chunks.
-__device__ __forceinline__ void sincos_entry(float t, int k, int half, float* emb) {
-  // f_k = 10000^(-k/half); the argument is formed in double for accuracy at 1000 t
-  const double f = exp(-9.210340371976184 * (double)k / (double)half);
-  const double arg = 1000.0 * (double)t * f;
-  emb[k] = (float)cos(arg);
-  emb[half + k] = (float)sin(arg);
-}
-
+// head output v[row][o] (bias included) of the tensor-core head GEMM, fused with the bf16
+// patch rows of the updated z (the A operand of the next patch embedding). One block per
+// EU_TOK tokens of one token row (p latent rows) of one candidate: v arrives by whole rows
+// into a shared-memory tile [o][token] (odd pitch), z is updated in memory order (each
+// element reads output o = (ch, y % p, x % p) of token x / p), and the new values leave the
+// tile as 16-byte patch-row chunks. One candidate's 1560 tokens are 120 blocks; a block per
+// whole token row (30) that also formed the next step's timestep embedding took 14 us.
+constexpr int EU_TOK = 16;
 __global__ void __launch_bounds__(256) euler_step_kernel(const float* __restrict__ v, int ldv,
-                                                         int n, int C, int H, int W, int p,
-                                                         HeadStep hs, float* __restrict__ z) {
-  extern __shared__ float tile[];  // [W / p tokens][C p p] when hs.patch_next
+                                                         int C, int H, int W, int p, HeadStep hs,
+                                                         float* __restrict__ z) {
+  extern __shared__ float tile[];  // [C p p][EU_TOK + 1]
   griddep_wait();
   griddep_launch();
-  const int PD = C * p * p, gw = W / p, gh = H / p, P = gh * gw;
-  const int r = blockIdx.x % gh, b = blockIdx.x / gh;  // token row r of candidate b
-  if (hs.emb_next && blockIdx.x == 0) {
-    const int half = hs.freq_dim / 2;
-    for (int k = threadIdx.x; k < half; k += blockDim.x)
-      sincos_entry(hs.t_next, k, half, hs.emb_next);
-  }
-  const size_t tok0 = (size_t)b * P + (size_t)r * gw;  // first token of the row
-  const int row_elems = C * p * W;                      // (ch, dy, x) of the p latent rows
-  for (int e = threadIdx.x; e < row_elems; e += blockDim.x) {
-    const int x = e % W, dy = (e / W) % p, ch = e / (W * p);
-    const size_t zi = (((size_t)b * C + ch) * H + (size_t)r * p + dy) * W + x;
-    const int tok = x / p, o = (ch * p + dy) * p + x % p;
-    float vv = v[(tok0 + tok) * ldv + o];
+  const int PD = C * p * p, gw = W / p, gh = H / p;
+  const int nchunk = (gw + EU_TOK - 1) / EU_TOK;
+  const int c = blockIdx.x % nchunk, r = blockIdx.x / nchunk % gh, b = blockIdx.x / nchunk / gh;
+  const int tok_in_row = c * EU_TOK, nt = min(EU_TOK, gw - tok_in_row);
+  const size_t tok0 = ((size_t)b * gh + r) * gw + tok_in_row;
+  for (int e = threadIdx.x; e < nt * PD; e += blockDim.x) {
+    const int t = e / PD, o = e % PD;
+    float vv = v[(tok0 + t) * ldv + o];
     if (hs.uncond_rows) {
-      const float vu = v[(tok0 + tok + hs.uncond_rows) * ldv + o];
+      const float vu = v[(tok0 + t + hs.uncond_rows) * ldv + o];
       vv = vu + hs.w * (vv - vu);
     }
-    const float zo = z[zi];
+    tile[o * (EU_TOK + 1) + t] = vv;
+  }
+  __syncthreads();
+  const int nx = nt * p;  // latent columns of the block
+  for (int e = threadIdx.x; e < C * p * nx; e += blockDim.x) {
+    const int xl = e % nx, dy = e / nx % p, ch = e / (nx * p);
+    const size_t zi = (((size_t)b * C + ch) * H + (size_t)r * p + dy) * W + tok_in_row * p + xl;
+    float& cell = tile[((ch * p + dy) * p + xl % p) * (EU_TOK + 1) + xl / p];
+    const float zo = z[zi], vv = cell;
     const float zn = hs.noise ? zo + (vv + hs.sde_c * (zo + (1.f - hs.t) * vv)) * hs.dt +
                                     hs.nscale * hs.noise[zi]
                               : zo + hs.dt * vv;
     z[zi] = zn;
-    if (hs.patch_next) tile[tok * PD + o] = zn;
+    cell = zn;
   }
   if (!hs.patch_next) return;
   __syncthreads();
-  for (int c = threadIdx.x; c < gw * (PD / 8); c += blockDim.x) {
-    const int tok = c / (PD / 8), o0 = (c % (PD / 8)) * 8;
-    store_bf16x8(hs.patch_next + (tok0 + tok) * PD + o0, tile + tok * PD + o0);
+  for (int q = threadIdx.x; q < nt * (PD / 8); q += blockDim.x) {
+    const int t = q / (PD / 8), o0 = (q % (PD / 8)) * 8;
+    float x[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) x[j] = tile[(o0 + j) * (EU_TOK + 1) + t];
+    store_bf16x8(hs.patch_next + (tok0 + t) * PD + o0, x);
   }
 }
 
@@ -371,40 +371,73 @@ __global__ void __launch_bounds__(256) head_euler_kernel(const bf16* __restrict_
 }
 
 // ---------------------------------------------------------------------------------
-// gemv: one warp per output row.
+// gemv: one warp per output row, for NS input vectors at once (the timesteps of a chunk: the
+// weights are read once). A lane has four 16-byte weight loads in flight; the sum of a vector
+// does not depend on NS or on the other vectors.
+template <int NS>
 __global__ void __launch_bounds__(256) gemv_kernel(const bf16* __restrict__ W,
                                                    const float* __restrict__ b,
                                                    const float* __restrict__ x,
-                                                   float* __restrict__ y, int O, int K,
-                                                   int act_in, int act_out) {
+                                                   float* __restrict__ y, float* __restrict__ ysilu,
+                                                   int O, int K, int ns) {
   griddep_wait();
   griddep_launch();
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
-  if (warp >= O) return;
-  const bf16* wr = W + (size_t)warp * K;
-  float acc = 0.f;
-  for (int k = lane * 8; k < K; k += 32 * 8) {
-    float wv[8], xv[8];
-    load_bf16x8(wr + k, wv);
-    load_f32x8(x + k, xv);
+  const int row = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x % 32;
+  if (row >= O) return;
+  const bf16* wr = W + (size_t)row * K;
+  float acc[NS];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc += wv[j] * (act_in ? silu_f(xv[j]) : xv[j]);
+  for (int s = 0; s < NS; ++s) acc[s] = 0.f;
+  for (int k0 = lane * 8; k0 < K; k0 += 4 * 256) {
+    uint4 u[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (k0 + i * 256 < K) u[i] = *reinterpret_cast<const uint4*>(wr + k0 + i * 256);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = k0 + i * 256;
+      if (k >= K) break;
+      const float2 a = unpack_bf16x2(u[i].x), c = unpack_bf16x2(u[i].y), d = unpack_bf16x2(u[i].z),
+                   e = unpack_bf16x2(u[i].w);
+      const float wv[8] = {a.x, a.y, c.x, c.y, d.x, d.y, e.x, e.y};
+#pragma unroll
+      for (int s = 0; s < NS; ++s) {
+        if (NS > 1 && s >= ns) break;
+        float xv[8];
+        load_f32x8(x + (size_t)s * K + k, xv);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[s] += wv[j] * xv[j];
+      }
+    }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) {
-    float v = acc + (b ? b[warp] : 0.f);
-    y[warp] = act_out ? silu_f(v) : v;
+  for (int s = 0; s < NS; ++s) {
+    if (NS > 1 && s >= ns) break;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[s] += __shfl_xor_sync(0xffffffffu, acc[s], o);
+    if (lane == 0) {
+      const float v = acc[s] + (b ? b[row] : 0.f);
+      if (y) y[(size_t)s * O + row] = v;
+      if (ysilu) ysilu[(size_t)s * O + row] = silu_f(v);
+    }
   }
 }
 
-__global__ void timestep_sincos_kernel(float t, int dim, float* emb) {
+// one block per timestep
+__global__ void timestep_sincos_kernel(CondSteps st, int dim, float* emb) {
   griddep_wait();
   griddep_launch();
   const int half = dim / 2;
-  for (int k = threadIdx.x; k < half; k += blockDim.x) sincos_entry(t, k, half, emb);
+  for (int k = threadIdx.x; k < half; k += blockDim.x) {
+    // f_k = 10000^(-k/half); the argument is formed in double for accuracy at 1000 t
+    const double f = exp(-9.210340371976184 * (double)k / (double)half);
+    const double arg = 1000.0 * (double)st.t[blockIdx.x] * f;
+    emb[(size_t)blockIdx.x * dim + k] = (float)cos(arg);
+    emb[(size_t)blockIdx.x * dim + half + k] = (float)sin(arg);
+  }
 }
 
+// blockIdx.y: timestep
 __global__ void mod_prepare_kernel(const float* __restrict__ mod,
                                    const float* __restrict__ tables, int L, int D,
                                    float* __restrict__ modl, const float* __restrict__ htab,
@@ -412,11 +445,14 @@ __global__ void mod_prepare_kernel(const float* __restrict__ mod,
   griddep_wait();
   griddep_launch();
   const size_t n6 = 6 * (size_t)D;
+  mod += blockIdx.y * n6;
+  modl += blockIdx.y * n6 * L;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (size_t)L * n6;
        i += (size_t)gridDim.x * blockDim.x)
     modl[i] = mod[i % n6] + tables[i];
   if (blockIdx.x == 0)
-    for (int i = threadIdx.x; i < 2 * D; i += blockDim.x) head_mod[i] = htab[i] + temb[i % D];
+    for (int i = threadIdx.x; i < 2 * D; i += blockDim.x)
+      head_mod[(size_t)blockIdx.y * 2 * D + i] = htab[i] + temb[(size_t)blockIdx.y * D + i % D];
 }
 
 __global__ void f32_to_bf16_kernel(const float* __restrict__ x, bf16* __restrict__ y, size_t n) {
@@ -495,11 +531,11 @@ cudaError_t euler_step(const float* v, int ldv, int n, int C, int H, int W, int 
                        const HeadStep& hs, float* z, cudaStream_t st) {
   const int PD = C * p * p;
   if (H % p || W % p || ldv < PD || PD % 8) return cudaErrorInvalidValue;
-  const size_t smem = hs.patch_next ? (size_t)(W / p) * PD * sizeof(float) : 0;
-  if (smem > 48 * 1024) return cudaErrorInvalidValue;  // one token row's tile
   if (n == 0) return cudaSuccess;
-  return launch_k(euler_step_kernel, dim3(n * (H / p)), dim3(256), smem, st, v, ldv, n, C, H, W, p,
-                  hs, z);
+  const size_t smem = (size_t)PD * (EU_TOK + 1) * sizeof(float);
+  const int nchunk = (W / p + EU_TOK - 1) / EU_TOK;
+  return launch_k(euler_step_kernel, dim3(n * (H / p) * nchunk), dim3(256), smem, st, v, ldv, C, H,
+                  W, p, hs, z);
 }
 
 cudaError_t proxy_add(float* h, size_t n_elems, const ProxyTerms& t, cudaStream_t st) {
@@ -540,21 +576,23 @@ cudaError_t head_euler(const bf16* a, int n, int C, int H, int W, int p, const b
 #undef HE
 }
 
-cudaError_t gemv(const bf16* W, const float* b, const float* x, float* y, int O, int K,
-                 int act_in, int act_out, cudaStream_t st) {
-  if (K % 8) return cudaErrorInvalidValue;
-  return launch_k(gemv_kernel, dim3((O * 32 + 255) / 256), dim3(256), 0, st, W, b, x, y, O, K,
-                  act_in, act_out);
+cudaError_t gemv(const bf16* W, const float* b, const float* x, float* y, float* ysilu, int O,
+                 int K, int ns, cudaStream_t st) {
+  if (K % 8 || ns < 1 || ns > FB_COND_STEPS) return cudaErrorInvalidValue;
+  const dim3 grid((O * 32 + 255) / 256);
+  return ns == 1 ? launch_k(gemv_kernel<1>, grid, dim3(256), 0, st, W, b, x, y, ysilu, O, K, ns)
+                 : launch_k(gemv_kernel<FB_COND_STEPS>, grid, dim3(256), 0, st, W, b, x, y, ysilu,
+                            O, K, ns);
 }
 
-cudaError_t timestep_sincos(float t, int dim, float* emb, cudaStream_t st) {
-  return launch_k(timestep_sincos_kernel, dim3(1), dim3(128), 0, st, t, dim, emb);
+cudaError_t timestep_sincos(const CondSteps& ts, int ns, int dim, float* emb, cudaStream_t st) {
+  return launch_k(timestep_sincos_kernel, dim3(ns), dim3(128), 0, st, ts, dim, emb);
 }
 
-cudaError_t mod_prepare(const float* mod, const float* tables, int L, int D, float* modl,
+cudaError_t mod_prepare(const float* mod, const float* tables, int L, int D, int ns, float* modl,
                         const float* htab, const float* temb, float* head_mod, cudaStream_t st) {
-  return launch_k(mod_prepare_kernel, dim3(grid_for((size_t)L * 6 * D, 256)), dim3(256), 0, st, mod,
-                  tables, L, D, modl, htab, temb, head_mod);
+  return launch_k(mod_prepare_kernel, dim3(grid_for((size_t)L * 6 * D, 256), ns), dim3(256), 0, st,
+                  mod, tables, L, D, modl, htab, temb, head_mod);
 }
 
 cudaError_t f32_to_bf16(const float* x, bf16* y, size_t n, cudaStream_t st) {
