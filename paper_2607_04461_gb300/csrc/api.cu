@@ -182,8 +182,9 @@ struct fb_model {
   float* zbuf = nullptr;
   bf16* anchors = nullptr;
   size_t anchor_elems = 0;
-  int* derr = nullptr;
-  int* herr = nullptr;  // pinned
+  int* derr = nullptr;   // the kernels' error record (FB_ERR_INTS)
+  int* herr = nullptr;   // its host copy (pinned, mapped)
+  bool open = false;     // a call has begun and not ended
   // cached draft state (fb_draft_ex with keep_state): per layer the anchor slot of its
   // last computed contribution (-1: none) and that step's t; rows of nr candidates per slot
   bool state_valid = false;
@@ -294,32 +295,44 @@ void collect_timings(fb_model* m) {
   m->pending.clear();
 }
 
-// Starts an API call: clears the device error word. Work the caller queued on the
-// stream before the call is not one of our kernels either.
-fb_status begin_call(fb_model* m) {
+// The error record is clear whenever no call is open. An error: the stream has finished, the
+// record and what a kernel that gave up may have left behind (stream-K counters counted in,
+// attention flags raised) are reset.
+fb_status reset_errors(fb_model* m) {
   fb_stream_op_not_kernel();
-  CK(cudaMemsetAsync(m->derr, 0, sizeof(int), m->st));
-  return FB_OK;
-}
-// Ends an API call: waits for the stream, checks the device error word.
-fb_status end_call(fb_model* m) {
-  fb_stream_op_not_kernel();
-  CK(cudaMemcpyAsync(m->herr, m->derr, sizeof(int), cudaMemcpyDeviceToHost, m->st));
   CK(cudaStreamSynchronize(m->st));
-  collect_timings(m);
-  if (*m->herr != 0 && m->sk_ctr && m->attn_flags) {
-    // a kernel that gave up may have left stream-K counters counted in or flags raised
-    fb_stream_op_not_kernel();
+  if (*reinterpret_cast<volatile int*>(m->herr) != 0) {
+    *m->herr = 0;
+    CK(cudaMemsetAsync(m->derr, 0, sizeof(int), m->st));  // (the error word only)
     CK(cudaMemsetAsync(m->sk_ctr, 0, (size_t)m->sk_clusters * SK_CTR_PER_CLUSTER * sizeof(int),
                        m->st));
     CK(cudaMemsetAsync(m->attn_flags, 0, (size_t)m->dev_sms * ATTN_FLAGS_PER_CTA * sizeof(int),
                        m->st));
     CK(cudaStreamSynchronize(m->st));
   }
-  if (*m->herr == FB_DEVERR_WAIT_TIMEOUT)
-    return fail(FB_ECUDA, "device wait timed out (a kernel gave up after its time limit)");
-  if (*m->herr != 0) return fail(FB_ECUDA, "device error %d", *m->herr);
   return FB_OK;
+}
+// Starts an API call. Work the caller queued on the stream before the call is not one of our
+// kernels. A call that returned early (an allocation failed, say) may have left kernels
+// running that report an error later: its record is cleared first.
+fb_status begin_call(fb_model* m) {
+  fb_stream_op_not_kernel();
+  if (m->open) CKS(reset_errors(m));
+  m->open = true;
+  return FB_OK;
+}
+// Ends an API call: waits for the stream, reads the host copy of the error word.
+fb_status end_call(fb_model* m) {
+  fb_stream_op_not_kernel();
+  CK(cudaStreamSynchronize(m->st));
+  m->open = false;
+  collect_timings(m);
+  const int code = *reinterpret_cast<volatile int*>(m->herr);
+  if (code == 0) return FB_OK;
+  CKS(reset_errors(m));
+  if (code == FB_DEVERR_WAIT_TIMEOUT)
+    return fail(FB_ECUDA, "device wait timed out (a kernel gave up after its time limit)");
+  return fail(FB_ECUDA, "device error %d", code);
 }
 
 // ---- kernel wrappers with statistics ------------------------------------------------
@@ -959,8 +972,9 @@ fb_status fb_init_model(const fb_cfg* cfg, const float* weights_host, fb_model**
   if (cudaStreamCreateWithFlags(&m->own, cudaStreamDefault) != cudaSuccess)
     return bail(fail(FB_ECUDA, "cudaStreamCreate failed"));
   m->st = m->own;
-  if (cudaMallocHost(&m->herr, sizeof(int)) != cudaSuccess)
-    return bail(fail(FB_ENOMEM, "cudaMallocHost failed"));
+  if (cudaHostAlloc(&m->herr, sizeof(int), cudaHostAllocMapped) != cudaSuccess)
+    return bail(fail(FB_ENOMEM, "cudaHostAlloc failed"));
+  *m->herr = 0;
 
   // weights: matrices bf16, vectors fp32 (all per-layer tables first, contiguous)
   auto table = weight_table(c);
@@ -1069,7 +1083,7 @@ fb_status fb_init_model(const fb_cfg* cfg, const float* weights_host, fb_model**
       (s = dalloc_t(m, &m->modl, (size_t)FB_COND_STEPS * c.depth * 6 * D)) ||
       (s = dalloc_t(m, &m->hmod, FB_COND_STEPS * 2 * D)) ||
       (s = dalloc_t(m, &m->rope, (size_t)m->P * c.head_dim / 2)) ||
-      (s = dalloc_t(m, &m->zbuf, zn)) || (s = dalloc_t(m, &m->derr, 1)))
+      (s = dalloc_t(m, &m->zbuf, zn)) || (s = dalloc_t(m, &m->derr, FB_ERR_INTS)))
     return bail(s);
   m->dev_sms = m->num_sms;
   m->sk_clusters = m->num_sms / 2;
@@ -1117,8 +1131,11 @@ fb_status fb_init_model(const fb_cfg* cfg, const float* weights_host, fb_model**
         cudaSuccess)
       return bail(fail(FB_ECUDA, "rope table upload failed"));
   }
-  if (cudaMemset(m->derr, 0, sizeof(int)) != cudaSuccess)
-    return bail(fail(FB_ECUDA, "cudaMemset failed"));
+  int* hdev = nullptr;
+  if (cudaHostGetDevicePointer(reinterpret_cast<void**>(&hdev), m->herr, 0) != cudaSuccess ||
+      cudaMemset(m->derr, 0, FB_ERR_INTS * sizeof(int)) != cudaSuccess ||
+      cudaMemcpy(m->derr + 2, &hdev, sizeof(hdev), cudaMemcpyHostToDevice) != cudaSuccess)
+    return bail(fail(FB_ECUDA, "error record set-up failed"));
   *out = m;
   return FB_OK;
 }
@@ -1384,7 +1401,7 @@ namespace {
 // word. Shared by all calls on a device, so overlapping calls race.
 static __device__ __align__(256) float g_na_ws[FB_NOALLOC_MAX_PAIRS * SK_WS_FLOATS_PER_CLUSTER];
 static __device__ __align__(256) int g_na_ctr[FB_NOALLOC_MAX_PAIRS * SK_CTR_PER_CLUSTER];
-static __device__ __align__(256) int g_na_err[1];
+static __device__ __align__(256) int g_na_err[FB_ERR_INTS];  // (no host copy: err + 2 is null)
 
 struct NoAllocDev {
   bool ready = false;
@@ -1495,7 +1512,7 @@ static fb_status run_probe(size_t n, std::vector<unsigned long long>& h, Launch 
   int* err = nullptr;
   float* sink = nullptr;
   if (cudaMalloc(&cyc, n * sizeof(unsigned long long)) != cudaSuccess ||
-      cudaMalloc(&err, sizeof(int)) != cudaSuccess || cudaMalloc(&sink, sizeof(float)) != cudaSuccess) {
+      cudaMalloc(&err, FB_ERR_INTS * sizeof(int)) != cudaSuccess || cudaMalloc(&sink, sizeof(float)) != cudaSuccess) {
     cudaFree(cyc);
     cudaFree(err);
     cudaFree(sink);
@@ -1504,7 +1521,7 @@ static fb_status run_probe(size_t n, std::vector<unsigned long long>& h, Launch 
   }
   h.assign(n, 0ull);
   int herr = 0;
-  cudaError_t e = cudaMemset(err, 0, sizeof(int));
+  cudaError_t e = cudaMemset(err, 0, FB_ERR_INTS * sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(cyc, 0, n * sizeof(unsigned long long));
   fb_stream_op_not_kernel();
   if (e == cudaSuccess) e = launch(cyc, err, sink);
@@ -1601,13 +1618,13 @@ fb_status fb_probe_mma_rate(int issuers, int n, int reps, double* mac_per_clk) {
   unsigned long long* cyc = nullptr;
   int* err = nullptr;
   CK(cudaMalloc(&cyc, sizeof(unsigned long long) * sms));
-  if (cudaMalloc(&err, sizeof(int)) != cudaSuccess) {
+  if (cudaMalloc(&err, FB_ERR_INTS * sizeof(int)) != cudaSuccess) {
     cudaFree(cyc);
     return fail(FB_ENOMEM, "cudaMalloc failed");
   }
   std::vector<unsigned long long> h(sms);
   int herr = 0;
-  cudaError_t e = cudaMemset(err, 0, sizeof(int));
+  cudaError_t e = cudaMemset(err, 0, FB_ERR_INTS * sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(cyc, 0, sizeof(unsigned long long) * sms);
   fb_stream_op_not_kernel();
   if (e == cudaSuccess) e = mma_rate_probe(issuers, n, reps, sms, cyc, err, nullptr);

@@ -886,7 +886,7 @@ __device__ __forceinline__ bool wait_flag(int* flag, int* err) {
   while (*(volatile int*)flag == 0) {
     if (*(volatile int*)err != 0) return false;
     if (fb_globaltimer() - t0 > fb_wait_limit()) {
-      atomicExch(err, FB_DEVERR_WAIT_TIMEOUT);
+      fb_report(err, FB_DEVERR_WAIT_TIMEOUT);
       return false;
     }
     __nanosleep(64);

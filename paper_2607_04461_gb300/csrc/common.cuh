@@ -10,6 +10,20 @@ typedef __nv_bfloat16 bf16;
 // Error codes a kernel writes to the model's device error word.
 enum { FB_DEVERR_NONE = 0, FB_DEVERR_WAIT_TIMEOUT = 1, FB_DEVERR_BAD_ARG = 2 };
 
+// A kernel's error record (16 bytes, 8-byte aligned): the error word at err[0], zero while all
+// is well, and at err + 2 the address of a second copy in mapped host memory, or null. The
+// second copy is written only when an error is reported, so a call learns of it by reading
+// host memory after the stream has finished, without a copy per call.
+constexpr int FB_ERR_INTS = 4;
+__device__ __forceinline__ void fb_report(int* err, int code) {
+  atomicExch(err, code);
+  int* host = *reinterpret_cast<int**>(err + 2);
+  if (host) {
+    *reinterpret_cast<volatile int*>(host) = code;
+    __threadfence_system();
+  }
+}
+
 // Time limit of one device-side wait (ns); a wait that runs past it reports
 // FB_DEVERR_WAIT_TIMEOUT and makes the kernel give up. Each translation unit that waits
 // holds its own copy of the limit (no relocatable device code); fb_set_wait_limit_tu
@@ -201,7 +215,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
     if ((i & 63u) == 0) {
       if (*(volatile int*)err != 0) return false;
       if (fb_globaltimer() - t0 > fb_wait_limit()) {
-        atomicExch(err, FB_DEVERR_WAIT_TIMEOUT);
+        fb_report(err, FB_DEVERR_WAIT_TIMEOUT);
         return false;
       }
     }

@@ -562,7 +562,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
             while (*(volatile int*)ctr < n_c - 1) {
               if (*(volatile int*)err != 0) { ok2 = false; break; }
               if (fb_globaltimer() - t0 > fb_wait_limit()) {
-                atomicExch(err, FB_DEVERR_WAIT_TIMEOUT);
+                fb_report(err, FB_DEVERR_WAIT_TIMEOUT);
                 ok2 = false;
                 break;
               }
