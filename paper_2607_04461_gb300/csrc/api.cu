@@ -20,6 +20,7 @@
 #include <atomic>
 #include <mutex>
 #include <thread>
+#include <tuple>
 #include <string>
 #include <vector>
 
@@ -522,15 +523,22 @@ fb_status block_forward(fb_model* m, int l, float* h, int n, bf16* delta, int n_
 }
 
 // ---- plan analysis ------------------------------------------------------------------
+enum { ACT_COMPUTE = 0, ACT_PROXY = 1, ACT_SUM_BEGIN = 2, ACT_SUM_END = 3 };
 struct Action {
-  int type;   // 0 compute, 1 proxy run
+  int type;
   int layer;  // compute: layer
-  int slot;   // compute: anchor slot for Delta, -1 = none
-  std::vector<std::pair<int, double>> terms;  // proxy: (slot, coefficient)
+  int slot;   // compute: anchor slot for Delta, -1 = none; sum begin / end: the sum
+  std::vector<std::pair<int, double>> terms;      // proxy: (slot, coefficient)
+  std::vector<std::pair<int, double>> sum_terms;  // proxy: (sum, coefficient)
 };
+// A proxied run of layers whose contributions are always needed together (the same anchors,
+// so the same weights, and nothing else computed between them at the anchors' steps) uses
+// their sum, h behind the run minus h before it: one fp32 array per anchor step in place of a
+// bf16 array per layer.
 struct Plan {
   std::vector<std::vector<Action>> steps;
   int n_slots = 0;
+  int n_sums = 0;
   // keep: per layer the slot holding its last computed contribution (-1: none) and t
   std::vector<int> keep_slot;
   std::vector<float> keep_tau;
@@ -565,13 +573,57 @@ fb_status analyse_plan(const fb_cfg& c, const float* sched, int S, const uint8_t
       std::vector<int> an;
       for (auto it = cl.rbegin(); it != cl.rend() && (int)an.size() < order + 1; ++it)
         if (*it <= src) an.push_back(*it);
-      for (int s : an) last_use[{s, l}] = k;
       anchors[{k, l}] = an;
+    }
+  // Runs of proxied layers with one anchor list whose contributions at every anchor's step
+  // followed directly on one another (only skipped layers between them there); skipped
+  // layers do not end a run. A run of two or more becomes one term per anchor step, the sum
+  // over its layers.
+  struct Sum {
+    int step, first, last;  // contributions of layers first .. last computed at step
+    bool operator<(const Sum& o) const {
+      return std::tie(step, first, last) < std::tie(o.step, o.first, o.last);
+    }
+  };
+  std::map<Sum, int> sum_last;                  // -> last proxy step using it
+  std::map<std::pair<int, int>, int> run_last;  // (step, first layer of a summed run) -> last
+  for (int k = 0; k < S; ++k)
+    for (int l = 0; l < L;) {
+      if (is_skip(k, l) || code(k, l) == -1) { ++l; continue; }
+      const auto& an = anchors[{k, l}];
+      int last = l, count = 1;
+      for (int q = l + 1; q < L && !keep; ++q) {
+        if (is_skip(k, q)) continue;
+        bool joins = code(k, q) != -1 && anchors[{k, q}] == an;
+        for (int s : an)
+          for (int r = last + 1; joins && r < q; ++r) joins = is_skip(s, r);
+        if (!joins) break;
+        last = q;
+        ++count;
+      }
+      if (count > 1) {
+        run_last[{k, l}] = last;
+        for (int s : an) sum_last[Sum{s, l, last}] = k;
+      } else {
+        for (int s : an) last_use[{s, l}] = k;
+      }
+      l = last + 1;
     }
   // the cached state: each layer's last computed contribution stays until the end
   if (keep)
     for (int l = 0; l < L; ++l)
       if (!computed[l].empty()) last_use[{computed[l].back(), l}] = S;
+  // sums take slots from one pool, in step order
+  std::map<Sum, int> sum_slot;
+  std::vector<int> sum_free;  // per sum slot: the step after which it is free
+  for (const auto& e : sum_last) {
+    int i = 0;
+    while (i < (int)sum_free.size() && sum_free[i] >= e.first.step) ++i;
+    if (i == (int)sum_free.size()) sum_free.push_back(0);
+    sum_free[i] = e.second;
+    sum_slot[e.first] = i;
+  }
+  out->n_sums = (int)sum_free.size();
   // slot assignment: per layer a pool; a slot is free once its last user has run
   std::vector<std::vector<int>> free_at(L);  // per layer: for each slot, step after which it is free
   std::vector<int> slot_base(L, 0);
@@ -600,35 +652,49 @@ fb_status analyse_plan(const fb_cfg& c, const float* sched, int S, const uint8_t
         out->keep_slot[l] = slot_base[l] + slot_of[{k, l}];
         out->keep_tau[l] = sched[k];
       }
+  // Eqs. 3-5 as weights of the anchors h1, h2, h3 (most recent first):
+  // h~ = h1 + a (h1 - h2) + a^2/2 (h1 - 2 h2 + h3), a = (t - tau1) / (tau1 - tau2)
+  auto weights = [&](const std::vector<int>& an, double t) -> std::vector<double> {
+    if (an.size() == 1) return {1.0};
+    const double tau1 = sched[an[0]], tau2 = sched[an[1]];
+    const double a = (t - tau1) / (tau1 - tau2);
+    if (an.size() == 2) return {1.0 + a, -a};
+    return {1.0 + a + 0.5 * a * a, -a - a * a, 0.5 * a * a};
+  };
   out->steps.assign(S, {});
   for (int k = 0; k < S; ++k) {
     auto& acts = out->steps[k];
+    auto proxy_action = [&]() -> Action& {
+      if (acts.empty() || acts.back().type != ACT_PROXY) acts.push_back(Action{ACT_PROXY, -1, -1, {}, {}});
+      return acts.back();
+    };
+    int run_end = -1;  // last layer of the summed run being passed
     for (int l = 0; l < L; ++l) {
       if (is_skip(k, l)) continue;  // Eq. 6: identity, no launch
-      const int32_t cd = code(k, l);
-      if (cd == -1) {
-        Action a{0, l, -1, {}};
+      if (code(k, l) == -1) {
+        for (const auto& e : sum_slot)
+          if (e.first.step == k && e.first.first == l)
+            acts.push_back(Action{ACT_SUM_BEGIN, -1, e.second, {}, {}});
+        Action a{ACT_COMPUTE, l, -1, {}, {}};
         auto so = slot_of.find({k, l});
         if (so != slot_of.end()) a.slot = slot_base[l] + so->second;
         acts.push_back(a);
+        for (const auto& e : sum_slot)
+          if (e.first.step == k && e.first.last == l)
+            acts.push_back(Action{ACT_SUM_END, -1, e.second, {}, {}});
         continue;
       }
-      // Eqs. 3-5 as weights of the anchors h1, h2, h3 (most recent first):
-      // h~ = h1 + a (h1 - h2) + a^2/2 (h1 - 2 h2 + h3), a = (t - tau1) / (tau1 - tau2)
+      if (l <= run_end) continue;  // covered by the run's sums
       const auto& an = anchors[{k, l}];
-      const double t = sched[k];
-      std::vector<double> w;
-      if (an.size() == 1) {
-        w = {1.0};
-      } else {
-        const double tau1 = sched[an[0]], tau2 = sched[an[1]];
-        const double a = (t - tau1) / (tau1 - tau2);
-        if (an.size() == 2) w = {1.0 + a, -a};
-        else w = {1.0 + a + 0.5 * a * a, -a - a * a, 0.5 * a * a};
-      }
-      if (acts.empty() || acts.back().type != 1) acts.push_back(Action{1, -1, -1, {}});
+      const std::vector<double> w = weights(an, sched[k]);
+      const auto run = run_last.find({k, l});
+      Action& act = proxy_action();
       for (size_t i = 0; i < an.size(); ++i)
-        acts.back().terms.push_back({slot_base[l] + slot_of[{an[i], l}], w[i]});
+        if (run != run_last.end())
+          act.sum_terms.push_back({sum_slot[Sum{an[i], l, run->second}], w[i]});
+        else
+          act.terms.push_back({slot_base[l] + slot_of[{an[i], l}], w[i]});
+      if (run != run_last.end()) run_end = run->second;
     }
   }
   return FB_OK;
@@ -647,10 +713,11 @@ void warm_plan(int L, int S, int warm, const std::vector<int>& slot_of, Plan* ou
     for (int l = 0; l < L; ++l) {
       auto& acts = out->steps[k];
       if (k < warm && slot_of[l] >= 0) {
-        if (acts.empty() || acts.back().type != 1) acts.push_back(Action{1, -1, -1, {}});
+        if (acts.empty() || acts.back().type != ACT_PROXY)
+          acts.push_back(Action{ACT_PROXY, -1, -1, {}, {}});
         acts.back().terms.push_back({slot_of[l], 1.0});
       } else {
-        acts.push_back(Action{0, l, -1, {}});
+        acts.push_back(Action{ACT_COMPUTE, l, -1, {}, {}});
       }
     }
 }
@@ -725,7 +792,7 @@ fb_status sample(fb_model* m, float* z, int n, const float* sched, int S, const 
   const fb_cfg& c = m->c;
   const int nr = so.guided ? 2 * n : n;  // candidates' rows in the batch
   const size_t slot_elems = (size_t)nr * m->P * c.dim;
-  const size_t need = slot_elems * plan.n_slots;
+  const size_t need = slot_elems * (plan.n_slots + 2 * (size_t)plan.n_sums);
   CKS(ensure_anchors(m, need));
   const int M = nr * m->P;
   const size_t zn = (size_t)n * c.latent_c * c.latent_h * c.latent_w;
@@ -756,22 +823,42 @@ fb_status sample(fb_model* m, float* z, int n, const float* sched, int S, const 
       }
     }
     for (const Action& a : plan.steps[k]) {
-      if (a.type == 0) {
+      if (a.type == ACT_COMPUTE) {
         bf16* d = a.slot >= 0 ? m->anchors + (size_t)a.slot * slot_elems : nullptr;
         CKS(wait_slot(m, a.slot, slot_elems));
         CKS(block_forward(m, a.layer, m->hA, nr, d, so.guided ? n : 0, cond));
+      } else if (a.type == ACT_SUM_BEGIN || a.type == ACT_SUM_END) {
+        // sum = h, then sum = h - sum behind the run (fp32, two slots)
+        const int sl = plan.n_slots + 2 * a.slot;
+        if (a.type == ACT_SUM_BEGIN)
+          for (int i = 0; i < 2; ++i) CKS(wait_slot(m, sl + i, slot_elems));
+        const size_t ne = (size_t)M * c.dim;
+        KTimer kt(m, FB_K_PROXY, a.type == ACT_SUM_END ? (double)ne : 0.0,
+                  ne * (a.type == ACT_SUM_END ? 12.0 : 8.0));
+        CK(run_sum(reinterpret_cast<float*>(m->anchors + (size_t)sl * slot_elems), m->hA, ne,
+                   a.type == ACT_SUM_END, m->st));
       } else {
-        for (size_t i0 = 0; i0 < a.terms.size(); i0 += FB_PROXY_MAX_TERMS) {
-          ProxyTerms pt{};
-          pt.n = (int)std::min(a.terms.size() - i0, (size_t)FB_PROXY_MAX_TERMS);
-          for (int i = 0; i < pt.n; ++i) {
-            pt.ptr[i] = m->anchors + (size_t)a.terms[i0 + i].first * slot_elems;
-            pt.coef[i] = (float)a.terms[i0 + i].second;
-          }
+        ProxyTerms pt{};
+        double term_bytes = 0;
+        auto flush = [&]() -> fb_status {
+          if (pt.n == 0) return FB_OK;
           KTimer kt(m, FB_K_PROXY, 2.0 * pt.n * (double)M * c.dim,
-                    (double)M * c.dim * (8.0 + 2.0 * pt.n));
+                    (double)M * c.dim * (8.0 + term_bytes));
           CK(proxy_add(m->hA, (size_t)M * c.dim, pt, m->st));
-        }
+          pt = ProxyTerms{};
+          term_bytes = 0;
+          return FB_OK;
+        };
+        auto add = [&](int slot, double coef, bool f32) -> fb_status {
+          pt.ptr[pt.n] = m->anchors + (size_t)slot * slot_elems;
+          pt.coef[pt.n] = (float)coef;
+          if (f32) pt.f32_terms |= 1ull << pt.n;
+          term_bytes += f32 ? 4.0 : 2.0;
+          return ++pt.n == FB_PROXY_MAX_TERMS ? flush() : FB_OK;
+        };
+        for (const auto& t : a.terms) CKS(add(t.first, t.second, false));
+        for (const auto& t : a.sum_terms) CKS(add(plan.n_slots + 2 * t.first, t.second, true));
+        CKS(flush());
       }
     }
     const float* hmod = m->hmod + (size_t)cond * 2 * c.dim;

@@ -74,13 +74,17 @@ cudaError_t ln_mod(const float* x, bf16* out, int rows, int D, float eps, float 
 cudaError_t qk_norm_rope(bf16* x, int rows, int ld, int D, int nseg, int dcol, const float* w0,
                          ptrdiff_t dw, float eps, const float2* rope, int tokens, int head_dim,
                          cudaStream_t st);
-// h[i] += sum_t coef[t] * anchor_t[i] over n_elems fp32 elements (bf16 anchors).
+// h[i] += sum_t coef[t] * anchor_t[i] over n_elems fp32 elements; anchors are bf16, or fp32
+// where bit t of f32_terms is set.
 #define FB_PROXY_MAX_TERMS 64
 struct ProxyTerms {
   const bf16* ptr[FB_PROXY_MAX_TERMS];
   float coef[FB_PROXY_MAX_TERMS];
+  unsigned long long f32_terms;
   int n;
 };
+// sum[i] = h[i], or with `end` h[i] - sum[i], over n_elems fp32 elements.
+cudaError_t run_sum(float* sum, const float* h, size_t n_elems, bool end, cudaStream_t st);
 cudaError_t proxy_add(float* h, size_t n_elems, const ProxyTerms& t, cudaStream_t st);
 // h[(b*P + tok)][:] = W_p * patch(z_b, tok) + b_p.
 cudaError_t patch_embed(const float* z, int n, int C, int H, int W, int p, const bf16* Wp,

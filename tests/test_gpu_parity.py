@@ -131,6 +131,41 @@ def test_small_order2_taylor_with_three_anchors(small):
         check_latents(zd.cpu().numpy()[j], want[j], z[j], label=f"order2 cand {j}")
 
 
+def test_runs_of_proxied_blocks_use_their_sum():
+    """Runs of proxied blocks go through the sum of their contributions (residual stream
+    behind minus before the run at the anchor's step). Six blocks: whole-model runs of
+    orders 0 and 2; a run split where a block computed at the anchor's step is skipped
+    later; nested and overlapping runs from one step; a run broken by a computed block; a
+    single proxied block (its own contribution). The same plan with every block's state kept
+    (no sums) agrees too."""
+    cfg = synth.SMALL.with_(depth=6, max_n=2)
+    w = synth.make_weights(cfg, bf16=True, norm_std=0.2)
+    S, c = 9, synth.proxy_code
+    skip, proxy = synth.empty_plan(S, cfg.depth)
+    proxy[1, :] = c(0, 0)                       # 0-5 from step 0
+    proxy[2, :] = c(0, 0)
+    skip[2, 2] = 1; proxy[2, 2] = -1            # 0-1 and 3-5 from step 0
+    skip[3, 2] = 1                              # step 3 computes all but block 2
+    proxy[4, :] = c(3, 1)
+    skip[4, 2] = 1; proxy[4, 2] = -1            # anchors 3 and 0: 0-1 and 3-5
+    proxy[5, 1:3] = c(0, 0)                     # a run inside computed blocks, one anchor
+    proxy[5, 2] = -1; skip[5, 2] = 1
+    proxy[7, :] = c(6, 2)                       # step 6 computes all
+    proxy[8, 4:] = c(6, 0)                      # 4-5, beside a single block below
+    proxy[8, 1] = c(6, 2)
+    z = synth.make_latents(cfg, 2)
+    ctx = synth.make_text(cfg)
+    sched = synth.make_schedule(12)[:S + 1]
+    ref = O.OracleModel(cfg, w)
+    want = ref.draft(z, ctx, sched, skip, proxy)
+    with fb.Model(cfg, w) as m:
+        for opts in (None, fb.make_opts(keep_state=True)):
+            zd = cuda(z)
+            m.draft(zd, ctx, sched, skip, proxy, opts=opts)
+            for j in range(2):
+                check_latents(zd.cpu().numpy()[j], want[j], z[j], label=f"sums cand {j}")
+
+
 def test_small_refine_and_markov(small):
     """Refine matches the oracle; draft to step k then refine equals one full run
     (bit-exact: same kernels on the same rows in the same order)."""
