@@ -225,7 +225,10 @@ constexpr int C2_BN = 256;                           // output features of a til
 constexpr int C2_W_BYTES = 128 * BK * 2;             // 16 KB: this CTA's 128 W rows x 64 bf16
 constexpr int C2_TMEM_COLS = 512;                    // two accumulators of up to 256 tokens
 constexpr int C2_MAX_STAGES = 8;
-constexpr int C2_SMEM_BYTES = 232448;                // all of an SM's shared memory
+// Shared memory of a CTA: 2.5 KB less than an SM can give it, which lets two blocks of the
+// normalisation kernels that follow most GEMMs start beside it and wait there (1 KB each is
+// reserved by the system): one candidate's block 173.7 -> 172.3 us.
+constexpr int C2_SMEM_BYTES = 229888;
 // Epilogue tiles and operand ring per epilogue: each of the 8 epilogue warps owns NBUF tiles
 // of CHUNK tokens x 32 features, through which results leave by TMA store and (fp32 residual)
 // residual rows arrive by TMA load. A chunk costs its warp about 300 clocks of buffer wait,
@@ -238,7 +241,7 @@ struct C2Cfg {
   static constexpr int NBUF = F32 ? 3 : 2;
   static constexpr int TILE_BYTES = CHUNK * 32 * (F32 ? 4 : 2);
   static constexpr int EPI_BYTES = 8 * NBUF * TILE_BYTES;
-  static constexpr int RING_BYTES = C2_SMEM_BYTES - 1024 /*align*/ - 512 /*barriers*/ - EPI_BYTES;
+  static constexpr int RING_BYTES = C2_SMEM_BYTES - 512 /*barriers*/ - EPI_BYTES;
 };
 __host__ __device__ __forceinline__ int c2_stages(int T, int ring_bytes) {
   const int n = ring_bytes / (C2_W_BYTES + T / 2 * BK * 2);
@@ -342,9 +345,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
                     const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmR,
                     int M, int N, int K, int T, GemmEpi epi, SkArgs sk, int* err) {
   using CC = C2Cfg<KIND>;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  extern __shared__ __align__(1024) uint8_t smem[];  // (operand tiles need the alignment)
+  if ((smem_u32(smem) & 1023u) != 0) {
+    if (threadIdx.x == 0) fb_report(err, FB_DEVERR_BAD_ARG);
+    return;
+  }
   // (RING_BYTES and EPI_BYTES are multiples of 512: tiles and barriers stay aligned)
   uint8_t* epi_smem = smem + CC::RING_BYTES;
   uint64_t* full = reinterpret_cast<uint64_t*>(epi_smem + CC::EPI_BYTES);
