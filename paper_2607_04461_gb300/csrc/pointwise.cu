@@ -33,8 +33,8 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
 
 // ---------------------------------------------------------------------------------
 // ln_mod: THREADS threads per row, VPT float4 per thread (D = 4 * VPT * THREADS), ROWS
-// rows per block (ROWS > 1 only with one warp per row).
-template <int THREADS, int VPT, int ROWS = 1>
+// rows per block (ROWS > 1 only with one warp per row). EARLY: see FEW_ROWS.
+template <int THREADS, int VPT, int ROWS, bool EARLY>
 __global__ void __launch_bounds__(THREADS * ROWS) ln_mod_kernel(const float* __restrict__ x,
                                                                 bf16* __restrict__ out, int rows,
                                                                 int D, float eps, float mul_base,
@@ -48,13 +48,19 @@ __global__ void __launch_bounds__(THREADS * ROWS) ln_mod_kernel(const float* __r
   if (row >= (size_t)rows) return;
   const int tid = threadIdx.x % THREADS;
   const float* xr = x + row * D;
-  float4 v[VPT];
+  float4 v[VPT], m[EARLY ? VPT : 1], ad[EARLY ? VPT : 1];
+#pragma unroll
+  for (int i = 0; i < VPT; ++i) v[i] = *reinterpret_cast<const float4*>(xr + (i * THREADS + tid) * 4);
+  if (EARLY) {
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+      m[i] = *reinterpret_cast<const float4*>(mul + (i * THREADS + tid) * 4);
+      ad[i] = *reinterpret_cast<const float4*>(add + (i * THREADS + tid) * 4);
+    }
+  }
   float s = 0.f;
 #pragma unroll
-  for (int i = 0; i < VPT; ++i) {
-    v[i] = *reinterpret_cast<const float4*>(xr + (i * THREADS + tid) * 4);
-    s += v[i].x + v[i].y + v[i].z + v[i].w;
-  }
+  for (int i = 0; i < VPT; ++i) s += v[i].x + v[i].y + v[i].z + v[i].w;
   const float mean = block_sum<THREADS>(s, red) / D;
   float q = 0.f;
 #pragma unroll
@@ -65,13 +71,15 @@ __global__ void __launch_bounds__(THREADS * ROWS) ln_mod_kernel(const float* __r
   const float rstd = rsqrtf(block_sum<THREADS>(q, red) / D + eps);
 #pragma unroll
   for (int i = 0; i < VPT; ++i) {
-    const int col = (i * THREADS + tid) * 4;
-    const float4 m = *reinterpret_cast<const float4*>(mul + col);
-    const float4 ad = *reinterpret_cast<const float4*>(add + col);
-    const float y0 = (v[i].x - mean) * rstd * (mul_base + m.x) + ad.x;
-    const float y1 = (v[i].y - mean) * rstd * (mul_base + m.y) + ad.y;
-    const float y2 = (v[i].z - mean) * rstd * (mul_base + m.z) + ad.z;
-    const float y3 = (v[i].w - mean) * rstd * (mul_base + m.w) + ad.w;
+    const int col = (i * THREADS + tid) * 4, e = EARLY ? i : 0;
+    if (!EARLY) {
+      m[e] = *reinterpret_cast<const float4*>(mul + col);
+      ad[e] = *reinterpret_cast<const float4*>(add + col);
+    }
+    const float y0 = (v[i].x - mean) * rstd * (mul_base + m[e].x) + ad[e].x;
+    const float y1 = (v[i].y - mean) * rstd * (mul_base + m[e].y) + ad[e].y;
+    const float y2 = (v[i].z - mean) * rstd * (mul_base + m[e].z) + ad[e].z;
+    const float y3 = (v[i].w - mean) * rstd * (mul_base + m[e].w) + ad[e].w;
     uint2 u;
     u.x = pack_bf16x2(y0, y1);
     u.y = pack_bf16x2(y2, y3);
@@ -79,21 +87,16 @@ __global__ void __launch_bounds__(THREADS * ROWS) ln_mod_kernel(const float* __r
   }
 }
 
-template <int THREADS, int VPT, int ROWS = 1>
+template <int THREADS, int VPT, int ROWS = 1, bool EARLY = false>
 cudaError_t ln_mod_launch(const float* x, bf16* out, int rows, int D, float eps, float mb,
                           const float* mul, const float* add, cudaStream_t st) {
-  return launch_k(ln_mod_kernel<THREADS, VPT, ROWS>, dim3((rows + ROWS - 1) / ROWS),
+  return launch_k(ln_mod_kernel<THREADS, VPT, ROWS, EARLY>, dim3((rows + ROWS - 1) / ROWS),
                   dim3(THREADS * ROWS), 0, st, x, out, rows, D, eps, mb, mul, add);
 }
 
 // ---------------------------------------------------------------------------------
 // qk_norm_rope: THREADS threads per (row, segment), VPT chunks of 4 bf16 per thread, ROWS
 // rows per block (ROWS > 1 only with one warp per row).
-__device__ __forceinline__ void load_bf16x4(const bf16* p, float* v) {
-  uint2 u = *reinterpret_cast<const uint2*>(p);
-  float2 a = unpack_bf16x2(u.x), b = unpack_bf16x2(u.y);
-  v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-}
 __device__ __forceinline__ void store_bf16x4(bf16* p, const float* v) {
   uint2 u;
   u.x = pack_bf16x2(v[0], v[1]);
@@ -101,7 +104,7 @@ __device__ __forceinline__ void store_bf16x4(bf16* p, const float* v) {
   *reinterpret_cast<uint2*>(p) = u;
 }
 
-template <int THREADS, int VPT, int ROWS>
+template <int THREADS, int VPT, int ROWS, bool EARLY>
 __global__ void __launch_bounds__(THREADS * ROWS) qk_norm_rope_kernel(
     bf16* __restrict__ x, int rows, int ld, int D, int dcol, const float* __restrict__ w0,
     ptrdiff_t dw, float eps, const float2* __restrict__ rope, int tokens, int head_dim) {
@@ -115,41 +118,56 @@ __global__ void __launch_bounds__(THREADS * ROWS) qk_norm_rope_kernel(
   const int seg = blockIdx.y;
   const float* w = w0 + seg * dw;
   bf16* xr = x + row * ld + (size_t)seg * dcol;
+  const float2* rp = rope ? rope + (size_t)(row % tokens) * (head_dim / 2) : nullptr;
   float v[VPT][4];
+  float4 wv[EARLY ? VPT : 1], cs[EARLY ? VPT : 1];  // weights; (cos, sin) of two pairs
+  uint2 u[VPT];
+#pragma unroll
+  for (int i = 0; i < VPT; ++i) u[i] = *reinterpret_cast<const uint2*>(xr + (i * THREADS + tid) * 4);
+  // a chunk of 4 never straddles a head (head_dim % 4 == 0)
+  auto load_w = [&](int i) { return *reinterpret_cast<const float4*>(w + (i * THREADS + tid) * 4); };
+  auto load_cs = [&](int i) {
+    return *reinterpret_cast<const float4*>(rp + (((i * THREADS + tid) * 4 % head_dim) >> 1));
+  };
+  if (EARLY) {
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+      wv[i] = load_w(i);
+      if (rp) cs[i] = load_cs(i);
+    }
+  }
   float ss = 0.f;
 #pragma unroll
   for (int i = 0; i < VPT; ++i) {
-    load_bf16x4(xr + (i * THREADS + tid) * 4, v[i]);
+    const float2 a = unpack_bf16x2(u[i].x), b = unpack_bf16x2(u[i].y);
+    v[i][0] = a.x; v[i][1] = a.y; v[i][2] = b.x; v[i][3] = b.y;
 #pragma unroll
     for (int j = 0; j < 4; ++j) ss += v[i][j] * v[i][j];
   }
   const float r = rsqrtf(block_sum<THREADS>(ss, red) / D + eps);
-  const float2* rp = rope ? rope + (size_t)(row % tokens) * (head_dim / 2) : nullptr;
 #pragma unroll
   for (int i = 0; i < VPT; ++i) {
-    const int col = (i * THREADS + tid) * 4;
-    const float4 wv = *reinterpret_cast<const float4*>(w + col);
-    v[i][0] *= r * wv.x; v[i][1] *= r * wv.y; v[i][2] *= r * wv.z; v[i][3] *= r * wv.w;
+    const int e = EARLY ? i : 0;
+    if (!EARLY) wv[e] = load_w(i);
+    v[i][0] *= r * wv[e].x; v[i][1] *= r * wv[e].y; v[i][2] *= r * wv[e].z; v[i][3] *= r * wv[e].w;
     if (rp) {
-      const int d0 = col % head_dim;  // a chunk never straddles a head (head_dim % 4 == 0)
-#pragma unroll
-      for (int j = 0; j < 4; j += 2) {
-        const float2 cs = rp[(d0 + j) >> 1];
-        const float a = v[i][j], b = v[i][j + 1];
-        v[i][j] = a * cs.x - b * cs.y;
-        v[i][j + 1] = a * cs.y + b * cs.x;
-      }
+      if (!EARLY) cs[e] = load_cs(i);
+      const float a = v[i][0], b = v[i][1], c = v[i][2], d = v[i][3];
+      v[i][0] = a * cs[e].x - b * cs[e].y;
+      v[i][1] = a * cs[e].y + b * cs[e].x;
+      v[i][2] = c * cs[e].z - d * cs[e].w;
+      v[i][3] = c * cs[e].w + d * cs[e].z;
     }
-    store_bf16x4(xr + col, v[i]);
+    store_bf16x4(xr + (i * THREADS + tid) * 4, v[i]);
   }
 }
 
-template <int THREADS, int VPT, int ROWS = 1>
+template <int THREADS, int VPT, int ROWS = 1, bool EARLY = false>
 cudaError_t qkn_launch(bf16* x, int rows, int ld, int D, int nseg, int dcol, const float* w0,
                        ptrdiff_t dw, float eps, const float2* rope, int tokens, int head_dim,
                        cudaStream_t st) {
   dim3 grid((rows + ROWS - 1) / ROWS, nseg);
-  return launch_k(qk_norm_rope_kernel<THREADS, VPT, ROWS>, grid, dim3(THREADS * ROWS), 0, st, x,
+  return launch_k(qk_norm_rope_kernel<THREADS, VPT, ROWS, EARLY>, grid, dim3(THREADS * ROWS), 0, st, x,
                   rows, ld, D, dcol, w0, dw, eps, rope, tokens, head_dim);
 }
 
@@ -499,6 +517,13 @@ int grid_for(size_t work, int threads) {
 
 // ---- launchers --------------------------------------------------------------------
 
+// Row kernels (ln_mod, qk_norm_rope): with few rows a launch is one or two waves of blocks and
+// its time is latency, so the row's parameters load together with the row (EARLY, 160
+// registers) instead of after its reductions; with many rows that occupancy costs more than
+// the latency. One candidate refined for two steps: 10.73 ms, 10.51 with ln_mod EARLY, 10.42
+// with both; two candidates 16.73 -> 16.48; three 21.56 -> 21.47; eight 52.2 -> 52.5.
+constexpr int FEW_ROWS = 32 * 152;
+
 cudaError_t ln_mod(const float* x, bf16* out, int rows, int D, float eps, float mul_base,
                    const float* mul, const float* add, cudaStream_t st) {
   if (rows == 0) return cudaSuccess;
@@ -507,13 +532,19 @@ cudaError_t ln_mod(const float* x, bf16* out, int rows, int D, float eps, float 
     case 256: return ln_mod_launch<64, 1>(x, out, rows, D, eps, mul_base, mul, add, st);
     case 512: return ln_mod_launch<128, 1>(x, out, rows, D, eps, mul_base, mul, add, st);
     case 1024: return ln_mod_launch<128, 2>(x, out, rows, D, eps, mul_base, mul, add, st);
-    // one warp per row, two rows per block, reductions by shuffles only: 5.93 TB/s against
+    // one warp per row, reductions by shuffles only: 5.93 TB/s with two rows per block against
     // 5.44 with 128 threads per row on the 16-candidate probe (24960 rows)
-    case 1536: return ln_mod_launch<32, 12, 2>(x, out, rows, D, eps, mul_base, mul, add, st);
+    case 1536:
+      return rows <= FEW_ROWS
+                 ? ln_mod_launch<32, 12, 4, true>(x, out, rows, D, eps, mul_base, mul, add, st)
+                 : ln_mod_launch<32, 12, 2>(x, out, rows, D, eps, mul_base, mul, add, st);
     case 2048: return ln_mod_launch<128, 4>(x, out, rows, D, eps, mul_base, mul, add, st);
     case 3072: return ln_mod_launch<256, 3>(x, out, rows, D, eps, mul_base, mul, add, st);
     case 4096: return ln_mod_launch<256, 4>(x, out, rows, D, eps, mul_base, mul, add, st);
-    case 5120: return ln_mod_launch<256, 5>(x, out, rows, D, eps, mul_base, mul, add, st);
+    case 5120:
+      return rows <= FEW_ROWS
+                 ? ln_mod_launch<256, 5, 1, true>(x, out, rows, D, eps, mul_base, mul, add, st)
+                 : ln_mod_launch<256, 5>(x, out, rows, D, eps, mul_base, mul, add, st);
   }
   return cudaErrorInvalidValue;
 }
@@ -533,11 +564,11 @@ cudaError_t qk_norm_rope(bf16* x, int rows, int ld, int D, int nseg, int dcol, c
     // 16-candidate probe (24960 rows x 2 x 1536) 5.04 TB/s against 4.90 with two rows
     // per block and 4.60 with eight (at 49920 rows two rows per block gave 6.1 TB/s, one
     // row 5.4)
-    case 1536: return QKN(32, 12, 4);
+    case 1536: return rows <= FEW_ROWS ? QKN(32, 12, 4, true) : QKN(32, 12, 4);
     case 2048: return QKN(128, 4);
     case 3072: return QKN(256, 3);
     case 4096: return QKN(256, 4);
-    case 5120: return QKN(256, 5);
+    case 5120: return rows <= FEW_ROWS ? QKN(256, 5, 1, true) : QKN(256, 5);
   }
 #undef QKN
   return cudaErrorInvalidValue;
