@@ -308,7 +308,9 @@ const char* fb_kernel_name(int kind);
  * 2-SM cta_group::2 kernel when N % 256 == 0, else the 1-SM kernel), 1 = force the
  * CUDA-core kernel, 2 = force the 1-SM tcgen05 kernel (same shape rules), 3 = the 2-SM
  * kernel over whole tiles only (256 output features x T rows, T a multiple of 16 up to 256
- * fitted to M), 4 = the 2-SM kernel with the stream-K split: every SM pair takes an equal
+ * fitted to M; where the split below would pay, K is summed in up to 8 parts that are added
+ * in fp32, which keeps the error no larger than the split's), 4 = the 2-SM kernel with the
+ * stream-K split: every SM pair takes an equal
  * share of the (256 x 256 tile, 64-wide K block) units and tiles cut between pairs are
  * summed from fp32 partials in the model's workspace, in K order (so the result does not
  * depend on timing). impl 4 needs N % 256 == 0 and at least 4 K blocks per SM pair

@@ -338,14 +338,14 @@ fb_status end_call(fb_model* m) {
 
 // ---- kernel wrappers with statistics ------------------------------------------------
 // impl: 0 automatic, 1 CUDA-core kernel, 2 the 1-SM tcgen05 kernel, 3 the 2-SM kernel
-// over whole tiles, 4 the 2-SM kernel with the stream-K split. The model's own launches take
-// the tcgen05 kernels over whole tiles where the shape allows (3).
-fb_status run_gemm(fb_model* m, const GemmArgs& g0, int impl = 3) {
+// over whole tiles, 4 the 2-SM kernel with the stream-K split, -1 (the model's own launches)
+// as 0 with the faster of the split and whole tiles.
+fb_status run_gemm(fb_model* m, const GemmArgs& g0, int impl = -1) {
   GemmArgs g = g0;
   g.sk_ws = m->sk_ws;
   g.sk_ctr = m->sk_ctr;
   g.sk_clusters = m->sk_clusters;
-  g.sk_mode = impl == 3 ? 1 : impl == 4 ? 2 : 0;
+  g.sk_mode = impl == 3 ? 1 : impl == 4 ? 2 : impl < 0 ? 3 : 0;
   const double flops = 2.0 * g.M * (double)g.N * g.K;
   double bytes = 2.0 * ((double)g.M * g.K + (double)g.N * g.K);
   bytes += (g.kind <= EPI_GELU_BF16) ? 2.0 * g.M * g.N : 8.0 * g.M * g.N;

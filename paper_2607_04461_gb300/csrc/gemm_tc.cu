@@ -225,6 +225,13 @@ constexpr int C2_BN = 256;                           // output features of a til
 constexpr int C2_W_BYTES = 128 * BK * 2;             // 16 KB: this CTA's 128 W rows x 64 bf16
 constexpr int C2_TMEM_COLS = 512;                    // two accumulators of up to 256 tokens
 constexpr int C2_MAX_STAGES = 8;
+constexpr int C2_MAX_ACCS = 8;
+// TMEM columns from one accumulator to the next, and accumulators of the ring
+__host__ __device__ __forceinline__ int c2_acc_cols(int T) { return (T + 31) / 32 * 32; }
+__host__ __device__ __forceinline__ int c2_accs(int T) {
+  const int n = C2_TMEM_COLS / c2_acc_cols(T);
+  return n < C2_MAX_ACCS ? n : C2_MAX_ACCS;
+}
 // Shared memory of a CTA: 2.5 KB less than an SM can give it, which lets two blocks of the
 // normalisation kernels that follow most GEMMs start beside it and wait there (1 KB each is
 // reserved by the system): one candidate's block 173.7 -> 172.3 us.
@@ -256,25 +263,31 @@ constexpr int C2_THREADS = 352;
 // Data-parallel: cluster c computes whole tiles c, c + G, c + 2G, ... (G clusters).
 // Stream-K: the U = tiles x nk (tile, K-block) units, tile-major, are cut into G
 // contiguous ranges of floor(c U / G) .. floor((c + 1) U / G); a cluster walks its range
-// as segments (one tile, K-blocks kb0..kb1). A tile cut between clusters c_lo..c_hi is
-// finished by c_lo, which holds its first K blocks as the last segment of its range; the
-// others reach it as the first segment of theirs. Each of their epilogue warps writes its
-// part of an fp32 partial to the workspace and counts itself on the tile's counter; c_lo's
-// matching warp waits (bounded) for the count, adds the partials in contributor (= K)
-// order, so the sum does not depend on arrival order, runs the epilogue and resets the
-// counter to zero. With U >= G every range is non-empty, so c_hi - c_lo + 1 clusters
-// contribute.
+// as segments (one tile, K-blocks kb0..kb1). With U >= G every range is non-empty, so the
+// parts of a cut tile are held by consecutive clusters, the first as the last segment of its
+// range and the others as the first of theirs. Partials go through the workspace in fp32, are
+// counted on the tile's counter per epilogue warp, and are added in K order, so the sum does
+// not depend on arrival order. The cut tiles are finished in one of two ways:
+// * Ranges no longer than a tile (U <= G nk, at most two segments): every contributor
+//   finishes a share of the tile's tokens in proportion to its K blocks, so that all clusters
+//   finish about the same amount after equal ranges. It publishes the tokens of the others'
+//   shares, waits (bounded) for the tile's count, and adds the others' partials of its own
+//   share to its accumulators, which stay in TMEM. One finisher per tile instead was the last
+//   to leave by far: 256 x 1536 x 8960 (13 contributors a tile) 18.6 us, 60.8 with one.
+// * Longer ranges: the first contributor finishes the tile alone as the others, which reach
+//   it at the start of their ranges, have published long before. (Sharing it too would put
+//   two more trips through the workspace at the end: 1040 x 5120 x 5120 50.3 us, 59.6.)
 struct Seg {
   int tile, kb0, kb1;
 };
 struct WorkIter {
-  long long u, u1;
+  long long u, u0, u1;
   int tile, n_tiles, nk, G;
   bool sk;
   __device__ WorkIter(bool sk_, int c, int G_, int n_tiles_, int nk_)
       : tile(c), n_tiles(n_tiles_), nk(nk_), G(G_), sk(sk_) {
     const long long U = (long long)n_tiles_ * nk_;
-    u = (long long)c * U / G_;
+    u = u0 = (long long)c * U / G_;
     u1 = (long long)(c + 1) * U / G_;
   }
   __device__ bool next(Seg& g) {
@@ -299,15 +312,56 @@ struct WorkIter {
 __device__ __forceinline__ int sk_owner(long long u, long long U, int G) {
   return (int)(((u + 1) * G - 1) / U);
 }
-// Workspace slot of cluster c's segment of `tile`: 2c for the first segment of its range,
-// 2c + 1 for the last (a range meets at most two cut tiles). Per slot and CTA of the pair,
-// 8 epilogue warps x 4096 floats: the warp's chunks of CH tokens [chunk][j/4][lane 32][4].
-__device__ __forceinline__ float* sk_part(float* ws, int c, int tile, long long U, int G, int nk,
-                                          int rank, int we) {
-  const int first_tile = (int)(((long long)c * U / G) / nk);
-  const int slot = 2 * c + (tile == first_tile ? 0 : 1);
+// Workspace slot `slot` (2c: the first segment of cluster c's range, 2c + 1: the last; a range
+// meets at most two cut tiles). Per slot and CTA of the pair, 8 epilogue warps x 4096 floats:
+// the warp's chunks of CH tokens [chunk][j/4][lane 32][4].
+__device__ __forceinline__ float* sk_part(float* ws, int slot, int rank, int we) {
   return ws + ((size_t)(slot * 2 + rank) * 8 + we) * 4096;
 }
+// A cut tile: its first contributor, the number of them, whether the first holds it as the
+// last segment of a longer range, this cluster's accumulator of it
+struct CutTile {
+  int tile = -1, lo = 0, n = 0, last = 0, acc = 0;
+};
+// counts `n` on a cut tile's counter after this warp's (syncwarp'ed) writes; the old value
+__device__ __forceinline__ int sk_count(int* ctr, int n) {
+  int old;
+  asm volatile("atom.add.release.gpu.global.s32 %0, [%1], %2;"
+               : "=r"(old) : "l"(ctr), "r"(n) : "memory");
+  return old;
+}
+__device__ __forceinline__ int sk_load(const int* ctr) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
+  return v;
+}
+// waits (bounded) for `n` counted in; the high half counts who has seen it
+__device__ __forceinline__ bool sk_wait(const int* ctr, int n, int* err) {
+  const uint64_t t0 = fb_globaltimer();
+  for (int c; (c = sk_load(ctr)) < 0 || (c & 0xffff) != n;) {
+    if (*(volatile int*)err != 0) return false;
+    if (fb_globaltimer() - t0 > fb_wait_limit()) {
+      fb_report(err, FB_DEVERR_WAIT_TIMEOUT);
+      return false;
+    }
+  }
+  return true;
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void ld_shared_v4(uint32_t a, uint32_t* r) {
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+constexpr int SK_SLOTS = 8;  // 2 KB slots of an epilogue warp: 16 KB of the operand ring
 
 // ---- epilogue of the 2-SM kernel ----------------------------------------------------
 // A lane owns one output feature, so bias and gate are one register each, and a warp's
@@ -343,7 +397,7 @@ template <int KIND>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
     gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                     const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmR,
-                    int M, int N, int K, int T, GemmEpi epi, SkArgs sk, int* err) {
+                    int M, int N, int K, int T, int parts, GemmEpi epi, SkArgs sk, int* err) {
   using CC = C2Cfg<KIND>;
   extern __shared__ __align__(1024) uint8_t smem[];  // (operand tiles need the alignment)
   if ((smem_u32(smem) & 1023u) != 0) {
@@ -355,9 +409,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
   uint64_t* full = reinterpret_cast<uint64_t*>(epi_smem + CC::EPI_BYTES);
   uint64_t* empty = full + C2_MAX_STAGES;
   uint64_t* tmem_full = empty + C2_MAX_STAGES;
-  uint64_t* tmem_empty = tmem_full + 2;
-  uint64_t* pload = tmem_empty + 2;  // stream-K finisher: one partial prefetch per epilogue warp
-  uint64_t* rload = pload + 8;       // residual tile loads: NBUF per epilogue warp
+  uint64_t* tmem_empty = tmem_full + C2_MAX_ACCS;
+  uint64_t* rload = tmem_empty + C2_MAX_ACCS;  // residual tile loads: NBUF per epilogue warp
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(rload + 8 * 3);
   uint32_t* gave_up = tmem_holder + 1;  // a role of this CTA gave up a wait
 
@@ -368,6 +421,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
   const int nk = K / BK;
   const int stage_bytes = C2_W_BYTES + T / 2 * BK * 2;
   const int stages = c2_stages(T, CC::RING_BYTES);
+  const int acc_cols = c2_acc_cols(T), n_accs = c2_accs(T);
   bool failed = false;
 
   if (threadIdx.x == 0) {
@@ -376,11 +430,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    for (int a = 0; a < 2; ++a) {
+    for (int a = 0; a < n_accs; ++a) {
       mbar_init(&tmem_full[a], 1);
       mbar_init(&tmem_empty[a], 16);  // 8 epilogue warps x 2 CTAs
     }
-    for (int b = 0; b < 8; ++b) mbar_init(&pload[b], 1);
     for (int b = 0; b < 8 * 3; ++b) mbar_init(&rload[b], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     tma_prefetch_desc(&tmA);
@@ -454,26 +507,32 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
       uint32_t phase = 0;
       WorkIter wi(use_sk, cluster, n_clusters, n_tiles, nk);
       Seg sg;
-      for (int it = 0; !failed && wi.next(sg); ++it) {
-        const int acc = it & 1;
-        const uint32_t acc_phase = (it >> 1) & 1;
-        if (!mbar_wait_warp(&tmem_empty[acc], acc_phase ^ 1u, err)) { failed = true; break; }
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * 256;
-        for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
-          if (!mbar_wait_warp(&full[stage], phase, err)) { failed = true; break; }
+      const int part_len = (nk + parts - 1) / parts;
+      int acc = 0;
+      uint32_t acc_phase = 0;
+      while (!failed && wi.next(sg)) {
+        // the tile's K parts (one, with the stream-K split), each in the ring's next accumulator
+        for (int kb = sg.kb0; !failed && kb < sg.kb1;) {
+          if (!mbar_wait_warp(&tmem_empty[acc], acc_phase ^ 1u, err)) { failed = true; break; }
           tc_fence_after();
-          const uint32_t wlo = ring_lo + (uint32_t)(stage * (stage_bytes >> 4));
-          const uint32_t alo = wlo + (C2_W_BYTES >> 4);
-          if (elect_one()) {
+          const uint32_t d_tmem = tmem_base + acc * acc_cols;
+          const int first = kb, end = sg.kb1 - kb < part_len ? sg.kb1 : kb + part_len;
+          for (; kb < end; ++kb) {
+            if (!mbar_wait_warp(&full[stage], phase, err)) { failed = true; break; }
+            tc_fence_after();
+            const uint32_t wlo = ring_lo + (uint32_t)(stage * (stage_bytes >> 4));
+            const uint32_t alo = wlo + (C2_W_BYTES >> 4);
+            if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < BK / 16; ++k)
-              tc_mma_cg2_lo(d_tmem, wlo + 2 * k, alo + 2 * k, DESC_HI, idesc,
-                            (kb > sg.kb0 || k > 0) ? 1u : 0u);
-            tc_commit_mc(&empty[stage], 0x3);
-            if (kb + 1 == sg.kb1) tc_commit_mc(&tmem_full[acc], 0x3);
+              for (int k = 0; k < BK / 16; ++k)
+                tc_mma_cg2_lo(d_tmem, wlo + 2 * k, alo + 2 * k, DESC_HI, idesc,
+                              (kb > first || k > 0) ? 1u : 0u);
+              tc_commit_mc(&empty[stage], 0x3);
+              if (kb + 1 == end) tc_commit_mc(&tmem_full[acc], 0x3);
+            }
+            if (++stage == stages) { stage = 0; phase ^= 1u; }
           }
-          if (++stage == stages) { stage = 0; phase ^= 1u; }
+          if (++acc == n_accs) { acc = 0; acc_phase ^= 1u; }
         }
       }
     }
@@ -489,26 +548,66 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
     uint64_t* wload = rload + we * 3;
     uint32_t rl_phase = 0;  // bit b: parity of tile b's next load
     WorkIter wi(use_sk, cluster, n_clusters, n_tiles, nk);
-    Seg sg;
-    for (int it = 0; wi.next(sg); ++it) {
-      const int acc = it & 1;
-      const uint32_t acc_phase = (it >> 1) & 1;
+    // the cut tiles of this cluster's range (at most two: newest, older): published when
+    // their segment is done, this cluster's share of their chunks finished after the range
+    CutTile cut0, cut1, ct;
+    int fin = 0;
+    int done_old = 0, done_all = -1;  // lanes 0 and 1: their cut tile's counter when read
+    // ranges of at most two segments: the accumulators stay in TMEM to the end, and a
+    // cluster's own share is neither published nor read back
+    const bool keep = U <= (long long)n_clusters * nk;
+    auto counter = [&](const CutTile& c) { return sk.ctr + ((size_t)c.lo * 2 + rank) * 8 + we; };
+    int next_acc = 0;
+    uint32_t next_phase = 0;
+    while (true) {
+      Seg sg;
+      const bool seg = wi.next(sg);
+      if (!seg) {
+        ct = fin == 0 ? cut0 : cut1;
+        if (fin++ > 1 || ct.tile < 0) break;
+        sg.tile = ct.tile;
+      }
       const int tile = sg.tile;
-      const bool whole = sg.kb0 == 0 && sg.kb1 == nk;
-      // the cluster holding K blocks 0.. of a cut tile finishes it (see the work split)
-      const bool head = sg.kb0 == 0;
+      // the accumulator of the tile's first K part; the others follow it in the ring
+      const int acc = seg ? next_acc : ct.acc;
+      const bool is_cut = seg && (sg.kb0 != 0 || sg.kb1 != nk);
+      const bool publish = is_cut && (keep || sg.kb0 != 0);
+      const bool from_parts = !seg || (is_cut && !publish);  // a cut tile is finished now
       const int m0 = (tile / n_nt) * T;
       const int f0 = (tile % n_nt) * C2_BN + 128 * (int)rank + quarter * 32;
       const int nv = M - m0 < T ? M - m0 : T;  // valid tokens of the tile
       // this warp's chunks: i = 0, 1, ... covers tokens (half + 2 i) * CH ..
       // (none if its features lie past N, a multiple of 128)
       const int ncht = (nv + CH - 1) / CH, nch = f0 < N ? (ncht + 1 - half) / 2 : 0;
+      // the chunks that this step finishes: all of a whole tile's, a share of a cut one's
+      int i0 = 0, i1 = nch, own = -1;
+      if (is_cut || !seg) {
+        if (seg) {
+          ct.tile = tile;
+          ct.lo = sk_owner((long long)tile * nk, U, n_clusters);
+          ct.n = sk_owner((long long)(tile + 1) * nk - 1, U, n_clusters) - ct.lo + 1;
+          ct.last = (long long)ct.lo * U / n_clusters < (long long)tile * nk;
+          ct.acc = acc;
+        }
+        if (keep) {
+          // in proportion to its K blocks: every cluster's shares add up to about the same
+          const long long k0 = wi.u0 - (long long)tile * nk, k1 = wi.u1 - (long long)tile * nk;
+          i0 = k0 <= 0 ? 0 : ((int)k0 * nch + nk / 2) / nk;
+          i1 = k1 >= nk ? nch : ((int)k1 * nch + nk / 2) / nk;
+          own = cluster - ct.lo;
+        } else if (from_parts) {
+          own = 0;
+        } else {
+          i1 = 0;
+        }
+      }
       const size_t off0 = (size_t)(m0 + half * CH) * epi.ldo + f0 + lane;
-      const float bias = nch && head && epi.bias ? __ldg(epi.bias + f0 + lane) : 0.f;
-      const float gate = CC::F32 && nch && head && epi.gate ? __ldg(epi.gate + f0 + lane) : 1.f;
-      // residual chunk i into tile i % NBUF (one lane)
+      const bool work = !publish && i0 < i1;
+      const float bias = work && epi.bias ? __ldg(epi.bias + f0 + lane) : 0.f;
+      const float gate = CC::F32 && work && epi.gate ? __ldg(epi.gate + f0 + lane) : 1.f;
+      // residual chunk i into tile (i - i0) % NBUF (one lane)
       auto rload_issue = [&](int i) {
-        const int t = i % NBUF;
+        const int t = (i - i0) % NBUF;
         mbar_expect_tx(&wload[t], CC::TILE_BYTES);
         tma_load_2d(wtiles + t * CC::TILE_BYTES, &tmR, &wload[t], f0, m0 + (half + 2 * i) * CH);
       };
@@ -519,31 +618,32 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
 #pragma unroll
         for (int j = 0; j < 16; ++j) bv[j] = j < left ? __ldcg(p + (size_t)j * epi.ldo) : 0.f;
       };
-      if (head && nch > 0) {
+      if (work) {
         if (elect_one()) {
           bulk_wait_read<0>();  // the previous output tile's stores have left the tiles
-          if (has_r) rload_issue(0);
-          if (has_r && nch > 1) rload_issue(1);
+          if (has_r) rload_issue(i0);
+          if (has_r && i0 + 1 < i1) rload_issue(i0 + 1);
         }
         __syncwarp();
-        if (KIND == EPI_RESID_DELTA) load_base(0);
+        if (KIND == EPI_RESID_DELTA) load_base(i0);
       }
-      const bool ok = mbar_wait(&tmem_full[acc], acc_phase, err);
-      if (!__all_sync(0xffffffffu, ok)) { failed = true; break; }
-      tc_fence_after();
       const uint32_t taddr =
-          tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * 256 + half * CH;
-      int c_lo = 0, n_c = 1;
-      if (!whole) {
-        c_lo = sk_owner((long long)tile * nk, U, n_clusters);
-        n_c = sk_owner((long long)(tile + 1) * nk - 1, U, n_clusters) - c_lo + 1;
-        int* ctr = sk.ctr + ((size_t)c_lo * 2 + rank) * 8 + we;
-        if (!head) {
-          // a later part of a cut tile: publish this warp's partial and count in
+          tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * acc_cols + half * CH;
+      if (seg) {
+        // the last part's accumulator is complete after all others of the tile
+        int last = acc + parts - 1;
+        uint32_t last_phase = next_phase;
+        if (last >= n_accs) { last -= n_accs; last_phase ^= 1u; }
+        const bool ok = mbar_wait(&tmem_full[last], last_phase, err);
+        if (!__all_sync(0xffffffffu, ok)) { failed = true; break; }
+        tc_fence_after();
+        if (publish) {
           float4* part = reinterpret_cast<float4*>(
-                             sk_part(sk.ws, cluster, tile, U, n_clusters, nk, (int)rank, we)) + lane;
+                             sk_part(sk.ws, 2 * cluster + (sg.kb0 == 0 && ct.last), (int)rank, we)) +
+                         lane;
 #pragma unroll 1
           for (int i = 0; i < nch; ++i) {
+            if (i >= i0 && i < i1) continue;
             uint32_t r[CH];
             tmem_ld_chunk<CH>(taddr + i * 2 * CH, r);
 #pragma unroll
@@ -552,81 +652,121 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
                   __uint_as_float(r[4 * j4]), __uint_as_float(r[4 * j4 + 1]),
                   __uint_as_float(r[4 * j4 + 2]), __uint_as_float(r[4 * j4 + 3]));
           }
-          __threadfence();
           __syncwarp();
-          if (lane == 0) atomicAdd(ctr, 1);
-        } else {
-          // the finisher: wait (bounded) until the other contributors' warps have counted
-          // in. They computed their parts at the start of their ranges, or over ranges no
-          // longer than this one, so the wait is short. Every contributor gets an SM: the
-          // grid is at most the resident-cluster count, and a dependent grid starts only
-          // after all of this grid's CTAs have started.
-          bool ok2 = true;
+          if (lane == 0) sk_count(counter(ct), 1);
+          if (keep) {
+            cut1 = cut0;
+            cut0 = ct;
+          }
+        } else if (is_cut) {
+          // the other contributors computed their parts at the start of their ranges
+          bool in = true;
           if (lane == 0) {
-            const uint64_t t0 = fb_globaltimer();
-            while (*(volatile int*)ctr < n_c - 1) {
-              if (*(volatile int*)err != 0) { ok2 = false; break; }
-              if (fb_globaltimer() - t0 > fb_wait_limit()) {
-                fb_report(err, FB_DEVERR_WAIT_TIMEOUT);
-                ok2 = false;
-                break;
-              }
-              __nanosleep(64);
-            }
-            if (ok2) *(volatile int*)ctr = 0;  // every contributor is in: ready for reuse
+            in = sk_wait(counter(ct), ct.n - 1, err);
+            if (in) *(volatile int*)counter(ct) = 0;  // every contributor is in: ready for reuse
           }
-          ok2 = __shfl_sync(0xffffffffu, ok2, 0);
-          if (!ok2) { failed = true; break; }
-          __threadfence();
-          // The next contributor's partial (up to 16 KB for this warp) into this warp's
-          // part of the operand ring, idle now: a head segment is the last of the
-          // cluster's range, so every MMA that read the ring has completed and no load
-          // follows. One bulk copy instead of a round trip per chunk below, which waits
-          // for it before the CTA can leave.
-          if (nch > 0) {
-            if (lane == 0) {
-              fence_proxy_async_global();
-              mbar_expect_tx(&pload[we], nch * CH * 128);
-              bulk_load_1d(smem + we * 16384,
-                           sk_part(sk.ws, c_lo + 1, tile, U, n_clusters, nk, (int)rank, we),
-                           nch * CH * 128, &pload[we]);
-            }
-            __syncwarp();
-            const bool pok = mbar_wait(&pload[we], 0, err);
-            if (!__all_sync(0xffffffffu, pok)) { failed = true; break; }
-          }
+          if (!__all_sync(0xffffffffu, in)) { failed = true; break; }
         }
+      } else if (fin == 1) {
+        // Wait (bounded) until every contributor's warp has counted in, for both cut tiles
+        // at once (lanes 0 and 1). All publish before they wait, at the ends of ranges of
+        // one length. Every contributor gets an SM: the grid is at most the resident-cluster
+        // count, and a dependent grid starts only after all of this grid's CTAs have started.
+        bool ok = true;
+        const CutTile w = lane == 0 ? cut0 : cut1;
+        if (lane < 2 && w.tile >= 0) {
+          ok = sk_wait(counter(w), w.n, err);
+          // seen by this warp; whoever is the last to see it zeroes the counter (at the end)
+          done_all = w.n * 0x10001;
+          if (ok) done_old = sk_count(counter(w), 0x10000) + 0x10000;
+        }
+        if (!__all_sync(0xffffffffu, ok)) { failed = true; break; }
       }
-      if (head) {
-        // the chunk's sums: this cluster's accumulators, for a cut tile plus the other
-        // contributors' partials in K order (this cluster's is the first), the next one's
-        // from the copy in shared memory
+      if (!publish) {
+        // TMEM columns from the tile's first accumulator to that of K part p
+        auto acc_col = [&](int p) { return (acc + p < n_accs ? p : p - n_accs) * acc_cols; };
+        // A cut tile's partials come through this warp's 16 KB of the operand ring, idle now
+        // (every MMA that read it has completed and no load follows), in the order they are
+        // summed and SK_SLOTS - 1 of 2 KB (16 tokens) in flight: lanes copy what they read.
+        int pi = i0, ph = 0, pq = own == 0 ? 1 : 0, slot = 0;
+        const uint32_t ring = smem_u32(smem) + we * (SK_SLOTS * 2048) + lane * 16;
+        auto fetch = [&](int into) {
+          if (pi < i1) {
+            const int part_slot = 2 * (ct.lo + pq) + (pq == 0 && ct.last);
+            const float* src = sk_part(sk.ws, part_slot, (int)rank, we) +
+                               (pi * (CH * 8) + ph * 8 + lane) * 4;
+#pragma unroll
+            for (int j4 = 0; j4 < 4; ++j4) cp_async16(ring + into * 2048 + j4 * 512, src + j4 * 128);
+            if (++pq == own) ++pq;
+            if (pq >= ct.n) {
+              pq = own == 0 ? 1 : 0;
+              ph += 16;
+              if (ph == CH) { ph = 0; ++pi; }
+            }
+          }
+          cp_async_commit();
+        };
+        if (from_parts)
+          for (int i = 0; i < SK_SLOTS - 1; ++i) fetch(i);
+        // chunk i's sums: the accumulators, or a cut tile's parts in K order
         auto chunk_sums = [&](int i, float* v) {
-          uint32_t r[CH];
-          tmem_ld_chunk<CH>(taddr + i * 2 * CH, r);
+          if (!from_parts) {
+            if (parts == 1) {
+              uint32_t r[CH];
+              tmem_ld_chunk<CH>(taddr + i * 2 * CH, r);
 #pragma unroll
-          for (int j = 0; j < CH; ++j) v[j] = __uint_as_float(r[j]);
-          for (int q = 1; q < n_c; ++q) {
-            const float4* src =
-                reinterpret_cast<const float4*>(
-                    q == 1 ? reinterpret_cast<const float*>(smem + we * 16384)
-                           : sk_part(sk.ws, c_lo + q, tile, U, n_clusters, nk, (int)rank, we)) +
-                i * (CH * 8) + lane;
+              for (int j = 0; j < CH; ++j) v[j] = __uint_as_float(r[j]);
+              return;
+            }
 #pragma unroll
-            for (int j4 = 0; j4 < CH / 4; ++j4) {
-              const float4 f = q == 1 ? src[j4 * 32] : __ldcg(src + j4 * 32);
-              v[4 * j4] += f.x;
-              v[4 * j4 + 1] += f.y;
-              v[4 * j4 + 2] += f.z;
-              v[4 * j4 + 3] += f.w;
+            for (int h = 0; h < CH; h += 16) {
+#pragma unroll 1
+              for (int p = 0; p < parts; p += 2) {  // two parts' loads in flight
+                uint32_t r[16], r2[16];
+                const bool two = p + 1 < parts;
+                tmem_ld16(taddr + acc_col(p) + i * 2 * CH + h, r);
+                if (two) tmem_ld16(taddr + acc_col(p + 1) + i * 2 * CH + h, r2);
+                tmem_ld_wait();
+                reg_fence16(r);
+                reg_fence16(r2);
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                  v[h + j] = p == 0 ? __uint_as_float(r[j]) : v[h + j] + __uint_as_float(r[j]);
+                if (two) {
+#pragma unroll
+                  for (int j = 0; j < 16; ++j) v[h + j] += __uint_as_float(r2[j]);
+                }
+              }
+            }
+            return;
+          }
+#pragma unroll
+          for (int h = 0; h < CH; h += 16) {
+#pragma unroll 1
+            for (int q = 0; q < ct.n; ++q) {
+              uint32_t r[16];
+              if (q == own) {
+                tmem_ld_chunk<16>(taddr + i * 2 * CH + h, r);
+              } else {
+                cp_async_wait<SK_SLOTS - 2>();
+#pragma unroll
+                for (int j4 = 0; j4 < 4; ++j4)
+                  ld_shared_v4(ring + slot * 2048 + j4 * 512, r + 4 * j4);
+                // into the slot that was read one part ago
+                fetch((slot + SK_SLOTS - 1) % SK_SLOTS);
+                slot = (slot + 1) % SK_SLOTS;
+              }
+#pragma unroll
+              for (int j = 0; j < 16; ++j)
+                v[h + j] = q == 0 ? __uint_as_float(r[j]) : v[h + j] + __uint_as_float(r[j]);
             }
           }
         };
 #pragma unroll 1
-        for (int i = 0; i < nch; ++i) {
+        for (int i = i0; i < i1; ++i) {
           float v[CH];
           chunk_sums(i, v);
-          const int b = i % NBUF;
+          const int b = (i - i0) % NBUF;
           uint8_t* tile_b = wtiles + b * CC::TILE_BYTES;
           if (CC::F32) {
             float* tf = reinterpret_cast<float*>(tile_b) + lane;
@@ -636,8 +776,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
               if (!__all_sync(0xffffffffu, lok)) { failed = true; break; }
 #pragma unroll
               for (int j = 0; j < CH; ++j) v[j] = tf[j * 32] + gate * (v[j] + bias);
-              // tile (i + 2) % 3 was stored from one chunk ago: free for chunk i + 2
-              if (i + 2 < nch && elect_one()) {
+              // its tile was stored from one chunk ago: free for chunk i + 2
+              if (i + 2 < i1 && elect_one()) {
                 bulk_wait_read<0>();
                 rload_issue(i + 2);
               }
@@ -681,15 +821,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
               const uint32_t w = pair_pack_bf16(v[j] - bv[j], v[j + 1] - bv[j + 1], lane);
               if (j + (lane & 1) < left) *reinterpret_cast<uint32_t*>(dl + (size_t)j * epi.ldo) = w;
             }
-            if (i + 1 < nch) load_base(i + 1);
+            if (i + 1 < i1) load_base(i + 1);
           }
         }
         if (failed) break;
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(te_remote + acc * (uint32_t)sizeof(uint64_t));
+      if (seg) {
+        if (own < 0) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0)
+            for (int p = 0; p < parts; ++p) {
+              const int a = acc + p < n_accs ? acc + p : acc + p - n_accs;
+              mbar_arrive_cluster(te_remote + a * (uint32_t)sizeof(uint64_t));
+            }
+        }
+        next_acc += parts;
+        if (next_acc >= n_accs) { next_acc -= n_accs; next_phase ^= 1u; }
+      }
     }
+    if (done_old == done_all)  // the last to see this cut tile's count: ready for reuse
+      *(volatile int*)counter(lane == 0 ? cut0 : cut1) = 0;
   }
 
   // own TMA stores complete (one lane issued them all)
@@ -794,20 +946,20 @@ bool make_epi_map(CUtensorMap* map, const void* ptr, bool f32, int rows, int col
 // 29.7 at 208 (32.0 at 256), 1560 x 1536 x 1536 with residual 11.4 at 144 (14.9 at 256),
 // 1560 x 1536 x 8960 32.3 at 144 (46.2 at 256), 4096 x 1536 x 1536 18.8 at 176 (22.3 at 256),
 // 49920 x 1536 x 1536 185 at 256 (197 at 208).
-int choose_tile(int M, int N, int nk, int mc) {
-  int best_T = 256;
-  double best = 0;
+struct TileChoice {
+  int T, rounds;
+  double clocks;
+};
+TileChoice choose_tile(int M, int N, int nk, int mc) {
+  TileChoice best{0, 0, 0};
   for (int T = 256; T >= 16; T -= 16) {
     const long tiles = (long)((M + T - 1) / T) * ((N + C2_BN - 1) / C2_BN);
     const long rounds = (tiles + mc - 1) / mc;
     const double main = (double)nk * (256 + T > 313 ? 256 + T : 313), epilogue = 16.0 * T + 400;
     const double est = rounds * (main > epilogue ? main : epilogue) + epilogue;
-    if (best == 0 || est < best) {
-      best = est;
-      best_T = T;
-    }
+    if (best.T == 0 || est < best.clocks) best = {T, (int)rounds, est};
   }
-  return best_T;
+  return best;
 }
 
 template <int KIND>
@@ -837,22 +989,49 @@ cudaError_t launch2(const GemmArgs& g, int* err, int num_sms, cudaStream_t st) {
   // Stream-K automatically (sk_mode 0, the single-op calls) only for a few rounds of
   // 256 x 256 tiles (<= 4) whose last round leaves at least 24 K blocks' worth of work per
   // pair idle ((rounds - tiles / pairs) * nk >= 24), with A and W together within half of
-  // L2: the cut tiles' partials are written and summed at a cost that a short K does not
-  // repay, and the contiguous unit ranges spread each round over far-apart tiles, so
-  // operands larger than L2 are read several times. The block's own launches use whole
-  // tiles (sk_mode 1): with the tile width fitted to the rows they are faster there
-  // (1560 x 1536 x 8960 on 76 pairs: 32.3 us over 66 tiles of T = 144, 43.0 us cut).
+  // L2 (or one row of tiles, which reads W once however it is cut): the cut tiles' partials
+  // are written and summed at a cost that a short K does not repay, and the contiguous unit
+  // ranges spread each round over far-apart tiles, so operands larger than L2 are read
+  // several times.
   const long tiles256 = (long)((g.M + 255) / 256) * (g.N / C2_BN);
   const long rounds256 = (tiles256 + mc - 1) / mc;
   const double operand_bytes = 2.0 * ((double)g.M + g.N) * g.K;
   const bool sk_ok =
       g.N % C2_BN == 0 && g.sk_ws && g.sk_ctr && mc <= g.sk_clusters && tiles256 * (long long)nk >= 4LL * mc;
   const bool sk_pays = rounds256 <= 4 && (rounds256 * mc - tiles256) * nk >= 24LL * mc &&
-                       operand_bytes <= 64.0 * 1024 * 1024;
+                       (operand_bytes <= 64.0 * 1024 * 1024 || g.M <= 256);
   if (g.sk_mode == 2 && !sk_ok) return cudaErrorInvalidValue;
-  SkArgs sk{g.sk_mode == 2 || (g.sk_mode == 0 && sk_ok && sk_pays) ? 1 : 0, g.sk_ws, g.sk_ctr};
-  // stream-K keeps T = 256: fewer tiles to cut and shorter K ranges to sum
-  const int T = sk.on ? 256 : choose_tile(g.M, g.N, nk, mc);
+  const TileChoice whole = choose_tile(g.M, g.N, nk, mc);
+  // stream-K keeps T = 256 (all rows of fewer): fewer tiles to cut, shorter K ranges to sum
+  const int sk_T = g.M < 256 ? (g.M + 15) / 16 * 16 : 256;
+  // Whole tiles where the split would pay sum K in parts with accumulators of their own,
+  // whose ranges are 0.9 of a pair's under the split or shorter, as far as TMEM goes: the
+  // tensor core's fp32 sums lose 7e-8 of the result per K block, and the shorter ranges keep
+  // the error no larger than the split's (1560 x 1536 x 8960: 3.2e-6 in 3 parts, 4.6e-6
+  // split, 1.0e-5 in one; 34.5 us in 3 parts, 32.7 in one).
+  int parts = 1;
+  if (sk_ok && sk_pays) {
+    parts = (int)(mc / (0.9 * tiles256)) + 1;
+    if (parts < 2) parts = 2;
+    if (parts > c2_accs(whole.T)) parts = c2_accs(whole.T);
+    const int len = (nk + parts - 1) / parts;  // K blocks of a part; the kernel takes as many
+    parts = (nk + len - 1) / len;
+  }
+  bool use_sk = g.sk_mode == 2 || (g.sk_mode != 1 && sk_ok && sk_pays);
+  // The model's own launches (sk_mode 3) take the faster of the two: a range of the split in
+  // the clocks of choose_tile, then publishing, waiting for and summing the parts; a further
+  // accumulator about 1500. Measured (us, split / whole tiles): rows x 1536 x 8960, 32 rows
+  // 12.4 / 29.8, 256 18.6 / 31.0, 640 24.5 / 31.5, 1040 31.4 / 31.6, 1560 38.6 / 34.5; rows x
+  // 5120 x 5120, 100 rows 15.6 / 20.6, 256 22.2 / 22.4, 400 28.2 / 23.1. More than one round
+  // of tiles: whole (1040 x 5120 x 5120 50.3 / 44.7).
+  if (g.sk_mode == 3 && use_sk) {
+    const double range = (double)((tiles256 * nk + mc - 1) / mc);
+    use_sk = rounds256 == 1 && range * (256 + sk_T > 313 ? 256 + sk_T : 313) + 51 * sk_T + 9500 <
+                                   whole.clocks + 1500 * (parts - 1);
+  }
+  if (use_sk) parts = 1;
+  const SkArgs sk{use_sk ? 1 : 0, g.sk_ws, g.sk_ctr};
+  const int T = use_sk ? sk_T : whole.T;
   const int tiles = (g.M + T - 1) / T * ((g.N + C2_BN - 1) / C2_BN);
   CUtensorMap ma, mw, mo, mr{};  // mr: unused without a residual
   if (!make_map(&ma, g.A, g.M, g.K, g.lda, T / 2) || !make_map(&mw, g.W, g.N, g.K, g.ldw, 128) ||
@@ -862,7 +1041,7 @@ cudaError_t launch2(const GemmArgs& g, int* err, int num_sms, cudaStream_t st) {
     return cudaErrorInvalidValue;
   const int clusters = sk.on ? mc : (tiles < mc ? tiles : mc);
   return launch_k(gemm_tc2_kernel<KIND>, dim3(2 * clusters), dim3(C2_THREADS), C2_SMEM_BYTES, st,
-                  ma, mw, mo, mr, g.M, g.N, g.K, T, g.epi, sk, err);
+                  ma, mw, mo, mr, g.M, g.N, g.K, T, parts, g.epi, sk, err);
 }
 
 cudaError_t dispatch2(const GemmArgs& g, int* err, int num_sms, cudaStream_t st) {

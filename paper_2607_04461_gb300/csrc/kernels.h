@@ -18,7 +18,8 @@ struct GemmArgs {
   GemmEpi epi;
   // Stream-K workspace of the 2-SM kernel (null: data-parallel tiles only): room for
   // sk_clusters clusters (sk_clusters * 131072 floats) and sk_clusters * 16 counters that
-  // start at zero and are left at zero. sk_mode: 0 automatic, 1 never, 2 always.
+  // start at zero and are left at zero. sk_mode: 0 automatic, 1 never, 2 always,
+  // 3 the faster of the split and whole tiles.
   float* sk_ws;
   int* sk_ctr;
   int sk_clusters;

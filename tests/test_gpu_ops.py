@@ -122,6 +122,36 @@ def test_gemm_stream_k_is_deterministic_and_matches_whole_tiles(model, M, N, K):
     assert rel_max(f64(outs[0]), f64(outs[2])) <= 1e-5
 
 
+@pytest.mark.parametrize("M,N,K,impl,blocks", [
+    (1, 1536, 8960, 4, 12),      # 11.05 K blocks per pair, 13 contributors, one token
+    (33, 1536, 8960, 0, 12),     # chunks that only some contributors finish
+    (257, 1536, 8960, 4, 24),    # a second row of tiles with one token
+    (640, 1536, 8960, 0, 34),    # ranges of two segments
+    (2304, 1536, 8960, 4, 100),  # 54 tiles: up to three contributors
+    (1040, 5120, 5120, 4, 80),   # ranges of three segments: one finisher
+    (16, 1536, 8960, 3, 18),     # whole tiles of 16 tokens, eight parts
+    (1560, 1536, 8960, 3, 47),   # three parts of 47, 47 and 46 K blocks
+    (1040, 5120, 5120, 3, 40),   # two rounds: two parts in a ring of three accumulators
+    (1400, 5120, 5120, 3, 40),   # two rounds: two parts in a ring of two
+])
+@pytest.mark.parametrize("epi", [0, 2])
+def test_gemm_k_ranges(model, M, N, K, impl, blocks, epi):
+    """Sums over K ranges joined in fp32, cut between SM pairs or kept in accumulators of
+    their own: the error is that of the longest range. A 64-wide K block is four MMAs, each
+    of which may truncate the running sum by one fp32 unit (1.2e-7 of it at most)."""
+    A = randn((M, K), 71)
+    W = randn((N, K), 72, scale=K ** -0.5)
+    out = torch.empty((M, N), dtype=torch.float32 if epi else torch.bfloat16, device="cuda")
+    for _ in range(2):  # (the second call finds the counters as the first left them)
+        out.fill_(float("nan"))
+        fb.fb_op_gemm(model.handle, M, N, K, A, W, None, epi, out, None, None, None, None, impl)
+    torch.cuda.synchronize()
+    want = A.double() @ W.double().T
+    err = ((out.double() - want).norm() / want.norm()).item()
+    # bf16 results: half a unit of 2^-8 at most
+    assert err <= (1.2e-7 * blocks if epi else 2.0 ** -9)
+
+
 @pytest.mark.parametrize("M,N,K,twin", [
     (1560, 1536, 8960, 4),   # 42 tiles, 140 K blocks: stream-K
     (640, 1536, 8960, 4),    # 18 tiles, 140 K blocks: stream-K
