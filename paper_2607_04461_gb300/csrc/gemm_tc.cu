@@ -940,23 +940,27 @@ bool make_epi_map(CUtensorMap* map, const void* ptr, bool f32, int rows, int col
 // bytes per SM, arrive at about 64 bytes per clock and SM, 256 + T clocks, which is also the
 // MMAs' time (2 T) at T = 256 and more than it below; 313 clocks is the loading and issuing
 // threads' time per K block (163 ns at 64 to 160 tokens x 1536 x 8960). As many rounds as the
-// fullest pair has tiles, each its mainloop or, if that is longer, the epilogue (about 16
-// clocks per token) that runs beside it, and the last round's epilogue. Measured (us, chosen
-// T first): 1560 x 4608 x 1536 18.3 at T = 208 (20.4 at 256, 19.8 at 160), 1560 x 8960 x 1536
-// 29.7 at 208 (32.0 at 256), 1560 x 1536 x 1536 with residual 11.4 at 144 (14.9 at 256),
-// 1560 x 1536 x 8960 32.3 at 144 (46.2 at 256), 4096 x 1536 x 1536 18.8 at 176 (22.3 at 256),
-// 49920 x 1536 x 1536 185 at 256 (197 at 208).
+// fullest pair has tiles: the first one's mainloop, for each further one its mainloop or, if
+// that is longer, the epilogue that runs beside it (a fixed part per tile, 12 clocks per
+// token, 30 with fp32 residual and output), and the last round's epilogue alone (16 or 28 per
+// token). Measured (us, chosen T first): 1560 x 4608 x 1536 18.3 at T = 208 (20.4 at 256,
+// 19.8 at 160), 1560 x 8960 x 1536 29.7 at 208 (32.0 at 256), 1560 x 1536 x 1536 with
+// residual 11.4 at 144 (14.9 at 256), 4096 x 1536 x 1536 18.8 at 176 (22.3 at 256), 49920 x
+// 1536 x 1536 185 at 256 (197 at 208); bound by the epilogue: 3259 x 768 x 256 6.4 at 160
+// (9.2 at 48), 9965 x 768 x 256 9.9 at 224 (14.4 at 80, 10.3 at 256).
 struct TileChoice {
   int T, rounds;
   double clocks;
 };
-TileChoice choose_tile(int M, int N, int nk, int mc) {
+TileChoice choose_tile(int M, int N, int nk, int mc, bool f32) {
   TileChoice best{0, 0, 0};
   for (int T = 256; T >= 16; T -= 16) {
     const long tiles = (long)((M + T - 1) / T) * ((N + C2_BN - 1) / C2_BN);
     const long rounds = (tiles + mc - 1) / mc;
-    const double main = (double)nk * (256 + T > 313 ? 256 + T : 313), epilogue = 16.0 * T + 400;
-    const double est = rounds * (main > epilogue ? main : epilogue) + epilogue;
+    const double main = (double)nk * (256 + T > 313 ? 256 + T : 313);
+    const double epilogue = f32 ? 3300 + 30.0 * T : 2900 + 12.0 * T;
+    const double last = (f32 ? 28.0 : 16.0) * T + 400;
+    const double est = main + (rounds - 1) * (main > epilogue ? main : epilogue) + last;
     if (best.T == 0 || est < best.clocks) best = {T, (int)rounds, est};
   }
   return best;
@@ -1001,7 +1005,7 @@ cudaError_t launch2(const GemmArgs& g, int* err, int num_sms, cudaStream_t st) {
   const bool sk_pays = rounds256 <= 4 && (rounds256 * mc - tiles256) * nk >= 24LL * mc &&
                        (operand_bytes <= 64.0 * 1024 * 1024 || g.M <= 256);
   if (g.sk_mode == 2 && !sk_ok) return cudaErrorInvalidValue;
-  const TileChoice whole = choose_tile(g.M, g.N, nk, mc);
+  const TileChoice whole = choose_tile(g.M, g.N, nk, mc, C2Cfg<KIND>::F32);
   // stream-K keeps T = 256 (all rows of fewer): fewer tiles to cut, shorter K ranges to sum
   const int sk_T = g.M < 256 ? (g.M + 15) / 16 * 16 : 256;
   // Whole tiles where the split would pay sum K in parts with accumulators of their own,
@@ -1019,15 +1023,16 @@ cudaError_t launch2(const GemmArgs& g, int* err, int num_sms, cudaStream_t st) {
   }
   bool use_sk = g.sk_mode == 2 || (g.sk_mode != 1 && sk_ok && sk_pays);
   // The model's own launches (sk_mode 3) take the faster of the two: a range of the split in
-  // the clocks of choose_tile, then publishing, waiting for and summing the parts; a further
+  // the clocks of choose_tile and 15 % (full-width tiles stay short of the rate), then publishing, waiting for and summing the parts; a further
   // accumulator about 1500. Measured (us, split / whole tiles): rows x 1536 x 8960, 32 rows
   // 12.4 / 29.8, 256 18.6 / 31.0, 640 24.5 / 31.5, 1040 31.4 / 31.6, 1560 38.6 / 34.5; rows x
   // 5120 x 5120, 100 rows 15.6 / 20.6, 256 22.2 / 22.4, 400 28.2 / 23.1. More than one round
   // of tiles: whole (1040 x 5120 x 5120 50.3 / 44.7).
   if (g.sk_mode == 3 && use_sk) {
     const double range = (double)((tiles256 * nk + mc - 1) / mc);
-    use_sk = rounds256 == 1 && range * (256 + sk_T > 313 ? 256 + sk_T : 313) + 51 * sk_T + 9500 <
-                                   whole.clocks + 1500 * (parts - 1);
+    use_sk = rounds256 == 1 &&
+             1.15 * range * (256 + sk_T > 313 ? 256 + sk_T : 313) + 51 * sk_T + 9500 <
+                 whole.clocks + 1500 * (parts - 1);
   }
   if (use_sk) parts = 1;
   const SkArgs sk{use_sk ? 1 : 0, g.sk_ws, g.sk_ctr};
@@ -1069,12 +1074,15 @@ cudaError_t gemm_tc_set_wait_limit(unsigned long long ns) { return fb_set_wait_l
 cudaError_t gemm_tc(const GemmArgs& g, int* err, int num_sms, cudaStream_t st, bool force_1sm) {
   if (!gemm_tc_supported(g)) return cudaErrorInvalidValue;
   // 2-SM tiles of 256 features x T tokens; where N leaves half of the last feature tile empty
-  // (N % 256 == 128) only past one 128-row tile, where T spreads the rows over more SMs than
-  // the 1-SM kernel's 128 x BN tiles (BN = 256 when that still gives every SM a tile): the
-  // head's 1560 x 128 x 1536 took 13 SMs and 13.3 us there.
+  // (N % 256 == 128) only from K = 1536 and past one 128-row tile, where T spreads the rows
+  // over more SMs than the 1-SM kernel's 128 x BN tiles (BN = 256 when that still gives every
+  // SM a tile), and with every tile half empty (N = 128) up to 2048 rows. Measured (us, 1-SM /
+  // 2-SM): N = 128, 1560 rows: K = 512 5.3 / 6.0, K = 1536 (the head) 9.1 / 8.7, K = 5120 22.3
+  // / 17.9; 12480 rows, K = 1536: 9.9 / 10.8, N = 384 17.4 / 16.2.
   const bool half_tile = g.N % C2_BN != 0;
-  if (!force_1sm && num_sms >= 2 && (!half_tile || (g.M > BM && g.sk_mode != 2)))
-    return dispatch2(g, err, num_sms, st);
+  const bool half_ok =
+      g.K >= 1536 && g.M > BM && (g.N > 128 || g.M <= 16 * BM) && g.sk_mode != 2;
+  if (!force_1sm && num_sms >= 2 && (!half_tile || half_ok)) return dispatch2(g, err, num_sms, st);
   if (g.sk_mode == 2) return cudaErrorInvalidValue;  // stream-K exists in the 2-SM kernel only
   const int mt = (g.M + BM - 1) / BM;
   if (g.N % 256 == 0 && mt * (g.N / 256) >= num_sms) return dispatch_kind<256>(g, err, num_sms, st);

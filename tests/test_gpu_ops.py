@@ -66,6 +66,8 @@ def test_gemm_tc_2sm_ragged_rows(model, M):
     (1560, 1536, 128),   # 11 token tiles, the last one partial
     (1560, 4608, 640),   # two rounds
     (2049, 512, 1536),   # one row in the last tile
+    (700, 128, 1536),    # every tile half empty
+    (3000, 384, 1600),   # the last feature tile half empty
 ])
 @pytest.mark.parametrize("epi", [0, 1, 2, 3])
 def test_gemm_2sm_tile_widths(model, M, N, K, epi):
