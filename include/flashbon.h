@@ -305,15 +305,15 @@ const char* fb_kernel_name(int kind);
  *   3: as 2, and also delta bf16 = out - base[M][N] (fp32), base may equal out
  * A, W bf16 row-major, leading dimensions K; out / resid / base / delta leading
  * dimension N. impl: 0 = automatic (tcgen05 when N % 128 == 0 and K % 64 == 0: the
- * 2-SM cta_group::2 kernel when N % 256 == 0, else the 1-SM kernel), 1 = force the
- * CUDA-core kernel, 2 = force the 1-SM tcgen05 kernel (same shape rules), 3 = the 2-SM
- * kernel over whole tiles only (256 output features x T rows, T a multiple of 16 up to 256
- * fitted to M; where the split below would pay, K is summed in up to 8 parts that are added
- * in fp32, which keeps the error no larger than the split's), 4 = the 2-SM kernel with the
- * stream-K split: every SM pair takes an equal
- * share of the (256 x 256 tile, 64-wide K block) units and tiles cut between pairs are
- * summed from fp32 partials in the model's workspace, in K order (so the result does not
- * depend on timing). impl 4 needs N % 256 == 0 and at least 4 K blocks per SM pair
+ * 2-SM cta_group::2 kernel when N % 256 == 0 or K is long enough to pay for a half-empty
+ * tile, else the 1-SM kernel), 1 = force the CUDA-core kernel, 2 = force the 1-SM tcgen05
+ * kernel (same shape rules), 3 = the 2-SM kernel over whole tiles only (256 output features
+ * x T rows, T a multiple of 16 up to 256 fitted to M; where the split below would pay, K is
+ * summed in up to 8 parts that are added in fp32, which keeps the error no larger than the
+ * split's), 4 = the 2-SM kernel with the stream-K split: every SM pair takes an equal share
+ * of the (256 x 256 tile, 64-wide K block) units and tiles cut between pairs are summed from
+ * fp32 partials in the model's workspace, in K order (so the result does not depend on
+ * timing). impl 4 needs N % 256 == 0 and at least 4 K blocks per SM pair
  * (ceil(M / 256) * N / 256 * K / 64 >= 4 * pairs), else FB_ECUDA; impl 0 takes the
  * stream-K split only when the 256 x 256 tiles fill at most 4 rounds of the resident SM
  * pairs and leave at least 24 K blocks per pair idle in the last (e.g. 1560 x 1536 x 8960),
@@ -332,7 +332,8 @@ fb_status fb_op_gemm(fb_model* m, int M, int N, int K, const void* A, const void
  * mma.sync kernel, 2 / 3 = force the tcgen05 kernel with 128- / 256-query CTAs, 4 = force
  * the persistent 256-query kernel (at most one CTA per SM looping over the (batch, head,
  * query-tile pair) items; the automatic choice unless the 256-query form saves no
- * waves: both forms fit one wave, or Lq <= 128)
+ * waves: both forms fit one wave, or Lq <= 128; where whole items leave SMs idle it cuts
+ * them by key range into equal shares and adds the parts in fp32 in a fixed order)
  * (2-4: head_dim 128 only, else FB_EINVAL). */
 fb_status fb_op_attention(fb_model* m, const void* Q, int ldq, const void* K, int ldk,
                           const void* V, int ldv, void* O, int ldo, int batch, int Lq,
