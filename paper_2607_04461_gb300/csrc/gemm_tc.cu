@@ -946,8 +946,8 @@ bool make_epi_map(CUtensorMap* map, const void* ptr, bool f32, int rows, int col
 // token). Measured (us, chosen T first): 1560 x 4608 x 1536 18.3 at T = 208 (20.4 at 256,
 // 19.8 at 160), 1560 x 8960 x 1536 29.7 at 208 (32.0 at 256), 1560 x 1536 x 1536 with
 // residual 11.4 at 144 (14.9 at 256), 4096 x 1536 x 1536 18.8 at 176 (22.3 at 256), 49920 x
-// 1536 x 1536 185 at 256 (197 at 208); bound by the epilogue: 3259 x 768 x 256 6.4 at 160
-// (9.2 at 48), 9965 x 768 x 256 9.9 at 224 (14.4 at 80, 10.3 at 256).
+// 1536 x 1536 185 at 256 (197 at 208). Bound by the epilogue: 3259 x 768 x 256 9.2 at 48, 7.3
+// at 128, 6.4 at 160; 9965 x 768 x 256 14.4 at 80, 9.9 at 224, 10.3 at 256.
 struct TileChoice {
   int T, rounds;
   double clocks;
