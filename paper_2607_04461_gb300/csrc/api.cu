@@ -177,8 +177,7 @@ struct fb_model {
   size_t noise_elems = 0;
   bool text_ready = false;
   // conditioning, FB_COND_STEPS rows each (tembs: SiLU(temb))
-  float *emb = nullptr, *th1 = nullptr, *temb = nullptr, *tembs = nullptr, *mod = nullptr, *modl = nullptr,
-        *hmod = nullptr;
+  float *emb = nullptr, *th1 = nullptr, *tembs = nullptr, *modl = nullptr, *hmod = nullptr;
   float2* rope = nullptr;
   float* zbuf = nullptr;
   bf16* anchors = nullptr;
@@ -439,7 +438,7 @@ fb_status encode_text(fb_model* m, const float* ctx, bf16* kv_dst) {
 
 // ---- conditioning: temb, mod, per-layer modulation, head modulation -------------------
 // for the ns <= FB_COND_STEPS timesteps t[0 .. ns - 1] (one row each of the buffers). The
-// sampler takes a chunk of steps at a time: five launches per chunk instead of per step, the
+// sampler takes a chunk of steps at a time: four launches per chunk instead of per step, the
 // weights (28 MB of modulation at dim 1536) read once per chunk.
 fb_status time_embed(fb_model* m, const float* t, int ns) {
   const fb_cfg& c = m->c;
@@ -447,13 +446,14 @@ fb_status time_embed(fb_model* m, const float* t, int ns) {
   CondSteps ts{};
   for (int i = 0; i < ns; ++i) ts.t[i] = t[i];
   KTimer k(m, FB_K_SMALL, 2.0 * ns * D * (c.freq_dim + D + 6.0 * D),
-           2.0 * D * (c.freq_dim + D + 6.0 * D), 5);
+           2.0 * D * (c.freq_dim + D + 6.0 * D), 4);
   CK(timestep_sincos(ts, ns, c.freq_dim, m->emb, m->st));
-  CK(gemv(m->time_w1, m->time_b1, m->emb, nullptr, m->th1, D, c.freq_dim, ns, m->st));
-  CK(gemv(m->time_w2, m->time_b2, m->th1, m->temb, m->tembs, D, D, ns, m->st));
-  CK(gemv(m->mod_w, m->mod_b, m->tembs, m->mod, nullptr, 6 * D, D, ns, m->st));
-  CK(mod_prepare(m->mod, m->tables, c.depth, D, ns, m->modl, m->head_table, m->temb, m->hmod,
-                 m->st));
+  CK(gemv(m->time_w1, m->time_b1, m->emb, {m->th1}, D, c.freq_dim, ns, m->st));
+  // the head's modulation and every layer's: their tables added where the vector is formed
+  CK(gemv(m->time_w2, m->time_b2, m->th1, {m->tembs, m->head_table, m->hmod, 2}, D, D, ns,
+          m->st));
+  CK(gemv(m->mod_w, m->mod_b, m->tembs, {nullptr, m->tables, m->modl, c.depth}, 6 * D, D,
+          ns, m->st));
   return FB_OK;
 }
 
@@ -1164,9 +1164,7 @@ fb_status fb_init_model(const fb_cfg* cfg, const float* weights_host, fb_model**
       (s = dalloc_t(m, &m->kvctx, (size_t)c.depth * c.text_len * 2 * D)) ||
       (s = dalloc_t(m, &m->emb, (size_t)FB_COND_STEPS * c.freq_dim)) ||
       (s = dalloc_t(m, &m->th1, FB_COND_STEPS * D)) ||
-      (s = dalloc_t(m, &m->temb, FB_COND_STEPS * D)) ||
       (s = dalloc_t(m, &m->tembs, FB_COND_STEPS * D)) ||
-      (s = dalloc_t(m, &m->mod, FB_COND_STEPS * 6 * D)) ||
       (s = dalloc_t(m, &m->modl, (size_t)FB_COND_STEPS * c.depth * 6 * D)) ||
       (s = dalloc_t(m, &m->hmod, FB_COND_STEPS * 2 * D)) ||
       (s = dalloc_t(m, &m->rope, (size_t)m->P * c.head_dim / 2)) ||

@@ -118,14 +118,18 @@ cudaError_t euler_step(const float* v, int ldv, int n, int C, int H, int W, int 
 struct CondSteps {
   float t[FB_COND_STEPS];
 };
-// y[s][o] = b[o] + sum_k W[o][k] x[s][k] and ysilu[s][o] = SiLU of it (either may be null).
-cudaError_t gemv(const bf16* W, const float* b, const float* x, float* y, float* ysilu, int O,
-                 int K, int ns, cudaStream_t st);
+// y[s][o] = b[o] + sum_k W[o][k] x[s][k]: ysilu[s][o] = SiLU of it (unless null), and
+// rows[s][l][:] = y_s + tables[l][:] for each of n_tables tables of O floats.
+struct GemvOut {
+  float* ysilu;
+  const float* tables;
+  float* rows;
+  int n_tables;
+};
+cudaError_t gemv(const bf16* W, const float* b, const float* x, const GemvOut& out, int O, int K,
+                 int ns, cudaStream_t st);
 // emb[s] = [cos(1000 t_s f_k), sin(1000 t_s f_k)], f_k = 10000^(-k/half).
 cudaError_t timestep_sincos(const CondSteps& ts, int ns, int dim, float* emb, cudaStream_t st);
-// modl[s][l][j][:] = mod[s][j][:] + table_l[j][:] (6 rows, all layers); head[s][j] = htab[j] + temb[s].
-cudaError_t mod_prepare(const float* mod, const float* tables, int L, int D, int ns, float* modl,
-                        const float* htab, const float* temb, float* head_mod, cudaStream_t st);
 cudaError_t f32_to_bf16(const float* x, bf16* y, size_t n, cudaStream_t st);
 
 // ---- measurement probe ----------------------------------------------------------------
