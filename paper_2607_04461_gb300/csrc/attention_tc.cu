@@ -23,6 +23,7 @@
 // All waits are bounded; on a timeout the kernel records the error and drains.
 #include <cudaTypedefs.h>
 
+#include <cfloat>
 #include <cmath>
 
 #include "kernels.h"
@@ -74,7 +75,9 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return r;
 }
 // maximum of a 128-score row: eight independent chains of three-input maxima, so the
-// reduction is a few dependent steps instead of 128
+// reduction is a few dependent steps instead of 128. At least the lowest finite value: a row
+// whose scores are all -inf (masked keys) then has exponentials of exp2(-inf) = 0 and joins
+// other tiles and parts with a factor of 0, where a maximum of -inf would give -inf + inf.
 __device__ __forceinline__ float rowmax128(const float* s) {
   float m[8];
 #pragma unroll
@@ -86,7 +89,7 @@ __device__ __forceinline__ float rowmax128(const float* s) {
   }
 #pragma unroll
   for (int k = 0; k < 8; ++k) m[k] = fmaxf(m[k], s[120 + k]);
-  return fmaxf(fmax3(m[0], m[1], m[2]), fmax3(fmax3(m[3], m[4], m[5]), m[6], m[7]));
+  return fmax3(fmax3(m[0], m[1], m[2]), fmax3(fmax3(m[3], m[4], m[5]), m[6], m[7]), -FLT_MAX);
 }
 
 __device__ __forceinline__ float ex2(float x) {
@@ -1277,7 +1280,10 @@ __global__ void __launch_bounds__(THREADS2, 1)
             if (i >= valid) s[i] = -INFINITY;
         }
         const float mx = rowmax128(s) * p.scale_log2;
-        if (m_used == -INFINITY) {  // the segment's first tile
+        // The segment's first tile: every lane's m_used is still -inf, which no maximum is. The
+        // vote keeps the branch, which is warp-wide (the rescale), uniform. (Comparing the tile's
+        // number instead takes 2 % longer: 8 x 1560 queries x 12 heads 103.6 -> 105.9 us.)
+        if (__all_sync(0xffffffffu, m_used == -INFINITY)) {
           m_used = mx;
         } else if (__any_sync(0xffffffffu, mx > m_used + 8.f)) {
           const float m_new = fmaxf(m_used, mx);

@@ -379,6 +379,54 @@ def test_attention_key_split(model, batch, Lq, Lkv, heads, shared):
             assert np.abs(got - want).mean() <= 2e-3
 
 
+@pytest.mark.parametrize("batch,Lq,Lkv,heads,impl", [
+    (3, 900, 1300, 14, 0),   # every item cut into two parts
+    (1, 2500, 4100, 6, 4),   # about three parts an item
+    (12, 300, 700, 12, 4),   # whole items, one or two query tiles
+    (2, 300, 700, 2, 2),     # 128-query CTAs
+    (2, 300, 700, 2, 3),     # 256-query CTAs, one item each
+])
+def test_attention_masked_keys(model, batch, Lq, Lkv, heads, impl):
+    """Scores of minus infinity through bias channels of q and k: the later half of the keys
+    for every row (whole parts of cut items), the first 300 keys (two tiles and a piece) for
+    one row per warp, and every key for another. The oracle sees the unmasked keys only; a row
+    without any has no value (NaN), and its neighbours in the warp keep theirs."""
+    D, lead, end = heads * 128, 300, Lkv // 2
+    q, k, v = (randn((batch * n, D), 100 + i) for i, n in enumerate((Lq, Lkv, Lkv)))
+    q4, k4 = q.view(batch, Lq, heads, 128), k.view(batch, Lkv, heads, 128)
+    row = torch.arange(Lq, device="cuda")
+    late, none = row % 32 == 9, row % 32 == 5
+    q4[..., :3] = 0
+    k4[..., :3] = 0
+    q4[..., 0] = 1.0                      # keys end .. : score -inf for every row
+    k4[:, end:, :, 0] = -float("inf")
+    q4[:, none, :, 1] = -float("inf")     # rows with no key left
+    k4[..., 1] = 1.0
+    q4[:, late, :, 2] = 2.0 ** 120        # 2^120 * -2^120 overflows to -inf
+    k4[:, :lead, :, 2] = -(2.0 ** 120)
+    o = torch.full((batch * Lq, D), 7.0, dtype=torch.bfloat16, device="cuda")
+    fb.fb_op_attention(model.handle, q, D, k, D, v, D, o, D, batch, Lq, Lkv, Lkv, heads, 128,
+                       impl)
+    torch.cuda.synchronize()
+    late, none = late.cpu().numpy(), none.cpu().numpy()
+    for b in sorted({0, batch - 1}):
+        for hd in sorted({0, heads - 1}):
+            c = slice(hd * 128, (hd + 1) * 128)
+            got = f64(o[b * Lq:(b + 1) * Lq, c])
+            qn = f64(q[b * Lq:(b + 1) * Lq, c])
+            kn, vn = (f64(x[b * Lkv:b * Lkv + end, c]) for x in (k, v))
+            for x in (qn, kn):
+                x[:, :3] = 0.0            # the bias channels add nothing to an unmasked score
+            kn[:, 1] = 0.0
+            assert np.isnan(got[none]).all()
+            for rows, first in ((~late & ~none, 0), (late, lead)):
+                want = O.attention(qn[rows][:, None], kn[first:][:, None],
+                                   vn[first:][:, None]).reshape(-1, 128)
+                assert np.isfinite(got[rows]).all()
+                assert rel_max(got[rows], want) <= 2e-2
+                assert np.abs(got[rows] - want).mean() <= 2e-3
+
+
 def test_attention_strided_qkv(model):
     """Self-attention reading q, k, v from one packed [rows][3D] buffer."""
     batch, L, heads, dh = 2, 97, 2, 128
