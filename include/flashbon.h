@@ -91,7 +91,7 @@ fb_status fb_set_stream(fb_model* m, void* stream);
  * device's). Persistent GEMM grids, the stream-K co-residency rule and the attention
  * kernel's CTA size are sized to it. Set it to the SM count of a partition whose stream
  * the model runs on (fb_sm_split_*): a GEMM that assumed more resident SM pairs than the
- * partition holds would leave its stream-K finishers waiting until their time limit.
+ * partition holds would have its stream-K contributors wait for pairs that have not started.
  * FB_EINVAL outside [2, device SMs]. Waits for the model's stream first. */
 fb_status fb_set_sm_budget(fb_model* m, int n_sms);
 
@@ -376,7 +376,9 @@ fb_status fb_gemm_streamk_noalloc(void* stream, int M, int N, int K, const void*
  * phases, stream-K counters) gives up after this many nanoseconds, records
  * "device wait timed out" in the call's error word, lets its copies in flight land,
  * frees its TMEM and returns; the call then returns FB_ECUDA and leaves the model
- * usable. ns = 0 restores the default (2 s). Applies to the current device and to every
+ * usable. (A stream-K contributor waits a 20000th of it for the others of its tile, 100 us by
+ * default; then it leaves its share to the last one, so that models on several streams of the
+ * whole device always make progress.) ns = 0 restores the default (2 s). Applies to the current device and to every
  * model and call on it; tests shorten it to make a wait run out quickly. Not for use
  * while kernels of the library are running.
  * fb_test_fail_alloc: host-side failure injection for device allocations. After the call
@@ -388,7 +390,11 @@ fb_status fb_gemm_streamk_noalloc(void* stream, int M, int N, int K, const void*
  * fb_gemm_streamk_noalloc) to a large negative value, as a crashed launch could leave
  * them, so that the next stream-K finisher waits for a count no launch will reach. The
  * wait runs out at the device wait limit, the call returns FB_ECUDA and clears the
- * counters; the call after it computes normally. */
+ * counters; the call after it computes normally.
+ * fb_test_request_handover: on != 0 puts every stream-K tile counter of the model into the
+ * state in which a tile's contributors hand their shares over to the last one (as when one
+ * has not started because other launches hold its SMs); a launch uses that state up on the
+ * tiles that it cuts. on = 0 clears the counters. */
 /* fb_probe_mma_rate: the tensor pipe's sustained rate on the current device, in MACs per SM
  * clock: every SM times (clock64) `reps` tcgen05.mma kind::f16 instructions of M = 128,
  * K = 16 and width n (64, 128 or 256) issued by each of `issuers` warps (1-4,
@@ -430,6 +436,7 @@ fb_status fb_set_device_wait_limit(unsigned long long ns);
 fb_status fb_test_fail_alloc(long k);
 long fb_test_alloc_calls(void);
 fb_status fb_test_poison_counters(fb_model* m);
+fb_status fb_test_request_handover(fb_model* m, int on);
 
 #ifdef __cplusplus
 }

@@ -1747,6 +1747,15 @@ fb_status fb_test_poison_counters(fb_model* m) {
   return FB_OK;
 }
 
+fb_status fb_test_request_handover(fb_model* m, int on) {
+  if (!m || !m->sk_ctr) return fail(FB_EINVAL, "model is NULL or has no stream-K counters");
+  const std::vector<int> v((size_t)m->sk_clusters * SK_CTR_PER_CLUSTER, on ? SK_HANDOVER : 0);
+  fb_stream_op_not_kernel();
+  CK(cudaMemcpyAsync(m->sk_ctr, v.data(), v.size() * sizeof(int), cudaMemcpyHostToDevice, m->st));
+  CK(cudaStreamSynchronize(m->st));
+  return FB_OK;
+}
+
 }  // extern "C"
 
 // ---- draft / refine pipeline step -------------------------------------------------

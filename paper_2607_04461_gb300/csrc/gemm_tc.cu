@@ -274,6 +274,7 @@ constexpr int C2_THREADS = 352;
 //   shares, waits (bounded) for the tile's count, and adds the others' partials of its own
 //   share to its accumulators, which stay in TMEM. One finisher per tile instead was the last
 //   to leave by far: 256 x 1536 x 8960 (13 contributors a tile) 18.6 us, 60.8 with one.
+//   If a contributor does not turn up, the others make room for it (sk_wait_all).
 // * Longer ranges: the first contributor finishes the tile alone as the others, which reach
 //   it at the start of their ranges, have published long before. (Sharing it too would put
 //   two more trips through the workspace at the end: 1040 x 5120 x 5120 50.3 us, 59.6.)
@@ -323,10 +324,24 @@ __device__ __forceinline__ float* sk_part(float* ws, int slot, int rank, int we)
 struct CutTile {
   int tile = -1, lo = 0, n = 0, last = 0, acc = 0;
 };
+// A cut tile's counter, one per CTA of the pair and epilogue warp, zero between launches:
+//   bits 0-9    contributors whose shares for the others are published
+//   bits 10-19  contributors that have seen all of them (the last one zeroes the counter)
+//   bits 20-29  contributors that have handed their own share over (the last one finishes the
+//               tile and zeroes the counter)
+//   bit 30      SK_HANDOVER, set while some contributor is missing
+constexpr int SK_SEEN = 1 << 10, SK_HANDED = 1 << 20, SK_COUNT = 0x3ff;
 // counts `n` on a cut tile's counter after this warp's (syncwarp'ed) writes; the old value
 __device__ __forceinline__ int sk_count(int* ctr, int n) {
   int old;
   asm volatile("atom.add.release.gpu.global.s32 %0, [%1], %2;"
+               : "=r"(old) : "l"(ctr), "r"(n) : "memory");
+  return old;
+}
+// the same, ordered before this warp's later reads of what others counted in too
+__device__ __forceinline__ int sk_count_acquire(int* ctr, int n) {
+  int old;
+  asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], %2;"
                : "=r"(old) : "l"(ctr), "r"(n) : "memory");
   return old;
 }
@@ -335,10 +350,10 @@ __device__ __forceinline__ int sk_load(const int* ctr) {
   asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
   return v;
 }
-// waits (bounded) for `n` counted in; the high half counts who has seen it
+// waits (bounded) until `n` contributors are in
 __device__ __forceinline__ bool sk_wait(const int* ctr, int n, int* err) {
   const uint64_t t0 = fb_globaltimer();
-  for (int c; (c = sk_load(ctr)) < 0 || (c & 0xffff) != n;) {
+  for (int c; (c = sk_load(ctr)) < 0 || (c & SK_COUNT) != n;) {
     if (*(volatile int*)err != 0) return false;
     if (fb_globaltimer() - t0 > fb_wait_limit()) {
       fb_report(err, FB_DEVERR_WAIT_TIMEOUT);
@@ -346,6 +361,30 @@ __device__ __forceinline__ bool sk_wait(const int* ctr, int n, int* err) {
     }
   }
   return true;
+}
+// Waits (bounded) until all `n` contributors of a shared tile are in, SK_SHARE. They may never
+// be while this grid waits: launches of other streams can hold the SMs that its missing clusters
+// need, waiting in the same way. So a contributor that has waited a 20000th of the wait limit
+// (100 us) for a missing one sets SK_HANDOVER: nobody waits any more, every contributor publishes
+// its own share too and counts that, and the last one to do so finishes the tile.
+enum { SK_GAVE_UP = 0, SK_SHARE, SK_HAND_OVER };
+__device__ __forceinline__ int sk_wait_all(int* ctr, int n, int* err) {
+  const uint64_t t0 = fb_globaltimer();
+  while (true) {
+    const int c = sk_load(ctr);
+    if (c >= 0) {
+      if (c & SK_HANDOVER) return SK_HAND_OVER;
+      if ((c & SK_COUNT) == n) return SK_SHARE;
+    }
+    if (*(volatile int*)err != 0) return SK_GAVE_UP;
+    const uint64_t waited = fb_globaltimer() - t0;
+    if (waited > fb_wait_limit()) {
+      fb_report(err, FB_DEVERR_WAIT_TIMEOUT);
+      return SK_GAVE_UP;
+    }
+    // (only while one is missing: the counter is still what was read)
+    if (c >= 0 && waited * 20000 > fb_wait_limit()) atomicCAS(ctr, c, c | SK_HANDOVER);
+  }
 }
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -552,11 +591,32 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
     // their segment is done, this cluster's share of their chunks finished after the range
     CutTile cut0, cut1, ct;
     int fin = 0;
-    int done_old = 0, done_all = -1;  // lanes 0 and 1: their cut tile's counter when read
+    // lanes 0 and 1 (cut0's, cut1's): how the tile is finished, whether this warp zeroes its
+    // counter at the end
+    int how = SK_SHARE;
+    bool reset_ctr = false;
     // ranges of at most two segments: the accumulators stay in TMEM to the end, and a
     // cluster's own share is neither published nor read back
     const bool keep = U <= (long long)n_clusters * nk;
     auto counter = [&](const CutTile& c) { return sk.ctr + ((size_t)c.lo * 2 + rank) * 8 + we; };
+    // chunks of a tile's accumulators into this cluster's slot of the workspace: its own share,
+    // i0 .. i1 - 1, or all others
+    auto publish_chunks = [&](const CutTile& c, uint32_t taddr, int nch, int i0, int i1, bool own) {
+      const int part_slot = 2 * cluster + (c.lo == cluster && c.last);
+      float4* part = reinterpret_cast<float4*>(sk_part(sk.ws, part_slot, (int)rank, we)) + lane;
+#pragma unroll 1
+      for (int i = 0; i < nch; ++i) {
+        if ((i >= i0 && i < i1) != own) continue;
+        uint32_t r[CH];
+        tmem_ld_chunk<CH>(taddr + i * 2 * CH, r);
+#pragma unroll
+        for (int j4 = 0; j4 < CH / 4; ++j4)
+          part[(i * (CH / 4) + j4) * 32] = make_float4(
+              __uint_as_float(r[4 * j4]), __uint_as_float(r[4 * j4 + 1]),
+              __uint_as_float(r[4 * j4 + 2]), __uint_as_float(r[4 * j4 + 3]));
+      }
+      __syncwarp();
+    };
     int next_acc = 0;
     uint32_t next_phase = 0;
     while (true) {
@@ -602,9 +662,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
         }
       }
       const size_t off0 = (size_t)(m0 + half * CH) * epi.ldo + f0 + lane;
-      const bool work = !publish && i0 < i1;
-      const float bias = work && epi.bias ? __ldg(epi.bias + f0 + lane) : 0.f;
-      const float gate = CC::F32 && work && epi.gate ? __ldg(epi.gate + f0 + lane) : 1.f;
+      const bool work = !publish && i0 < i1, any = !publish && nch > 0;
+      const float bias = any && epi.bias ? __ldg(epi.bias + f0 + lane) : 0.f;
+      const float gate = CC::F32 && any && epi.gate ? __ldg(epi.gate + f0 + lane) : 1.f;
       // residual chunk i into tile (i - i0) % NBUF (one lane)
       auto rload_issue = [&](int i) {
         const int t = (i - i0) % NBUF;
@@ -618,7 +678,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
 #pragma unroll
         for (int j = 0; j < 16; ++j) bv[j] = j < left ? __ldcg(p + (size_t)j * epi.ldo) : 0.f;
       };
-      if (work) {
+      auto first_loads = [&] {
         if (elect_one()) {
           bulk_wait_read<0>();  // the previous output tile's stores have left the tiles
           if (has_r) rload_issue(i0);
@@ -626,7 +686,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
         }
         __syncwarp();
         if (KIND == EPI_RESID_DELTA) load_base(i0);
-      }
+      };
+      if (work) first_loads();
       const uint32_t taddr =
           tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * acc_cols + half * CH;
       if (seg) {
@@ -638,21 +699,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
         if (!__all_sync(0xffffffffu, ok)) { failed = true; break; }
         tc_fence_after();
         if (publish) {
-          float4* part = reinterpret_cast<float4*>(
-                             sk_part(sk.ws, 2 * cluster + (sg.kb0 == 0 && ct.last), (int)rank, we)) +
-                         lane;
-#pragma unroll 1
-          for (int i = 0; i < nch; ++i) {
-            if (i >= i0 && i < i1) continue;
-            uint32_t r[CH];
-            tmem_ld_chunk<CH>(taddr + i * 2 * CH, r);
-#pragma unroll
-            for (int j4 = 0; j4 < CH / 4; ++j4)
-              part[(i * (CH / 4) + j4) * 32] = make_float4(
-                  __uint_as_float(r[4 * j4]), __uint_as_float(r[4 * j4 + 1]),
-                  __uint_as_float(r[4 * j4 + 2]), __uint_as_float(r[4 * j4 + 3]));
-          }
-          __syncwarp();
+          publish_chunks(ct, taddr, nch, i0, i1, false);
           if (lane == 0) sk_count(counter(ct), 1);
           if (keep) {
             cut1 = cut0;
@@ -667,20 +714,42 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
           }
           if (!__all_sync(0xffffffffu, in)) { failed = true; break; }
         }
-      } else if (fin == 1) {
-        // Wait (bounded) until every contributor's warp has counted in, for both cut tiles
-        // at once (lanes 0 and 1). All publish before they wait, at the ends of ranges of
-        // one length. Every contributor gets an SM: the grid is at most the resident-cluster
-        // count, and a dependent grid starts only after all of this grid's CTAs have started.
+      } else {
         bool ok = true;
-        const CutTile w = lane == 0 ? cut0 : cut1;
-        if (lane < 2 && w.tile >= 0) {
-          ok = sk_wait(counter(w), w.n, err);
-          // seen by this warp; whoever is the last to see it zeroes the counter (at the end)
-          done_all = w.n * 0x10001;
-          if (ok) done_old = sk_count(counter(w), 0x10000) + 0x10000;
+        if (fin == 1) {
+          // Wait (bounded) until every contributor's warp has counted in, for both cut tiles
+          // at once (lanes 0 and 1). All publish before they wait, at the ends of ranges of
+          // one length. With no other launch on its SMs every contributor is running: the grid
+          // is at most the resident-cluster count, and a dependent grid starts only after all of
+          // this grid's CTAs have started.
+          const CutTile w = lane == 0 ? cut0 : cut1;
+          if (lane < 2 && w.tile >= 0) {
+            how = sk_wait_all(counter(w), w.n, err);
+            ok = how != SK_GAVE_UP;
+            // seen by this warp; whoever is the last to see it zeroes the counter (at the end)
+            if (how == SK_SHARE)
+              reset_ctr = ((sk_count(counter(w), SK_SEEN) >> 10) & SK_COUNT) == w.n - 1;
+          }
+          if (!__all_sync(0xffffffffu, ok)) { failed = true; break; }
         }
-        if (!__all_sync(0xffffffffu, ok)) { failed = true; break; }
+        if (__shfl_sync(0xffffffffu, how, fin - 1) == SK_HAND_OVER) {
+          // the residual rows of this share have been asked for and are not used
+          for (int t = 0; t < 2 && has_r && i0 + t < i1; ++t) {
+            ok = mbar_wait(&wload[t], (rl_phase >> t) & 1u, err) && ok;
+            rl_phase ^= 1u << t;
+          }
+          if (!__all_sync(0xffffffffu, ok)) { failed = true; break; }
+          publish_chunks(ct, taddr, nch, i0, i1, true);
+          int handed = 0;
+          if (lane == 0) {
+            handed = (sk_count_acquire(counter(ct), SK_HANDED) >> 20) & SK_COUNT;
+            if (handed == ct.n - 1) *(volatile int*)counter(ct) = 0;  // nobody reads it any more
+          }
+          if (__shfl_sync(0xffffffffu, handed, 0) != ct.n - 1) continue;
+          i0 = 0;  // the last one: everything is published
+          i1 = nch;
+          if (nch > 0) first_loads();
+        }
       }
       if (!publish) {
         // TMEM columns from the tile's first accumulator to that of K part p
@@ -840,7 +909,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(C2_THREADS, 1)
         if (next_acc >= n_accs) { next_acc -= n_accs; next_phase ^= 1u; }
       }
     }
-    if (done_old == done_all)  // the last to see this cut tile's count: ready for reuse
+    if (reset_ctr)  // the last to see this cut tile's count: ready for reuse
       *(volatile int*)counter(lane == 0 ? cut0 : cut1) = 0;
   }
 

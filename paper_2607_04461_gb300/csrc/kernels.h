@@ -28,6 +28,7 @@ struct GemmArgs {
 // floats and counters of the stream-K workspace per cluster
 constexpr size_t SK_WS_FLOATS_PER_CLUSTER = 2 * 2 * 8 * 4096;
 constexpr int SK_CTR_PER_CLUSTER = 16;
+constexpr int SK_HANDOVER = 1 << 30;  // a counter's bit: see sk_wait_all
 // tcgen05 path: requires N % 128 == 0, K % 64 == 0, 16-byte aligned rows. Uses the
 // 2-SM (cta_group::2) kernel when N % 256 == 0 unless force_1sm.
 bool gemm_tc_supported(const GemmArgs& g);

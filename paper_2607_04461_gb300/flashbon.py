@@ -56,6 +56,7 @@ EXPORTS = ["fb_weights_count", "fb_weights_entry", "fb_init_model", "fb_free", "
            "fb_state_wait", "fb_set_sm_budget", "fb_sm_split_create", "fb_sm_split_info",
            "fb_sm_split_free", "fb_pipeline_step", "fb_set_device_wait_limit",
            "fb_test_fail_alloc", "fb_test_alloc_calls", "fb_test_poison_counters",
+           "fb_test_request_handover",
            "fb_probe_mma_rate", "fb_probe_mma_gap", "fb_probe_mufu", "fb_probe_tmem_load",
            "fb_probe_mma_mix"]
 
@@ -112,6 +113,7 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
         "fb_test_fail_alloc": (I, [ctypes.c_long]),
         "fb_test_alloc_calls": (ctypes.c_long, []),
         "fb_test_poison_counters": (I, [P]),
+        "fb_test_request_handover": (I, [P, I]),
         "fb_probe_mma_rate": (I, [I, I, I, ctypes.POINTER(ctypes.c_double)]),
         "fb_probe_mma_gap": (I, [I, ctypes.POINTER(ctypes.c_double)]),
         "fb_probe_mufu": (I, [I, ctypes.POINTER(ctypes.c_double)]),
@@ -393,6 +395,12 @@ def fb_test_poison_counters(model) -> None:
     """Sets the stream-K counters of `model` (None: the allocation-free entry point's) to
     a large negative value, so the next stream-K finisher's wait cannot complete."""
     _check(load_library().fb_test_poison_counters(model))
+
+
+def fb_test_request_handover(model, on: bool) -> None:
+    """Makes the contributors of the next launch's cut stream-K tiles hand their shares over
+    to the last one (on), or clears the counters (off)."""
+    _check(load_library().fb_test_request_handover(model, int(on)))
 
 
 def fb_probe_mma_rate(issuers: int, n: int, reps: int = 16384) -> float:

@@ -154,6 +154,45 @@ def test_gemm_k_ranges(model, M, N, K, impl, blocks, epi):
     assert err <= (1.2e-7 * blocks if epi else 2.0 ** -9)
 
 
+@pytest.mark.parametrize("M,N,K", [
+    (1, 1536, 8960),      # 13 contributors a tile, one token: most shares are empty
+    (256, 1536, 8960),    # 13 contributors, full tiles
+    (200, 512, 9728),     # two tiles, 38 contributors each
+    (640, 1536, 8960),    # ranges that meet two cut tiles
+    (1560, 1536, 8960),   # 42 tiles, two to four contributors
+])
+@pytest.mark.parametrize("epi", [0, 1, 2, 3])
+def test_gemm_stream_k_handover(M, N, K, epi):
+    """Contributors that hand their shares over to a tile's last one (as they do when one of
+    them does not start): the sums keep their K order, so the result is that of the shared
+    finish bit for bit, and the counters are zero again for the next launch."""
+    A, W = randn((M, K), 61), randn((N, K), 62, scale=K ** -0.5)
+    bias, gate = randn((N,), 63, dtype=torch.float32), randn((N,), 64, dtype=torch.float32)
+    resid = randn((M, N), 65, dtype=torch.float32) if epi >= 2 else None
+    outs = []
+    with fb.Model(synth.TINY, synth.make_weights(synth.TINY)) as m:
+        for handover in (False, True, False):
+            out = torch.full((M, N), float("nan"), device="cuda",
+                             dtype=torch.float32 if epi >= 2 else torch.bfloat16)
+            delta = torch.full((M, N), float("nan"), dtype=torch.bfloat16, device="cuda")
+            if handover:
+                fb.fb_test_request_handover(m.handle, True)
+            fb.fb_op_gemm(m.handle, M, N, K, A, W, bias, epi, out, resid,
+                          gate if epi >= 2 else None, resid if epi == 3 else None,
+                          delta if epi == 3 else None, 4)
+            outs.append((out, delta))
+        fb.fb_test_request_handover(m.handle, False)
+    torch.cuda.synchronize()
+    want = f64(A) @ f64(W).T + f64(bias)
+    got = f64(outs[0][0])
+    want = O.gelu_tanh(want) if epi == 1 else want if epi == 0 else f64(resid) + f64(gate) * want
+    assert rel_max(got, want) <= (1e-2 if epi < 2 else 1e-4)
+    for out, delta in outs[1:]:
+        assert torch.equal(out, outs[0][0])
+        if epi == 3:
+            assert torch.equal(delta, outs[0][1])
+
+
 @pytest.mark.parametrize("M,N,K,twin", [
     (1560, 1536, 8960, 4),   # 42 tiles, 140 K blocks: stream-K
     (640, 1536, 8960, 4),    # 18 tiles, 140 K blocks: stream-K
