@@ -386,15 +386,18 @@ fb_status fb_gemm_streamk_noalloc(void* stream, int M, int N, int K, const void*
  * numbered k fails as an out-of-memory cudaMalloc would (the caller sees FB_ENOMEM).
  * k < 0 disarms. fb_test_alloc_calls: allocations counted since the last
  * fb_test_fail_alloc. Process-wide; not thread-safe against concurrent model creation.
- * fb_test_poison_counters: sets the model's stream-K tile counters (m = NULL: those of
- * fb_gemm_streamk_noalloc) to a large negative value, as a crashed launch could leave
- * them, so that the next stream-K finisher waits for a count no launch will reach. The
- * wait runs out at the device wait limit, the call returns FB_ECUDA and clears the
- * counters; the call after it computes normally.
+ * fb_test_poison_counters: sets the model's stream-K tile counters and the flags of its
+ * attention's key split (m = NULL: the counters of fb_gemm_streamk_noalloc) to a large
+ * negative value, as a crashed launch could leave them, so that the next stream-K finisher
+ * waits for a count, and the next finisher of a cut attention item for a flag, that no launch
+ * will reach. The wait runs out at the device wait limit, the call returns FB_ECUDA and
+ * clears both; the call after it computes normally.
  * fb_test_request_handover: on != 0 puts every stream-K tile counter of the model into the
  * state in which a tile's contributors hand their shares over to the last one (as when one
  * has not started because other launches hold its SMs); a launch uses that state up on the
- * tiles that it cuts. on = 0 clears the counters. */
+ * tiles that it cuts. on = 0 clears the counters.
+ * fb_test_attention_split: *ctas = the CTAs among which fb_op_attention of these sizes
+ * (head_dim 128, 16-byte aligned rows) cuts its items by key range, 0 where none is cut. */
 /* fb_probe_mma_rate: the tensor pipe's sustained rate on the current device, in MACs per SM
  * clock: every SM times (clock64) `reps` tcgen05.mma kind::f16 instructions of M = 128,
  * K = 16 and width n (64, 128 or 256) issued by each of `issuers` warps (1-4,
@@ -437,6 +440,8 @@ fb_status fb_test_fail_alloc(long k);
 long fb_test_alloc_calls(void);
 fb_status fb_test_poison_counters(fb_model* m);
 fb_status fb_test_request_handover(fb_model* m, int on);
+fb_status fb_test_attention_split(fb_model* m, int batch, int Lq, int Lkv, int heads, int impl,
+                                  int* ctas);
 
 #ifdef __cplusplus
 }

@@ -373,14 +373,17 @@ GemmArgs gemm_args(int M, int N, int K, const bf16* A, const bf16* W, const floa
 }
 
 // impl: 0 automatic (tcgen05 for head_dim 128), 1 the mma.sync kernel, 2 / 3 the tcgen05
-// kernel with 128- / 256-query CTAs
-fb_status run_attn(fb_model* m, const AttnArgs& a0, int kind, int impl = 0) {
-  AttnArgs a = a0;
+// kernel with 128- / 256-query CTAs, 4 the persistent 256-query kernel
+void attn_resources(fb_model* m, int impl, AttnArgs& a) {
   a.tc_variant = impl >= 2 ? impl - 1 : 0;
   a.sms = m->num_sms;
   a.ws = m->attn_ws;
   a.flags = m->attn_flags;
   a.ws_ctas = m->dev_sms;
+}
+fb_status run_attn(fb_model* m, const AttnArgs& a0, int kind, int impl = 0) {
+  AttnArgs a = a0;
+  attn_resources(m, impl, a);
   const double flops = 4.0 * a.batch * a.heads * (double)a.Lq * a.Lkv * a.head_dim;
   const double kvb = (a.kv_batch_rows ? a.batch : 1) * 2.0 * a.Lkv * a.heads * a.head_dim * 2;
   const double bytes = 2.0 * a.batch * a.Lq * (double)a.heads * a.head_dim * 2 + kvb;
@@ -1743,7 +1746,22 @@ fb_status fb_test_poison_counters(fb_model* m) {
   if (!ctr) return fail(FB_EINVAL, "no stream-K counters");
   fb_stream_op_not_kernel();
   CK(cudaMemsetAsync(ctr, 0x80, n * sizeof(int), st));  // every counter 0x80808080 < 0
+  if (m)
+    CK(cudaMemsetAsync(m->attn_flags, 0x80, (size_t)m->dev_sms * ATTN_FLAGS_PER_CTA * sizeof(int),
+                       st));
   CK(cudaStreamSynchronize(st));
+  return FB_OK;
+}
+
+fb_status fb_test_attention_split(fb_model* m, int batch, int Lq, int Lkv, int heads, int impl,
+                                  int* ctas) {
+  if (!m || !ctas) return fail(FB_EINVAL, "null argument");
+  if (batch < 1 || Lq < 1 || Lkv < 1 || heads < 1 || impl < 0 || impl > 4)
+    return fail(FB_EINVAL, "bad sizes or impl");
+  AttnArgs a{};
+  a.batch = batch; a.Lq = Lq; a.Lkv = Lkv; a.heads = heads; a.head_dim = 128;
+  attn_resources(m, impl, a);
+  *ctas = impl == 1 ? 0 : attention_tc_split(a);
   return FB_OK;
 }
 

@@ -883,10 +883,11 @@ __device__ __forceinline__ bool get_seg(const Params& p, const SplitPlan& pl, in
   g = Seg{pl.tail_item, pl.tail_j0, n_kv, SEG_FINISH};
   return true;
 }
-// Waits (bounded, as mbar_wait) until another CTA has raised its flag.
+// Waits (bounded, as mbar_wait) until another CTA has raised its flag from 0 to 1 (any other
+// value, as a crashed launch could leave it, is waited on until the time limit).
 __device__ __forceinline__ bool wait_flag(int* flag, int* err) {
   const uint64_t t0 = fb_globaltimer();
-  while (*(volatile int*)flag == 0) {
+  while (*(volatile int*)flag != 1) {
     if (*(volatile int*)err != 0) return false;
     if (fb_globaltimer() - t0 > fb_wait_limit()) {
       fb_report(err, FB_DEVERR_WAIT_TIMEOUT);
@@ -896,11 +897,11 @@ __device__ __forceinline__ bool wait_flag(int* flag, int* err) {
   }
   return true;
 }
-// Whole warp: makes its earlier stores visible and sets the flag.
+// Whole warp: makes its earlier stores visible and raises the flag.
 __device__ __forceinline__ void raise_flag(int* flag, int lane) {
   __threadfence();
   __syncwarp();
-  if (lane == 0) atomicExch(flag, 1);
+  if (lane == 0) atomicAdd(flag, 1);
 }
 // The finisher of a cut item waits for the parts of CTAs c_lo .. blockIdx.x - 1 (this warp's
 // rows: flags by lane), updates the row's maximum m and sum l with theirs, in CTA order, and
@@ -1486,9 +1487,9 @@ bool map_o(CUtensorMap* m, const bf16* ptr, int batch, int Lq, int cols, int ld)
 // 40.8 / 35.2, 4 x 1560 60.9 / 57.8, 8 x 1560 103.3 / 102.7, 16 x 1560 186.9 / 202.9, 1 x 4096
 // 93.8 / 71.8, 4 x 4096 279.7 / 258.6, 1 x 1560 on 40 SMs 58.3 / 51.4, cross-attention (4 key
 // tiles) 4 x 1560 23.9 / 27.5.
-int plan_split(const AttnArgs& a, int sms, long items, Params* p) {
+int plan_split(const AttnArgs& a, int sms, Params* p) {
   const int n_kv = (a.Lkv + TB - 1) / TB;
-  const long bh = (long)a.heads * a.batch;
+  const long bh = (long)a.heads * a.batch, items = (a.Lq + 2 * TB - 1) / (2 * TB) * bh;
   p->n_full_qb = (a.Lq + TB - 1) / (2 * TB);
   const long n_full = p->n_full_qb * bh, lone = items - n_full;
   p->n_full = (int)n_full;
@@ -1522,42 +1523,16 @@ int plan_split(const AttnArgs& a, int sms, long items, Params* p) {
   return (int)G;
 }
 
-}  // namespace
-
-cudaError_t attention_tc_set_wait_limit(unsigned long long ns) {
-  return fb_set_wait_limit_tu(ns);
-}
-
-bool attention_tc_supported(const AttnArgs& a) {
-  auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
-  return a.head_dim == 128 && a.Lq >= 1 && a.Lkv >= 1 && a.batch >= 1 && a.ldq % 8 == 0 &&
-         a.ldk % 8 == 0 && a.ldv % 8 == 0 && a.ldo % 8 == 0 && al16(a.Q) && al16(a.K) &&
-         al16(a.V) && al16(a.O);
-}
-
-cudaError_t attention_tc(const AttnArgs& a, int* err, cudaStream_t st) {
-  if (!attention_tc_supported(a)) return cudaErrorInvalidValue;
-  const int cols = a.heads * 128;
-  const int kv_rows = a.kv_batch_rows ? (a.batch - 1) * a.kv_batch_rows + a.Lkv : a.Lkv;
-  CUtensorMap mq, mk, mv, mo;
-  if (!map_128x64(&mq, a.Q, a.batch * a.Lq, cols, a.ldq) ||
-      !map_128x64(&mk, a.K, kv_rows, cols, a.ldk) || !map_128x64(&mv, a.V, kv_rows, cols, a.ldv) ||
-      !map_o(&mo, a.O, a.batch, a.Lq, cols, a.ldo))
-    return cudaErrorInvalidValue;
+int sms_of(const AttnArgs& a) {
   int dev = 0, sms = a.sms;
   if (sms <= 0 && (cudaGetDevice(&dev) != cudaSuccess ||
                    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess))
     sms = 148;
-  Params p;
-  p.Lq = a.Lq;
-  p.Lkv = a.Lkv;
-  p.kv_batch_rows = a.kv_batch_rows;
-  p.O = a.O;
-  p.ldo = a.ldo;
-  p.scale_log2 = 1.4426950408889634f / sqrtf(128.f);
-  p.err = err;
-  p.batch = a.batch;
-  p.heads = a.heads;
+  return sms;
+}
+
+enum Form { Q128, Q256, PERSISTENT };
+Form choose_form(const AttnArgs& a, int sms) {
   // 256-query items share each K/V tile between two query tiles and overlap one tile's
   // softmax with the other's MMAs; in the persistent kernel one costs about 1.25 times a
   // 128-query CTA (measured on a 40-SM partition, 1 x 1560 queries x 12 heads: 4 waves of
@@ -1576,8 +1551,53 @@ cudaError_t attention_tc(const AttnArgs& a, int* err, cudaStream_t st) {
   // kernel
   const bool persistent = (a.tc_variant >= 3 || (two && a.tc_variant == 0)) &&
                           ctas2 * (a.heads > nqb ? a.heads : nqb) < (1ll << 32);  // see div_by
-  if (persistent) {
-    const int grid = plan_split(a, sms, ctas2, &p);
+  return persistent ? PERSISTENT : two ? Q256 : Q128;
+}
+
+}  // namespace
+
+cudaError_t attention_tc_set_wait_limit(unsigned long long ns) {
+  return fb_set_wait_limit_tu(ns);
+}
+
+bool attention_tc_supported(const AttnArgs& a) {
+  auto al16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
+  return a.head_dim == 128 && a.Lq >= 1 && a.Lkv >= 1 && a.batch >= 1 && a.ldq % 8 == 0 &&
+         a.ldk % 8 == 0 && a.ldv % 8 == 0 && a.ldo % 8 == 0 && al16(a.Q) && al16(a.K) &&
+         al16(a.V) && al16(a.O);
+}
+
+int attention_tc_split(const AttnArgs& a) {
+  const int sms = sms_of(a);
+  Params p;
+  if (!attention_tc_supported(a) || choose_form(a, sms) != PERSISTENT) return 0;
+  const int grid = plan_split(a, sms, &p);
+  return p.split ? grid : 0;
+}
+
+cudaError_t attention_tc(const AttnArgs& a, int* err, cudaStream_t st) {
+  if (!attention_tc_supported(a)) return cudaErrorInvalidValue;
+  const int cols = a.heads * 128;
+  const int kv_rows = a.kv_batch_rows ? (a.batch - 1) * a.kv_batch_rows + a.Lkv : a.Lkv;
+  CUtensorMap mq, mk, mv, mo;
+  if (!map_128x64(&mq, a.Q, a.batch * a.Lq, cols, a.ldq) ||
+      !map_128x64(&mk, a.K, kv_rows, cols, a.ldk) || !map_128x64(&mv, a.V, kv_rows, cols, a.ldv) ||
+      !map_o(&mo, a.O, a.batch, a.Lq, cols, a.ldo))
+    return cudaErrorInvalidValue;
+  const int sms = sms_of(a);
+  Params p;
+  p.Lq = a.Lq;
+  p.Lkv = a.Lkv;
+  p.kv_batch_rows = a.kv_batch_rows;
+  p.O = a.O;
+  p.ldo = a.ldo;
+  p.scale_log2 = 1.4426950408889634f / sqrtf(128.f);
+  p.err = err;
+  p.batch = a.batch;
+  p.heads = a.heads;
+  const Form form = choose_form(a, sms);
+  if (form == PERSISTENT) {
+    const int grid = plan_split(a, sms, &p);
     auto kern = p.split ? attn_tc2p_kernel<true> : attn_tc2p_kernel<false>;
     cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES);
@@ -1586,7 +1606,7 @@ cudaError_t attention_tc(const AttnArgs& a, int* err, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
   }
-  if (two) {
+  if (form == Q256) {
     cudaError_t e = cudaFuncSetAttribute(attn_tc2_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM2_BYTES);
     if (e != cudaSuccess) return e;

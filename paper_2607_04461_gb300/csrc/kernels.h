@@ -65,6 +65,8 @@ bool attention_tc_supported(const AttnArgs& a);
 cudaError_t attention_tc(const AttnArgs& a, int* err, cudaStream_t st);
 // Sets the attention_tc unit's device wait limit on the current device (ns).
 cudaError_t attention_tc_set_wait_limit(unsigned long long ns);
+// The CTAs among which attention_tc cuts items by key range, 0 where it does not cut any.
+int attention_tc_split(const AttnArgs& a);
 
 // ---- pointwise / small kernels ------------------------------------------------------
 // out[r][:] = bf16(LN(x[r][:]) * (mul_base + mul[:]) + add[:]), x fp32 [rows][D].

@@ -56,7 +56,7 @@ EXPORTS = ["fb_weights_count", "fb_weights_entry", "fb_init_model", "fb_free", "
            "fb_state_wait", "fb_set_sm_budget", "fb_sm_split_create", "fb_sm_split_info",
            "fb_sm_split_free", "fb_pipeline_step", "fb_set_device_wait_limit",
            "fb_test_fail_alloc", "fb_test_alloc_calls", "fb_test_poison_counters",
-           "fb_test_request_handover",
+           "fb_test_request_handover", "fb_test_attention_split",
            "fb_probe_mma_rate", "fb_probe_mma_gap", "fb_probe_mufu", "fb_probe_tmem_load",
            "fb_probe_mma_mix"]
 
@@ -114,6 +114,7 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
         "fb_test_alloc_calls": (ctypes.c_long, []),
         "fb_test_poison_counters": (I, [P]),
         "fb_test_request_handover": (I, [P, I]),
+        "fb_test_attention_split": (I, [P, I, I, I, I, I, ctypes.POINTER(I)]),
         "fb_probe_mma_rate": (I, [I, I, I, ctypes.POINTER(ctypes.c_double)]),
         "fb_probe_mma_gap": (I, [I, ctypes.POINTER(ctypes.c_double)]),
         "fb_probe_mufu": (I, [I, ctypes.POINTER(ctypes.c_double)]),
@@ -395,6 +396,14 @@ def fb_test_poison_counters(model) -> None:
     """Sets the stream-K counters of `model` (None: the allocation-free entry point's) to
     a large negative value, so the next stream-K finisher's wait cannot complete."""
     _check(load_library().fb_test_poison_counters(model))
+
+
+def fb_test_attention_split(model, batch, Lq, Lkv, heads, impl=0) -> int:
+    """CTAs among which fb_op_attention cuts its items by key range (0: none is cut)."""
+    ctas = ctypes.c_int()
+    _check(load_library().fb_test_attention_split(model, batch, Lq, Lkv, heads, impl,
+                                                  ctypes.byref(ctas)))
+    return ctas.value
 
 
 def fb_test_request_handover(model, on: bool) -> None:

@@ -1,9 +1,9 @@
 """Failure detection without a GPU fault.
 
-* A device-side wait that runs out: with the stream-K tile counters poisoned (as a
-  crashed launch could leave them) a finisher waits for a count no launch reaches; with a
-  short wait limit the wait gives up, the call must return FB_ECUDA with "device wait
-  timed out", and the model must work again at once.
+* Device-side waits that run out: with the stream-K tile counters and the flags of the
+  attention's key split poisoned (as a crashed launch could leave them) a finisher waits for
+  a count or flag no launch reaches; with a short wait limit the wait gives up, the call must
+  return FB_ECUDA with "device wait timed out", and the model must work again at once.
 * Host-injected allocation failures: every device allocation of fb_init_model is made to
   fail in turn; each attempt must return FB_ENOMEM, leave *out NULL and leak no device
   memory. A failure inside a sampling call leaves the model usable.
@@ -63,6 +63,56 @@ def test_stream_k_wait_times_out_then_recovers(model):
         fb.fb_op_gemm(model.handle, M, N, K, A, W, bias, 2, again, resid, gate, None, None, 4)
         torch.cuda.synchronize()
         assert torch.equal(again, ref)
+
+
+def test_stream_k_single_finisher_times_out_then_recovers(model):
+    """The same where ranges are longer than a tile: the tile's first contributor waits."""
+    M, N, K = 1040, 5120, 5120
+    A, W = randn((M, K), 11), randn((N, K), 12, scale=K ** -0.5)
+    run = lambda out: fb.fb_op_gemm(model.handle, M, N, K, A, W, None, 0, out, None, None,  # noqa: E731
+                                    None, None, 4)
+    ref, out = (torch.zeros((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    run(ref)
+    fb.fb_test_poison_counters(model.handle)
+    fb.fb_set_device_wait_limit(SHORT_WAIT_NS)
+    try:
+        with pytest.raises(fb.FlashBonError) as e:
+            run(out)
+    finally:
+        fb.fb_set_device_wait_limit(0)
+    assert e.value.status == fb.FB_ECUDA and "device wait timed out" in str(e.value)
+    for _ in range(2):
+        out.zero_()
+        run(out)
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref)
+
+
+def test_attention_split_wait_times_out_then_recovers(model):
+    """With the flags of the key split poisoned, the finishers of cut items wait for a value
+    that no launch raises them to; the failed call clears them."""
+    batch, L, heads = 1, 2500, 8
+    assert fb.fb_test_attention_split(model.handle, batch, L, L, heads, 4) > 0
+    D = heads * 128
+    q, k, v = (randn((batch * L, D), 21 + i) for i in range(3))
+    run = lambda out: fb.fb_op_attention(model.handle, q, D, k, D, v, D, out, D, batch, L, L,  # noqa: E731
+                                         L, heads, 128, 4)
+    ref, out = (torch.zeros((batch * L, D), dtype=torch.bfloat16, device="cuda")
+                for _ in range(2))
+    run(ref)
+    fb.fb_test_poison_counters(model.handle)
+    fb.fb_set_device_wait_limit(SHORT_WAIT_NS)
+    try:
+        with pytest.raises(fb.FlashBonError) as e:
+            run(out)
+    finally:
+        fb.fb_set_device_wait_limit(0)
+    assert e.value.status == fb.FB_ECUDA and "device wait timed out" in str(e.value)
+    for _ in range(2):
+        out.zero_()
+        run(out)
+        torch.cuda.synchronize()
+        assert torch.equal(out, ref)
 
 
 def _raw_init(cfg, weights):

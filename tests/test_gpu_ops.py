@@ -394,6 +394,8 @@ def test_attention_key_split(model, batch, Lq, Lkv, heads, shared):
     """Items whose key range is cut between CTAs (equal shares per SM): against the fp64
     oracle on sampled heads, and bit for bit the same on a second and third call (the parts
     are added in CTA order; the flags are back at zero)."""
+    cut = fb.fb_test_attention_split(model.handle, batch, Lq, Lkv, heads)
+    assert (cut > 0) == (Lkv > 512)
     D = heads * 128
     q = randn((batch * Lq, D), 81)
     k = randn(((1 if shared else batch) * Lkv, D), 82)
@@ -430,6 +432,8 @@ def test_attention_masked_keys(model, batch, Lq, Lkv, heads, impl):
     for every row (whole parts of cut items), the first 300 keys (two tiles and a piece) for
     one row per warp, and every key for another. The oracle sees the unmasked keys only; a row
     without any has no value (NaN), and its neighbours in the warp keep theirs."""
+    cut = fb.fb_test_attention_split(model.handle, batch, Lq, Lkv, heads, impl)
+    assert (cut > 0) == (Lkv > 700)
     D, lead, end = heads * 128, 300, Lkv // 2
     q, k, v = (randn((batch * n, D), 100 + i) for i, n in enumerate((Lq, Lkv, Lkv)))
     q4, k4 = q.view(batch, Lq, heads, 128), k.view(batch, Lkv, heads, 128)
