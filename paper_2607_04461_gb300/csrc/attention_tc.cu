@@ -50,8 +50,9 @@ struct Params {
   int* err;
   int batch, heads;
   // the persistent kernel's work split (see SplitPlan)
-  int n_full_qb;     // 256-query items per head with both query tiles in range
-  int n_full, n_items;         // such items in all, items in all
+  int n_full_qb;     // 256-query items per head among the first n_full items
+  int n_full, n_items;         // of all items; those behind the first n_full have one query tile
+  int lone_qb;       // and among the first n_full those of this pair have (-1: none)
   unsigned div_qb, div_heads;  // ceil(2^32 / n_full_qb), ceil(2^32 / heads): see div_by
   int split;         // != 0: the items from `rounds` full rounds on are cut into equal shares
   int rounds;
@@ -753,7 +754,8 @@ __global__ void __launch_bounds__(THREADS2, 1)
 // whole items (batch b, head h, query-tile pair qb) and, where whole items would leave SMs
 // idle in the last round, parts of the key range of one item. Items are numbered with the
 // pairs of two query tiles first (qb fastest, so that the CTAs running at the same time
-// share their K/V tiles in L2), then the items of a last single tile. Per CTA the work of
+// share their K/V tiles in L2), then the items of a last single tile, or by head throughout
+// (single_tiles_in_place). Per CTA the work of
 // consecutive segments overlaps:
 //  * the producer loads the next segment's Q as soon as the current one's last S MMAs are
 //    done (q_empty) and carries on through the K/V rings, whose slots and phases count
@@ -968,7 +970,14 @@ __device__ __forceinline__ int decode_item(const Params& p, int item, int& qb, i
   }
   b = div_by(bh, p.div_heads);
   h = bh - b * p.heads;
-  return full ? 2 : 1;
+  return full && qb != p.lone_qb ? 2 : 1;
+}
+// groups with work of an item
+template <bool SPLIT>
+__device__ __forceinline__ int item_tiles(const Params& p, int item) {
+  if (item >= p.n_full) return 1;
+  if (SPLIT) return 2;  // (cut items: single query tiles are the last items)
+  return item - div_by(item, p.div_qb) * p.n_full_qb != p.lone_qb ? 2 : 1;
 }
 
 // One O row: 32 columns at a time, scaled by inv and rounded to bf16, in 32-byte stores (whole
@@ -1166,7 +1175,7 @@ __global__ void __launch_bounds__(THREADS2, 1)
     for (int it = 0; ok; ++it) {
       Seg sg;
       if (!__all_sync(0xffffffffu, get_seg<SPLIT>(p, plan, it, n_kv, sg))) break;
-      const bool two = __all_sync(0xffffffffu, sg.item < p.n_full);  // both query tiles
+      const bool two = __all_sync(0xffffffffu, item_tiles<SPLIT>(p, sg.item) == 2);
       int j = sg.j0;
       bool last = __all_sync(0xffffffffu, j + 1 == n_kv);
       if (!(ok = mbar_wait_warp(q_full, it & 1, err))) break;
@@ -1243,7 +1252,7 @@ __global__ void __launch_bounds__(THREADS2, 1)
       {
         Seg sg;
         if (!get_seg<SPLIT>(p, plan, it, n_kv, sg)) break;
-        const int ng = sg.item < p.n_full ? 2 : 1;
+        const int ng = item_tiles<SPLIT>(p, sg.item);
         if (g >= ng) {  // this tile lies past Lq: no work
           kt += sg.j1 - sg.j0;
           if (SPLIT) raise_due();
@@ -1479,6 +1488,20 @@ bool map_o(CUtensorMap* m, const bf16* ptr, int batch, int Lq, int cols, int ld)
              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Whole items: whether the single query tiles (Lq's last one) run behind the other tiles of their
+// head instead of after all pairs. Last they fill the last round better, but read their head's
+// K / V again: from DRAM where the K / V of all heads are more than about half of L2, once more
+// per n_pairs reads. Measured (us, last / in place; 12 heads): 16 x 384 queries (38 MB of K / V)
+// 20.4 / 21.5, 24 x 384 29.0 / 30.8, 16 x 600 41.9 / 41.8, 16 x 640 (63 MB) 42.3 / 41.0, 32 x 384
+// 43.2 / 42.2, 64 x 384 81.1 / 73.2, 64 x 600 156.1 / 148.7, 64 x 640 159.7 / 148.2, 32 x 896
+// 141.7 / 136.7, 32 x 1100 209.4 / 204.7, 32 x 1408 302.7 / 299.3; from six pairs on within 1.5 %
+// either way (8 x 1560 105.0 / 106.7, 32 x 1560 390.6 / 389.8, on 112 SMs 478.4 / 481.7, 8 x 3200
+// 341.4 / 344.8). Shared K / V stay in L2: 64 x 384 x 77 keys 39.1 / 43.5.
+bool single_tiles_in_place(const AttnArgs& a, int n_pairs) {
+  const double kv = 4.0 * 128 * a.heads * (double)a.Lkv * (a.kv_batch_rows ? a.batch : 1);
+  return n_pairs <= 5 && kv > 60e6;
+}
+
 // Chooses the persistent kernel's split and grid. Times in 128-key steps of a 256-query item
 // (1.45-1.55 us): whole items take their rounds; with the split every CTA takes an equal share,
 // its steps are about 5 % longer (the ranges share less K / V, the loop keeps more registers),
@@ -1497,12 +1520,22 @@ int plan_split(const AttnArgs& a, int sms, Params* p) {
   auto recip = [](int d) { return d > 1 ? (unsigned)((0x100000000ull + d - 1) / d) : 0u; };
   p->div_qb = recip(p->n_full_qb);
   p->div_heads = recip(a.heads);
+  p->lone_qb = -1;
   p->ws = a.ws;
   p->flags = a.flags;
   p->split = 0;
   p->rounds = 0;
   const int grid = (int)(items < sms ? items : sms);
-  if (!a.ws || !a.flags || sms > a.ws_ctas) return grid;
+  auto whole = [&] {
+    if (lone > 0 && single_tiles_in_place(a, p->n_full_qb)) {
+      p->n_full_qb += 1;
+      p->n_full = p->n_items;
+      p->lone_qb = p->n_full_qb - 1;
+      p->div_qb = recip(p->n_full_qb);
+    }
+    return grid;
+  };
+  if (!a.ws || !a.flags || sms > a.ws_ctas) return whole();
   // full rounds of two-tile items but one, so that every CTA's share of the rest is at least
   // about one item and an item is cut in few parts
   const double total = (4.0 * n_full + 3.0 * lone) * n_kv / 4;  // steps
@@ -1517,7 +1550,7 @@ int plan_split(const AttnArgs& a, int sms, Params* p) {
   const double t_split = 1.05 * (rounds * n_kv + share) + 4.5 + parts;
   const double t_whole = (double)((items + sms - 1) / sms) * n_kv;
   // (the split's 32-bit unit arithmetic: see SplitUnits)
-  if (G <= 1 || t_split >= 0.98 * t_whole || total * 4 * sms > 4e9) return grid;
+  if (G <= 1 || t_split >= 0.98 * t_whole || total * 4 * sms > 4e9) return whole();
   p->split = 1;
   p->rounds = (int)rounds;
   return (int)G;

@@ -420,6 +420,33 @@ def test_attention_key_split(model, batch, Lq, Lkv, heads, shared):
             assert np.abs(got - want).mean() <= 2e-3
 
 
+@pytest.mark.parametrize("batch,Lq,heads", [
+    (40, 300, 11),   # one pair and a single tile with 44 rows
+    (20, 640, 12),   # two pairs and a full single tile
+    (14, 1400, 9),   # five pairs and a single tile
+])
+def test_attention_single_tiles_in_place(model, batch, Lq, heads):
+    """More than 60 MB of K / V: the single last query tiles are numbered with their heads. The
+    first, a middle and the last batch element's heads against the fp64 oracle; every row of
+    the others agrees with the one-item-per-CTA kernel (bf16 rounding of P and O)."""
+    D = heads * 128
+    q, k, v = (randn((batch * Lq, D), 110 + i) for i in range(3))
+    o, one = (torch.full((batch * Lq, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+              for _ in range(2))
+    assert 4 * batch * Lq * D > 60e6
+    assert fb.fb_test_attention_split(model.handle, batch, Lq, Lq, heads) == 0
+    for out, impl in ((o, 0), (one, 3)):
+        fb.fb_op_attention(model.handle, q, D, k, D, v, D, out, D, batch, Lq, Lq, Lq, heads, 128,
+                           impl)
+    torch.cuda.synchronize()
+    assert rel_max(f64(o), f64(one)) <= 2e-2
+    for b in (0, batch // 2, batch - 1):
+        for hd in (0, heads - 1):
+            r, c = slice(b * Lq, (b + 1) * Lq), slice(hd * 128, (hd + 1) * 128)
+            want = O.attention(*(f64(x[r, c])[:, None] for x in (q, k, v))).reshape(Lq, 128)
+            assert rel_max(f64(o[r, c]), want) <= 2e-2
+
+
 @pytest.mark.parametrize("batch,Lq,Lkv,heads,impl", [
     (3, 900, 1300, 14, 0),   # every item cut into two parts
     (1, 2500, 4100, 6, 4),   # about three parts an item
