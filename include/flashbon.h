@@ -397,7 +397,12 @@ fb_status fb_gemm_streamk_noalloc(void* stream, int M, int N, int K, const void*
  * has not started because other launches hold its SMs); a launch uses that state up on the
  * tiles that it cuts. on = 0 clears the counters.
  * fb_test_attention_split: *ctas = the CTAs among which fb_op_attention of these sizes
- * (head_dim 128, 16-byte aligned rows) cuts its items by key range, 0 where none is cut. */
+ * (head_dim 128, 16-byte aligned rows) cuts its items by key range, 0 where none is cut.
+ * fb_test_plan_traffic (host only): what fb_draft's cache of block contributions takes under a
+ * plan whose residual stream has `elems` elements: *slots = its size in bf16 copies of the
+ * stream, *n_sums = sums of proxied runs formed in place of contributions, *bytes = memory
+ * traffic per element of writing and reading both. elems = 1: contributions alone (a sum's
+ * launches never pay); elems = 0: launches count nothing. */
 /* fb_probe_mma_rate: the tensor pipe's sustained rate on the current device, in MACs per SM
  * clock: every SM times (clock64) `reps` tcgen05.mma kind::f16 instructions of M = 128,
  * K = 16 and width n (64, 128 or 256) issued by each of `issuers` warps (1-4,
@@ -440,6 +445,9 @@ fb_status fb_test_fail_alloc(long k);
 long fb_test_alloc_calls(void);
 fb_status fb_test_poison_counters(fb_model* m);
 fb_status fb_test_request_handover(fb_model* m, int on);
+fb_status fb_test_plan_traffic(const fb_cfg* cfg, const float* schedule, int n_steps,
+                               const uint8_t* skip_mask, const int32_t* proxy_plan, size_t elems,
+                               int* slots, int* n_sums, double* bytes);
 fb_status fb_test_attention_split(fb_model* m, int batch, int Lq, int Lkv, int heads, int impl,
                                   int* ctas);
 

@@ -20,7 +20,6 @@
 #include <atomic>
 #include <mutex>
 #include <thread>
-#include <tuple>
 #include <string>
 #include <vector>
 
@@ -531,13 +530,14 @@ struct Action {
   int type;
   int layer;  // compute: layer
   int slot;   // compute: anchor slot for Delta, -1 = none; sum begin / end: the sum
+  int base;   // sum end: the sum whose slot holds the stream before the run
   std::vector<std::pair<int, double>> terms;      // proxy: (slot, coefficient)
   std::vector<std::pair<int, double>> sum_terms;  // proxy: (sum, coefficient)
 };
-// A proxied run of layers whose contributions are always needed together (the same anchors,
-// so the same weights, and nothing else computed between them at the anchors' steps) uses
-// their sum, h behind the run minus h before it: one fp32 array per anchor step in place of a
-// bf16 array per layer.
+// A proxied run of layers whose contributions are needed together (the same anchors, so the same
+// weights, and nothing else computed between them at the anchors' steps) can use their sum, h
+// behind the run minus h before it: one fp32 array per anchor step in place of a bf16 array per
+// layer.
 struct Plan {
   std::vector<std::vector<Action>> steps;
   int n_slots = 0;
@@ -549,15 +549,71 @@ struct Plan {
   std::vector<int> warm_src;
 };
 
+// The sum of layers first .. last at one anchor step (`count` contributions)
+struct Sum {
+  int first, last, count;
+  int uses, last_use;  // proxied runs that take it, the last one's step
+  int slot, base;      // its place; whose place holds the stream before it
+  bool on;             // taken in place of its layers' contributions
+};
+// Bytes of memory traffic per element of the residual stream: a contribution is written from the
+// old stream's rows (4 + 2) and read by each use (2); a sum copies the stream before its run (8,
+// once for all that begin at one layer), subtracts it from the stream behind (12) and is read by
+// each use (4). Each of a sum's launches takes the time of 14 MB (2 us) beside its bytes.
+constexpr double DELTA_BYTES = 6, DELTA_USE = 2, SUM_BEGIN = 8, SUM_END = 12, SUM_USE = 4;
+constexpr double SUM_LAUNCH_BYTES = 14e6;
+// Sets which of one anchor step's sums to take. alone: the layers whose contributions are needed
+// whatever the sums; computed: the layers computed at the step. Starts with every sum, drops the
+// ones that do not pay, given the others, until all do, and takes none if contributions alone
+// are as cheap. Returns what the sums save. Wan2.1-1.3B, two candidates: the searched plan (runs
+// of 22 and 6 blocks) 7580 -> 828 bytes an element, 86.7 -> 80.7 ms; the pool's random plan (runs
+// of 2 to 4 used once) keeps its contributions, 400 bytes, where a sum for each run made 472.
+double choose_sums(std::vector<Sum>& sums, const std::vector<char>& alone,
+                   const std::vector<char>& computed, double launch_bytes) {
+  const int L = (int)alone.size();
+  std::vector<int> need(alone.begin(), alone.end()), begins(L, 0);
+  double saves = 0;  // of the sums taken against contributions alone
+  for (auto& e : sums) {
+    e.on = true;
+    ++begins[e.first];
+    saves += DELTA_USE * e.count * e.uses - (SUM_END + SUM_USE * e.uses + launch_bytes);
+  }
+  for (int l = 0; l < L; ++l) {
+    if (begins[l]) saves -= SUM_BEGIN + launch_bytes;
+    bool covered = false;
+    for (const auto& e : sums) covered |= e.first <= l && l <= e.last;
+    if (covered && computed[l] && !need[l]) saves += DELTA_BYTES;
+  }
+  for (bool changed = true; changed;) {
+    changed = false;
+    for (auto& e : sums) {
+      if (!e.on) continue;
+      double gain = SUM_END + SUM_USE * e.uses + launch_bytes - DELTA_USE * e.count * e.uses;
+      if (begins[e.first] == 1) gain += SUM_BEGIN + launch_bytes;
+      for (int l = e.first; l <= e.last; ++l)
+        if (computed[l] && !need[l]) gain -= DELTA_BYTES;
+      if (gain < 0) continue;
+      e.on = false;
+      changed = true;
+      saves += gain;
+      --begins[e.first];
+      for (int l = e.first; l <= e.last; ++l) need[l] += computed[l];
+    }
+  }
+  if (saves <= 0)
+    for (auto& e : sums) e.on = false;
+  return saves;
+}
+
+// elems: elements of the residual stream (0: launches count nothing)
 fb_status analyse_plan(const fb_cfg& c, const float* sched, int S, const uint8_t* skip,
-                       const int32_t* proxy, Plan* out, bool keep = false) {
+                       const int32_t* proxy, Plan* out, size_t elems, bool keep = false) {
   const int L = c.depth;
   auto is_skip = [&](int k, int l) { return skip && skip[(size_t)k * L + l] != 0; };
   auto code = [&](int k, int l) { return proxy ? proxy[(size_t)k * L + l] : -1; };
-  // computed steps per layer; anchors per proxy; last use per (step, layer)
+  // computed steps per layer; anchors per proxy
   std::vector<std::vector<int>> computed(L);
   std::map<std::pair<int, int>, std::vector<int>> anchors;
-  std::map<std::pair<int, int>, int> last_use;  // (step, layer) -> last proxy step using it
   for (int k = 0; k < S; ++k)
     for (int l = 0; l < L; ++l) {
       const int32_t cd = code(k, l);
@@ -580,16 +636,11 @@ fb_status analyse_plan(const fb_cfg& c, const float* sched, int S, const uint8_t
     }
   // Runs of proxied layers with one anchor list whose contributions at every anchor's step
   // followed directly on one another (only skipped layers between them there); skipped
-  // layers do not end a run. A run of two or more becomes one term per anchor step, the sum
-  // over its layers.
-  struct Sum {
-    int step, first, last;  // contributions of layers first .. last computed at step
-    bool operator<(const Sum& o) const {
-      return std::tie(step, first, last) < std::tie(o.step, o.first, o.last);
-    }
-  };
-  std::map<Sum, int> sum_last;                  // -> last proxy step using it
-  std::map<std::pair<int, int>, int> run_last;  // (step, first layer of a summed run) -> last
+  // layers do not end a run. A run of two or more can be one term per anchor step, the sum
+  // over its layers; at each anchor step the sums that pay (choose_sums) are taken.
+  std::vector<std::vector<Sum>> sums(S);        // by anchor step
+  std::map<std::pair<int, int>, int> run_last;  // (step, first layer of a run) -> last
+  std::map<std::pair<int, int>, std::vector<int>> uses;  // (step, layer) -> its use by proxies
   for (int k = 0; k < S; ++k)
     for (int l = 0; l < L;) {
       if (is_skip(k, l) || code(k, l) == -1) { ++l; continue; }
@@ -604,48 +655,99 @@ fb_status analyse_plan(const fb_cfg& c, const float* sched, int S, const uint8_t
         last = q;
         ++count;
       }
-      if (count > 1) {
-        run_last[{k, l}] = last;
-        for (int s : an) sum_last[Sum{s, l, last}] = k;
-      } else {
-        for (int s : an) last_use[{s, l}] = k;
+      if (count > 1) run_last[{k, l}] = last;
+      for (int s : an) {
+        if (count > 1) {
+          auto& at = sums[s];
+          auto it = std::find_if(at.begin(), at.end(), [&](const Sum& e) {
+            return e.first == l && e.last == last;
+          });
+          if (it == at.end()) it = at.insert(at.end(), Sum{l, last, count, 0, 0, -1, -1, false});
+          ++it->uses;
+          it->last_use = k;
+        } else {
+          uses[{s, l}].push_back(k);
+        }
       }
       l = last + 1;
     }
-  // the cached state: each layer's last computed contribution stays until the end
-  if (keep)
-    for (int l = 0; l < L; ++l)
-      if (!computed[l].empty()) last_use[{computed[l].back(), l}] = S;
-  // sums take slots from one pool, in step order
-  std::map<Sum, int> sum_slot;
-  std::vector<int> sum_free;  // per sum slot: the step after which it is free
-  for (const auto& e : sum_last) {
-    int i = 0;
-    while (i < (int)sum_free.size() && sum_free[i] >= e.first.step) ++i;
-    if (i == (int)sum_free.size()) sum_free.push_back(0);
-    sum_free[i] = e.second;
-    sum_slot[e.first] = i;
+  const double launch_bytes = elems ? SUM_LAUNCH_BYTES / (double)elems : 0;
+  std::vector<std::pair<double, int>> saved;  // anchor steps with sums, by what these save
+  for (int s = 0; s < S; ++s) {
+    std::vector<char> alone(L), computed_at(L);
+    for (int l = 0; l < L; ++l) {
+      alone[l] = uses.count({s, l}) != 0;
+      computed_at[l] = !is_skip(s, l) && code(s, l) == -1;
+    }
+    const double gain = choose_sums(sums[s], alone, computed_at, launch_bytes);
+    if (gain > 0) saved.push_back({gain, s});
   }
-  out->n_sums = (int)sum_free.size();
-  // slot assignment: per layer a pool; a slot is free once its last user has run
-  std::vector<std::vector<int>> free_at(L);  // per layer: for each slot, step after which it is free
+  std::sort(saved.begin(), saved.end());
+
+  // The cache's slots: per layer a pool of contributions, one pool of sums (two slots each); an
+  // entry is free once its last user has run.
   std::vector<int> slot_base(L, 0);
   std::map<std::pair<int, int>, int> slot_of;  // (step, layer) -> local slot
-  for (int k = 0; k < S; ++k)
-    for (int l = 0; l < L; ++l) {
-      auto lu = last_use.find({k, l});
-      if (lu == last_use.end()) continue;
-      auto& pool = free_at[l];
-      int s = -1;
-      for (size_t i = 0; i < pool.size(); ++i)
-        if (pool[i] < k) { s = (int)i; break; }
-      if (s < 0) { s = (int)pool.size(); pool.push_back(0); }
-      pool[s] = lu->second;
-      slot_of[{k, l}] = s;
+  auto assign_slots = [&](bool with_sums) {
+    std::map<std::pair<int, int>, int> last_use;  // (step, layer) -> last proxy step using it
+    auto use = [&](int s, int l, int k) {
+      int& e = last_use[{s, l}];
+      e = std::max(e, k);
+    };
+    for (const auto& e : uses) use(e.first.first, e.first.second, e.second.back());
+    out->n_sums = 0;
+    std::vector<int> sum_free;  // per sum slot: the step after which it is free
+    for (int s = 0; s < S; ++s) {
+      for (auto& e : sums[s])
+        if (e.on && with_sums) {
+          size_t i = 0;
+          while (i < sum_free.size() && sum_free[i] >= s) ++i;
+          if (i == sum_free.size()) sum_free.push_back(0);
+          sum_free[i] = e.last_use;
+          e.slot = (int)i;
+        } else {
+          for (int l = e.first; l <= e.last; ++l)
+            if (!is_skip(s, l)) use(s, l, e.last_use);
+        }
+      // where several begin at one layer, the longest one's slot holds the stream before them
+      for (auto& e : sums[s])
+        if (e.on && with_sums) {
+          const Sum* longest = &e;
+          for (const auto& o : sums[s])
+            if (o.on && o.first == e.first && o.last > longest->last) longest = &o;
+          e.base = longest->slot;
+        }
     }
-  int total = 0;
-  for (int l = 0; l < L; ++l) { slot_base[l] = total; total += (int)free_at[l].size(); }
-  out->n_slots = total;
+    out->n_sums = (int)sum_free.size();
+    // the cached state: each layer's last computed contribution stays until the end
+    if (keep)
+      for (int l = 0; l < L; ++l)
+        if (!computed[l].empty()) last_use[{computed[l].back(), l}] = S;
+    slot_of.clear();
+    std::vector<std::vector<int>> free_at(L);  // per layer and slot: the step after which it is free
+    for (const auto& e : last_use) {           // in step order
+      const int k = e.first.first;
+      auto& pool = free_at[e.first.second];
+      size_t i = 0;
+      while (i < pool.size() && pool[i] >= k) ++i;
+      if (i == pool.size()) pool.push_back(0);
+      pool[i] = e.second;
+      slot_of[e.first] = (int)i;
+    }
+    out->n_slots = 0;
+    for (int l = 0; l < L; ++l) { slot_base[l] = out->n_slots; out->n_slots += (int)free_at[l].size(); }
+    return out->n_slots + 2 * out->n_sums;
+  };
+  // no more memory than contributions alone: if need be, sums go, the least useful half of the
+  // steps at a time
+  const int slots_alone = assign_slots(false);
+  while (!saved.empty() && assign_slots(true) > slots_alone) {
+    const size_t drop = (saved.size() + 1) / 2;
+    for (size_t i = 0; i < drop; ++i)
+      for (auto& e : sums[saved[i].second]) e.on = false;
+    saved.erase(saved.begin(), saved.begin() + drop);
+  }
+  if (saved.empty()) assign_slots(false);
   out->keep_slot.assign(keep ? L : 0, -1);
   out->keep_tau.assign(keep ? L : 0, std::nanf(""));
   if (keep)
@@ -668,36 +770,41 @@ fb_status analyse_plan(const fb_cfg& c, const float* sched, int S, const uint8_t
   for (int k = 0; k < S; ++k) {
     auto& acts = out->steps[k];
     auto proxy_action = [&]() -> Action& {
-      if (acts.empty() || acts.back().type != ACT_PROXY) acts.push_back(Action{ACT_PROXY, -1, -1, {}, {}});
+      if (acts.empty() || acts.back().type != ACT_PROXY) acts.push_back(Action{ACT_PROXY, -1, -1, -1, {}, {}});
       return acts.back();
     };
     int run_end = -1;  // last layer of the summed run being passed
     for (int l = 0; l < L; ++l) {
       if (is_skip(k, l)) continue;  // Eq. 6: identity, no launch
       if (code(k, l) == -1) {
-        for (const auto& e : sum_slot)
-          if (e.first.step == k && e.first.first == l)
-            acts.push_back(Action{ACT_SUM_BEGIN, -1, e.second, {}, {}});
-        Action a{ACT_COMPUTE, l, -1, {}, {}};
+        for (const auto& e : sums[k])
+          if (e.on && e.first == l && e.base == e.slot)
+            acts.push_back(Action{ACT_SUM_BEGIN, -1, e.slot, -1, {}, {}});
+        Action a{ACT_COMPUTE, l, -1, -1, {}, {}};
         auto so = slot_of.find({k, l});
         if (so != slot_of.end()) a.slot = slot_base[l] + so->second;
         acts.push_back(a);
-        for (const auto& e : sum_slot)
-          if (e.first.step == k && e.first.last == l)
-            acts.push_back(Action{ACT_SUM_END, -1, e.second, {}, {}});
+        for (const auto& e : sums[k])
+          if (e.on && e.last == l)
+            acts.push_back(Action{ACT_SUM_END, -1, e.slot, e.base, {}, {}});
         continue;
       }
-      if (l <= run_end) continue;  // covered by the run's sums
+      if (l <= run_end) continue;  // covered by the run
       const auto& an = anchors[{k, l}];
       const std::vector<double> w = weights(an, sched[k]);
       const auto run = run_last.find({k, l});
+      run_end = run != run_last.end() ? run->second : l;
       Action& act = proxy_action();
+      std::vector<int> sum_of(an.size(), -1);  // the sums that stand for the run
+      for (size_t i = 0; i < an.size() && run_end > l; ++i)
+        for (const auto& e : sums[an[i]])
+          if (e.on && e.first == l && e.last == run_end) sum_of[i] = e.slot;
+      for (int q = l; q <= run_end; ++q)
+        for (size_t i = 0; i < an.size(); ++i)
+          if (!is_skip(k, q) && sum_of[i] < 0)
+            act.terms.push_back({slot_base[q] + slot_of[{an[i], q}], w[i]});
       for (size_t i = 0; i < an.size(); ++i)
-        if (run != run_last.end())
-          act.sum_terms.push_back({sum_slot[Sum{an[i], l, run->second}], w[i]});
-        else
-          act.terms.push_back({slot_base[l] + slot_of[{an[i], l}], w[i]});
-      if (run != run_last.end()) run_end = run->second;
+        if (sum_of[i] >= 0) act.sum_terms.push_back({sum_of[i], w[i]});
     }
   }
   return FB_OK;
@@ -717,10 +824,10 @@ void warm_plan(int L, int S, int warm, const std::vector<int>& slot_of, Plan* ou
       auto& acts = out->steps[k];
       if (k < warm && slot_of[l] >= 0) {
         if (acts.empty() || acts.back().type != ACT_PROXY)
-          acts.push_back(Action{ACT_PROXY, -1, -1, {}, {}});
+          acts.push_back(Action{ACT_PROXY, -1, -1, -1, {}, {}});
         acts.back().terms.push_back({slot_of[l], 1.0});
       } else {
-        acts.push_back(Action{ACT_COMPUTE, l, -1, {}, {}});
+        acts.push_back(Action{ACT_COMPUTE, l, -1, -1, {}, {}});
       }
     }
 }
@@ -831,15 +938,17 @@ fb_status sample(fb_model* m, float* z, int n, const float* sched, int S, const 
         CKS(wait_slot(m, a.slot, slot_elems));
         CKS(block_forward(m, a.layer, m->hA, nr, d, so.guided ? n : 0, cond));
       } else if (a.type == ACT_SUM_BEGIN || a.type == ACT_SUM_END) {
-        // sum = h, then sum = h - sum behind the run (fp32, two slots)
-        const int sl = plan.n_slots + 2 * a.slot;
-        if (a.type == ACT_SUM_BEGIN)
-          for (int i = 0; i < 2; ++i) CKS(wait_slot(m, sl + i, slot_elems));
+        // sum = h before the run, then sum = h - base behind it (fp32, two slots)
+        const bool end = a.type == ACT_SUM_END;
+        auto sum = [&](int i) {
+          return reinterpret_cast<float*>(m->anchors + (plan.n_slots + 2 * (size_t)i) * slot_elems);
+        };
+        if (!end || a.base != a.slot)  // its first write
+          for (int i = 0; i < 2; ++i)
+            CKS(wait_slot(m, plan.n_slots + 2 * a.slot + i, slot_elems));
         const size_t ne = (size_t)M * c.dim;
-        KTimer kt(m, FB_K_PROXY, a.type == ACT_SUM_END ? (double)ne : 0.0,
-                  ne * (a.type == ACT_SUM_END ? 12.0 : 8.0));
-        CK(run_sum(reinterpret_cast<float*>(m->anchors + (size_t)sl * slot_elems), m->hA, ne,
-                   a.type == ACT_SUM_END, m->st));
+        KTimer kt(m, FB_K_PROXY, end ? (double)ne : 0.0, ne * (end ? SUM_END : SUM_BEGIN));
+        CK(run_sum(sum(a.slot), m->hA, end ? sum(a.base) : nullptr, ne, m->st));
       } else {
         ProxyTerms pt{};
         double term_bytes = 0;
@@ -1269,7 +1378,8 @@ fb_status fb_draft_ex(fb_model* m, float* latents, int n, const float* text_ctx,
   if (!latents || !text_ctx) return fail(FB_EINVAL, "null latents or text_ctx");
   CKS(check_schedule(schedule, n_steps));
   Plan plan;
-  CKS(analyse_plan(m->c, schedule, n_steps, skip_mask, proxy_plan, &plan,
+  const size_t rows = (size_t)(opts && opts->text_uncond ? 2 * n : n) * m->P;
+  CKS(analyse_plan(m->c, schedule, n_steps, skip_mask, proxy_plan, &plan, rows * m->c.dim,
                    opts && opts->keep_state));
   return run_sampler(m, latents, n, text_ctx, schedule, n_steps, plan, opts);
 }
@@ -1304,7 +1414,7 @@ fb_status fb_refine_ex(fb_model* m, float* latent, const float* text_ctx,
     warm_plan(L, n_steps, opts->warm_steps, slot_of, &plan);
   } else {
     if (opts && opts->warm_steps < 0) return fail(FB_EINVAL, "warm_steps < 0");
-    CKS(analyse_plan(m->c, full_schedule, n_steps, nullptr, nullptr, &plan));
+    CKS(analyse_plan(m->c, full_schedule, n_steps, nullptr, nullptr, &plan, 0));
   }
   return run_sampler(m, latent, 1, text_ctx, full_schedule, n_steps, plan, opts);
 }
@@ -1750,6 +1860,27 @@ fb_status fb_test_poison_counters(fb_model* m) {
     CK(cudaMemsetAsync(m->attn_flags, 0x80, (size_t)m->dev_sms * ATTN_FLAGS_PER_CTA * sizeof(int),
                        st));
   CK(cudaStreamSynchronize(st));
+  return FB_OK;
+}
+
+fb_status fb_test_plan_traffic(const fb_cfg* cfg, const float* schedule, int n_steps,
+                               const uint8_t* skip_mask, const int32_t* proxy_plan, size_t elems,
+                               int* slots, int* n_sums, double* bytes) {
+  if (!cfg || !schedule || !slots || !n_sums || !bytes || n_steps < 1 || cfg->depth < 1)
+    return fail(FB_EINVAL, "null argument or bad sizes");
+  Plan plan;
+  CKS(analyse_plan(*cfg, schedule, n_steps, skip_mask, proxy_plan, &plan, elems));
+  *slots = plan.n_slots + 2 * plan.n_sums;
+  *n_sums = 0;
+  *bytes = 0;
+  for (const auto& acts : plan.steps)
+    for (const Action& a : acts) {
+      if (a.type == ACT_COMPUTE) *bytes += a.slot >= 0 ? DELTA_BYTES : 0;
+      if (a.type == ACT_SUM_BEGIN) *bytes += SUM_BEGIN;
+      if (a.type == ACT_SUM_END) *bytes += SUM_END;
+      *n_sums += a.type == ACT_SUM_END;
+      *bytes += DELTA_USE * a.terms.size() + SUM_USE * a.sum_terms.size();
+    }
   return FB_OK;
 }
 

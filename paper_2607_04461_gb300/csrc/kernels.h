@@ -87,8 +87,9 @@ struct ProxyTerms {
   unsigned long long f32_terms;
   int n;
 };
-// sum[i] = h[i], or with `end` h[i] - sum[i], over n_elems fp32 elements.
-cudaError_t run_sum(float* sum, const float* h, size_t n_elems, bool end, cudaStream_t st);
+// sum[i] = h[i] - base[i] (base null: h[i]), over n_elems fp32 elements; base may be sum.
+cudaError_t run_sum(float* sum, const float* h, const float* base, size_t n_elems,
+                    cudaStream_t st);
 cudaError_t proxy_add(float* h, size_t n_elems, const ProxyTerms& t, cudaStream_t st);
 // h[(b*P + tok)][:] = W_p * patch(z_b, tok) + b_p.
 cudaError_t patch_embed(const float* z, int n, int C, int H, int W, int p, const bf16* Wp,

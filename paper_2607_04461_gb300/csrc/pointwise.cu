@@ -197,19 +197,18 @@ __global__ void __launch_bounds__(256) proxy_add_kernel(float* __restrict__ h, s
 // run_sum: the sum of a run of blocks' contributions from the residual stream before and
 // behind it. Against a bf16 contribution per block (28 arrays of 9.6 MB at two 1560-token
 // candidates) a proxied step reads one fp32 array per anchor step: 84 terms, 118 us, become
-// 3 terms, 15 us, and the run's blocks write no contributions.
-__global__ void __launch_bounds__(256) run_sum_kernel(float* __restrict__ sum,
-                                                      const float* __restrict__ h, size_t n8,
-                                                      int end) {
+// 3 terms, 15 us, and the run's blocks write no contributions. base may be sum itself.
+__global__ void __launch_bounds__(256) run_sum_kernel(float* sum, const float* __restrict__ h,
+                                                      const float* base, size_t n8) {
   griddep_wait();
   griddep_launch();
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n8;
        i += (size_t)gridDim.x * blockDim.x) {
     float a[8];
     load_f32x8(h + i * 8, a);
-    if (end) {
+    if (base) {
       float b[8];
-      load_f32x8(sum + i * 8, b);
+      load_f32x8(base + i * 8, b);
 #pragma unroll
       for (int j = 0; j < 8; ++j) a[j] -= b[j];
     }
@@ -592,11 +591,12 @@ cudaError_t proxy_add(float* h, size_t n_elems, const ProxyTerms& t, cudaStream_
   return launch_k(proxy_add_kernel, dim3(grid_for(n8, 256)), dim3(256), 0, st, h, n8, t);
 }
 
-cudaError_t run_sum(float* sum, const float* h, size_t n_elems, bool end, cudaStream_t st) {
+cudaError_t run_sum(float* sum, const float* h, const float* base, size_t n_elems,
+                    cudaStream_t st) {
   if (n_elems == 0) return cudaSuccess;
   if (n_elems % 8) return cudaErrorInvalidValue;
-  return launch_k(run_sum_kernel, dim3(grid_for(n_elems / 8, 256)), dim3(256), 0, st, sum, h,
-                  n_elems / 8, end ? 1 : 0);
+  return launch_k(run_sum_kernel, dim3(grid_for(n_elems / 8, 256)), dim3(256), 0, st, sum, h, base,
+                  n_elems / 8);
 }
 
 cudaError_t patch_embed(const float* z, int n, int C, int H, int W, int p, const bf16* Wp,

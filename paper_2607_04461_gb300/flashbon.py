@@ -56,7 +56,7 @@ EXPORTS = ["fb_weights_count", "fb_weights_entry", "fb_init_model", "fb_free", "
            "fb_state_wait", "fb_set_sm_budget", "fb_sm_split_create", "fb_sm_split_info",
            "fb_sm_split_free", "fb_pipeline_step", "fb_set_device_wait_limit",
            "fb_test_fail_alloc", "fb_test_alloc_calls", "fb_test_poison_counters",
-           "fb_test_request_handover", "fb_test_attention_split",
+           "fb_test_request_handover", "fb_test_attention_split", "fb_test_plan_traffic",
            "fb_probe_mma_rate", "fb_probe_mma_gap", "fb_probe_mufu", "fb_probe_tmem_load",
            "fb_probe_mma_mix"]
 
@@ -114,6 +114,8 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
         "fb_test_alloc_calls": (ctypes.c_long, []),
         "fb_test_poison_counters": (I, [P]),
         "fb_test_request_handover": (I, [P, I]),
+        "fb_test_plan_traffic": (I, [ctypes.POINTER(fb_cfg), P, I, P, P, S, ctypes.POINTER(I),
+                                     ctypes.POINTER(I), ctypes.POINTER(D)]),
         "fb_test_attention_split": (I, [P, I, I, I, I, I, ctypes.POINTER(I)]),
         "fb_probe_mma_rate": (I, [I, I, I, ctypes.POINTER(ctypes.c_double)]),
         "fb_probe_mma_gap": (I, [I, ctypes.POINTER(ctypes.c_double)]),
@@ -396,6 +398,19 @@ def fb_test_poison_counters(model) -> None:
     """Sets the stream-K counters of `model` (None: the allocation-free entry point's) to
     a large negative value, so the next stream-K finisher's wait cannot complete."""
     _check(load_library().fb_test_poison_counters(model))
+
+
+def fb_test_plan_traffic(cfg, schedule, skip_mask, proxy_plan, elems):
+    """(slots, sums, bytes per element) of the contribution cache under a plan."""
+    sched = np.ascontiguousarray(schedule, np.float32)
+    skip = np.ascontiguousarray(skip_mask, np.uint8)
+    proxy = np.ascontiguousarray(proxy_plan, np.int32)
+    slots, sums, nbytes = ctypes.c_int(), ctypes.c_int(), ctypes.c_double()
+    c = make_cfg(cfg)
+    _check(load_library().fb_test_plan_traffic(
+        ctypes.byref(c), sched.ctypes.data, len(sched) - 1, skip.ctypes.data, proxy.ctypes.data,
+        int(elems), ctypes.byref(slots), ctypes.byref(sums), ctypes.byref(nbytes)))
+    return slots.value, sums.value, nbytes.value
 
 
 def fb_test_attention_split(model, batch, Lq, Lkv, heads, impl=0) -> int:

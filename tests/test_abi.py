@@ -24,6 +24,47 @@ def lib():
     return fb.load_library()
 
 
+def _own_plan(steps, every, frac, order, skip_frac, seed):
+    """A full step every `every`, the others proxy a random share of their blocks from it and
+    skip another."""
+    rng = np.random.default_rng(seed)
+    skip, proxy = synth.empty_plan(steps, synth.WAN13.depth)
+    for k in range(steps):
+        if k % every == 0:
+            continue
+        skip[k, rng.choice(skip.shape[1], int(skip.shape[1] * skip_frac), replace=False)] = 1
+        live = np.flatnonzero(skip[k] == 0)
+        for l in rng.permutation(live)[:int(round(frac * len(live)))]:
+            proxy[k, l] = synth.proxy_code(k // every * every, order)
+    return skip, proxy
+
+
+@pytest.mark.parametrize("steps,plan,sums,nbytes", [
+    (49, lambda: fb.fb_plan_from_phi(50, 49, 3, 22, 23, 5, 2, 30), 16, 828),  # the searched plan
+    (10, lambda: synth.random_plan(10, 30, 1 / 3, 0.5), 0, 400),
+    (50, lambda: _own_plan(50, 50, 0.8, 0, 0, 1), None, None),   # its own blocks at every step
+    (50, lambda: _own_plan(50, 10, 1.0, 2, 1 / 3, 2), None, None),  # its own skips
+    (40, lambda: _own_plan(40, 2, 1.0, 2, 0, 3), None, None),
+    (40, lambda: _own_plan(40, 5, 0.9, 1, 0.1, 4), None, None),
+    (40, lambda: _own_plan(40, 8, 1.0, 1, 0.05, 5), None, None),
+    (200, lambda: _own_plan(200, 40, 0.95, 1, 0.05, 6), None, None),
+])
+def test_sums_of_proxied_runs_pay(lib, steps, plan, sums, nbytes):
+    """Sums of proxied runs are formed only where they save memory traffic, and never take
+    more room than contributions alone."""
+    cfg = synth.WAN13
+    skip, proxy = plan()
+    sched = synth.make_schedule(max(50, steps))[:steps + 1]
+    slots1, sums1, bytes1 = fb.fb_test_plan_traffic(cfg, sched, skip, proxy, 1)
+    assert sums1 == 0
+    for elems in (0, 1560 * 1536, 64 * 4096 * 1536):
+        slots, n_sums, traffic = fb.fb_test_plan_traffic(cfg, sched, skip, proxy, elems)
+        assert slots <= slots1
+        assert traffic < bytes1 if n_sums else traffic == bytes1
+        if sums is not None:
+            assert n_sums == sums and traffic <= nbytes
+
+
 def declared_functions():
     names = []
     for f in os.listdir(os.path.join(ROOT, "include")):

@@ -137,7 +137,8 @@ def test_runs_of_proxied_blocks_use_their_sum():
     orders 0 and 2; a run split where a block computed at the anchor's step is skipped
     later; nested and overlapping runs from one step; a run broken by a computed block; a
     single proxied block (its own contribution). The same plan with every block's state kept
-    (no sums) agrees too."""
+    (no sums) agrees too. (At 150 tokens a sum's launches do not pay, so the runs here are cut
+    into their blocks; the next test's are not.)"""
     cfg = synth.SMALL.with_(depth=6, max_n=2)
     w = synth.make_weights(cfg, bf16=True, norm_std=0.2)
     S, c = 9, synth.proxy_code
@@ -158,6 +159,34 @@ def test_runs_of_proxied_blocks_use_their_sum():
     sched = synth.make_schedule(12)[:S + 1]
     ref = O.OracleModel(cfg, w)
     want = ref.draft(z, ctx, sched, skip, proxy)
+    with fb.Model(cfg, w) as m:
+        for opts in (None, fb.make_opts(keep_state=True)):
+            zd = cuda(z)
+            m.draft(zd, ctx, sched, skip, proxy, opts=opts)
+            for j in range(2):
+                check_latents(zd.cpu().numpy()[j], want[j], z[j], label=f"sums cand {j}")
+
+
+def test_runs_of_proxied_blocks_sums_that_pay():
+    """A plan on which sums pay (1536 tokens): two sums of one step with the same beginning
+    (blocks 0-5 and 0-3, one copy of the stream before them), first-order runs of blocks 0-3
+    and 4-5 with different second anchors, a run around a skipped block. Against the oracle, and
+    the same plan with every block's state kept (no sums)."""
+    cfg = synth.SMALL.with_(depth=6, max_n=2, latent_h=64, latent_w=96)
+    S, c = 41, synth.proxy_code
+    skip, proxy = synth.empty_plan(S, cfg.depth)
+    proxy[1:11] = c(0, 0)
+    proxy[11:21, :4] = c(0, 0)        # 4-5 computed
+    proxy[22:32] = c(21, 1)           # 0-3 from steps 21 and 0, 4-5 from 21 and 20
+    skip[32:, 2] = 1                  # step 32 computes the rest
+    proxy[33:41] = c(32, 0)
+    proxy[32:, 2] = -1
+    sched = synth.make_schedule(60)[:S + 1]
+    elems = 2 * cfg.tokens * cfg.dim
+    assert fb.fb_test_plan_traffic(cfg, sched, skip, proxy, elems)[:2] == (8, 4)
+    w = synth.make_weights(cfg, bf16=True, norm_std=0.2)
+    z, ctx = synth.make_latents(cfg, 2), synth.make_text(cfg)
+    want = O.OracleModel(cfg, w).draft(z, ctx, sched, skip, proxy)
     with fb.Model(cfg, w) as m:
         for opts in (None, fb.make_opts(keep_state=True)):
             zd = cuda(z)
