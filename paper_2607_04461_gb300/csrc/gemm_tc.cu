@@ -1035,28 +1035,40 @@ TileChoice choose_tile(int M, int N, int nk, int mc, bool f32) {
   return best;
 }
 
+// Clusters of the 2-SM kernel that the current device can hold at once (pairs must share a GPC),
+// asked once per device for the whole device, whatever SM budget the first launch has; without an
+// answer, the launch's SMs in pairs.
+template <int KIND>
+int resident_clusters(int num_sms) {
+  constexpr int DEVICES = 64;
+  static std::atomic<int> known[DEVICES];  // zero until a launch has asked (any thread)
+  int dev = 0, sms = 0, n = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && dev < DEVICES) {
+    n = known[dev].load(std::memory_order_relaxed);
+    if (n > 0) return n;
+  }
+  cudaLaunchConfig_t cfg = {};
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
+    cfg.gridDim = dim3(sms / 2 * 2, 1, 1);
+    cfg.blockDim = dim3(C2_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = C2_SMEM_BYTES;
+    if (cudaOccupancyMaxActiveClusters(&n, gemm_tc2_kernel<KIND>, &cfg) == cudaSuccess && n > 0) {
+      if (dev < DEVICES) known[dev].store(n, std::memory_order_relaxed);
+      return n;
+    }
+  }
+  cudaGetLastError();
+  return num_sms / 2;
+}
+
 template <int KIND>
 cudaError_t launch2(const GemmArgs& g, int* err, int num_sms, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(gemm_tc2_kernel<KIND>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, C2_SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  // as many clusters as can be resident at once (pairs must share a GPC), and no more than
-  // the num_sms SMs this launch may use allow
-  static std::atomic<int> occ_clusters[4];  // zero until a launch has asked (any thread)
-  int occ = occ_clusters[KIND].load(std::memory_order_relaxed);
-  if (occ == 0) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(num_sms, 1, 1);
-    cfg.blockDim = dim3(C2_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = C2_SMEM_BYTES;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_tc2_kernel<KIND>, &cfg) != cudaSuccess || n < 1) {
-      cudaGetLastError();
-      n = num_sms / 2;
-    }
-    occ = n;
-    occ_clusters[KIND].store(n, std::memory_order_relaxed);
-  }
+  // as many clusters as can be resident at once, and no more than the num_sms SMs that this launch
+  // may use allow
+  const int occ = resident_clusters<KIND>(num_sms);
   const int mc = occ < num_sms / 2 ? occ : num_sms / 2;
   const int nk = g.K / BK;
   // Stream-K automatically (sk_mode 0, the single-op calls) only for a few rounds of

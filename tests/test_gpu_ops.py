@@ -2,6 +2,10 @@
 epilogues, ragged M, both N tile widths), the CUDA-core GEMM, and flash attention
 (self / shared-K/V cross, head_dim 64 and 128, ragged tails) against the oracle's fp64
 primitives on the same bf16 inputs."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -12,6 +16,8 @@ from paper_2607_04461_gb300 import synth
 from _metrics import rel_max
 
 pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -238,6 +244,35 @@ def test_gemm_stream_k_forced_rejects(model, M, N, K):
         fb.fb_op_gemm(model.handle, M, N, K, A, W, None, 0, out, None, None, None, None, 4)
     assert e.value.status == fb.FB_ECUDA
     _gemm_case(model, M, N, K, 0, impl=0)   # the model is still usable
+
+
+@pytest.mark.parametrize("budget", [3, 40])
+def test_gemm_first_call_on_few_sms(budget):
+    """The resident-cluster count is the device's, also when a process's first launch has a small
+    or odd SM budget: on the whole device the stream-K split then still refuses a shape with
+    fewer than four K blocks per SM pair (4 K blocks in all)."""
+    code = f"""
+import torch
+from paper_2607_04461_gb300 import flashbon as fb, synth
+m = fb.Model(synth.TINY, synth.make_weights(synth.TINY))
+A, W = (torch.randn(n, 128).bfloat16().cuda() for n in (300, 256))
+out = torch.empty(300, 256, dtype=torch.bfloat16, device="cuda")
+run = lambda impl: fb.fb_op_gemm(m.handle, 300, 256, 128, A, W, None, 0, out, None, None, None, None, impl)
+m.set_sm_budget({budget})
+run(3)
+m.set_sm_budget(0)
+try:
+    run(4)
+    raise SystemExit("split taken")
+except fb.FlashBonError as e:
+    assert e.status == fb.FB_ECUDA
+run(3)
+torch.cuda.synchronize()
+assert ((out.float() - A.float() @ W.float().T).abs().max() < 0.5).item()
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
 
 
 @pytest.mark.parametrize("M,N,K", [(300, 256, 128), (77, 24, 40)])
