@@ -317,7 +317,8 @@ const char* fb_kernel_name(int kind);
  * (ceil(M / 256) * N / 256 * K / 64 >= 4 * pairs), else FB_ECUDA; impl 0 takes the
  * stream-K split only when the 256 x 256 tiles fill at most 4 rounds of the resident SM
  * pairs and leave at least 24 K blocks per pair idle in the last (e.g. 1560 x 1536 x 8960),
- * whole tiles otherwise. */
+ * and A and W together are at most 64 MiB or M <= 256 (2304 x 1536 x 8960 is past that),
+ * whole tiles in one K chain otherwise. */
 /* fb_set_op_repeat: fb_op_gemm / fb_op_attention launch their kernel n >= 1 times back
  * to back (default 1), for timing a kernel without a stream synchronisation per launch. */
 fb_status fb_set_op_repeat(fb_model* m, int n);

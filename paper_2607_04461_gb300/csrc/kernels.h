@@ -30,7 +30,8 @@ constexpr size_t SK_WS_FLOATS_PER_CLUSTER = 2 * 2 * 8 * 4096;
 constexpr int SK_CTR_PER_CLUSTER = 16;
 constexpr int SK_HANDOVER = 1 << 30;  // a counter's bit: see sk_wait_all
 // tcgen05 path: requires N % 128 == 0, K % 64 == 0, 16-byte aligned rows. Uses the
-// 2-SM (cta_group::2) kernel when N % 256 == 0 unless force_1sm.
+// 2-SM (cta_group::2) kernel unless force_1sm or N % 256 == 128 with a short K or few or, at
+// N = 128, many rows (see its dispatch).
 bool gemm_tc_supported(const GemmArgs& g);
 cudaError_t gemm_tc(const GemmArgs& g, int* err, int num_sms, cudaStream_t st,
                     bool force_1sm = false);

@@ -205,10 +205,13 @@ def test_gemm_stream_k_handover(M, N, K, epi):
     (1560, 1536, 1536, 3),   # 24 K blocks: whole tiles
     (49920, 1536, 8960, 3),  # more tiles than SM pairs: whole tiles
     (8192, 1536, 8960, 3),   # 2.5 rounds but A and W (166 MB) larger than half of L2
+    (2304, 1536, 8960, 3),   # one round, 40 idle K blocks a pair, but A and W are 68.8 MB
+    (256, 5120, 13824, 4),   # 149 MB, but one row of tiles
 ])
 def test_gemm_automatic_stream_k_choice(model, M, N, K, twin):
-    """impl 0 takes the stream-K split only for a long K under one wave of pair tiles: its
-    result is bit-identical to the forced variant it chose."""
+    """impl 0 takes the stream-K split where the last of at most four rounds of pair tiles
+    leaves many K blocks idle and the operands are small or M is: its result is bit-identical
+    to the forced variant it chose."""
     A = randn((M, K), 51)
     W = randn((N, K), 52, scale=K ** -0.5)
     resid = randn((M, N), 53, dtype=torch.float32)
