@@ -396,7 +396,8 @@ fb_status run_attn(fb_model* m, const AttnArgs& a0, int kind, int impl = 0) {
 fb_status run_ln(fb_model* m, const float* x, bf16* out, int rows, float mb, const float* mul,
                  const float* add) {
   KTimer t(m, FB_K_NORM, 8.0 * rows * m->c.dim, 6.0 * rows * m->c.dim);
-  CK(ln_mod(x, out, rows, m->c.dim, m->c.eps_ln, mb, mul, add, m->st));
+  CK(ln_mod(x, out, rows, m->c.dim, m->c.eps_ln, mb, mul, add,
+            norm_few_rows(m->num_sms, m->num_sms == m->dev_sms), m->st));
   return FB_OK;
 }
 
@@ -404,7 +405,7 @@ fb_status run_qkn(fb_model* m, bf16* x, int rows, int ld, int nseg, int dcol, co
                   ptrdiff_t dw, const float2* rope) {
   KTimer t(m, FB_K_QKNORM, 6.0 * rows * nseg * m->c.dim, 4.0 * rows * nseg * m->c.dim);
   CK(qk_norm_rope(x, rows, ld, m->c.dim, nseg, dcol, w0, dw, m->c.eps_rms, rope, m->P,
-                  m->c.head_dim, m->st));
+                  m->c.head_dim, norm_few_rows(m->num_sms, m->num_sms == m->dev_sms), m->st));
   return FB_OK;
 }
 

@@ -72,13 +72,15 @@ int attention_tc_split(const AttnArgs& a);
 // ---- pointwise / small kernels ------------------------------------------------------
 // out[r][:] = bf16(LN(x[r][:]) * (mul_base + mul[:]) + add[:]), x fp32 [rows][D].
 cudaError_t ln_mod(const float* x, bf16* out, int rows, int D, float eps, float mul_base,
-                   const float* mul, const float* add, cudaStream_t st);
+                   const float* mul, const float* add, int few_rows, cudaStream_t st);
 // In place on bf16 rows, for each segment s < nseg (at most 65535): x[r][s dcol + :D] =
 // RMSNorm(.) * w0[s dw + :], then (if rope != null) RoPE with table rope[(r % tokens)]
 // [head_dim/2] of (cos, sin) per adjacent pair.
 cudaError_t qk_norm_rope(bf16* x, int rows, int ld, int D, int nseg, int dcol, const float* w0,
                          ptrdiff_t dw, float eps, const float2* rope, int tokens, int head_dim,
-                         cudaStream_t st);
+                         int few_rows, cudaStream_t st);
+// Rows up to which the two above run in the form for few rows (same results).
+int norm_few_rows(int sms, bool whole_device);
 // h[i] += sum_t coef[t] * anchor_t[i] over n_elems fp32 elements; anchors are bf16, or fp32
 // where bit t of f32_terms is set.
 #define FB_PROXY_MAX_TERMS 64

@@ -33,7 +33,7 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
 
 // ---------------------------------------------------------------------------------
 // ln_mod: THREADS threads per row, VPT float4 per thread (D = 4 * VPT * THREADS), ROWS
-// rows per block (ROWS > 1 only with one warp per row). EARLY: see FEW_ROWS.
+// rows per block (ROWS > 1 only with one warp per row). EARLY: see norm_few_rows.
 template <int THREADS, int VPT, int ROWS, bool EARLY>
 __global__ void __launch_bounds__(THREADS * ROWS) ln_mod_kernel(const float* __restrict__ x,
                                                                 bf16* __restrict__ out, int rows,
@@ -509,12 +509,16 @@ int grid_for(size_t work, int threads) {
 // Row kernels (ln_mod, qk_norm_rope): with few rows a launch is one or two waves of blocks and
 // its time is latency, so the row's parameters load together with the row (EARLY, 160
 // registers) instead of after its reductions; with many rows that occupancy costs more than
-// the latency. One candidate refined for two steps: 10.73 ms, 10.51 with ln_mod EARLY, 10.42
-// with both; two candidates 16.73 -> 16.48; three 21.56 -> 21.47; eight 52.2 -> 52.5.
-constexpr int FEW_ROWS = 32 * 152;
+// the latency. The caller says up to how many rows (norm_few_rows). One candidate refined for
+// two steps: 10.73 ms, 10.51 with ln_mod EARLY, 10.42 with both; two candidates 16.73 -> 16.48;
+// three 21.56 -> 21.47; eight 52.2 -> 52.5. On an SM partition the line lies lower, at one wave
+// of EARLY blocks (12 rows an SM); four refine steps, without / with EARLY: 384 rows on 112 SMs
+// 14.34 / 13.61 ms, on 64 16.64 / 15.91, on 40 18.14 / 17.61; 1560 rows on 112 SMs 23.34 / 23.40,
+// on 40 49.11 / 49.52; 3072 rows on 64 59.62 / 60.94, on 16 200.1 / 203.1.
+int norm_few_rows(int sms, bool whole_device) { return (whole_device ? 32 : 12) * sms; }
 
 cudaError_t ln_mod(const float* x, bf16* out, int rows, int D, float eps, float mul_base,
-                   const float* mul, const float* add, cudaStream_t st) {
+                   const float* mul, const float* add, int few_rows, cudaStream_t st) {
   if (rows == 0) return cudaSuccess;
   switch (D) {  // threads * 4 * VPT == D
     case 128: return ln_mod_launch<32, 1>(x, out, rows, D, eps, mul_base, mul, add, st);
@@ -524,14 +528,14 @@ cudaError_t ln_mod(const float* x, bf16* out, int rows, int D, float eps, float 
     // one warp per row, reductions by shuffles only: 5.93 TB/s with two rows per block against
     // 5.44 with 128 threads per row on the 16-candidate probe (24960 rows)
     case 1536:
-      return rows <= FEW_ROWS
+      return rows <= few_rows
                  ? ln_mod_launch<32, 12, 4, true>(x, out, rows, D, eps, mul_base, mul, add, st)
                  : ln_mod_launch<32, 12, 2>(x, out, rows, D, eps, mul_base, mul, add, st);
     case 2048: return ln_mod_launch<128, 4>(x, out, rows, D, eps, mul_base, mul, add, st);
     case 3072: return ln_mod_launch<256, 3>(x, out, rows, D, eps, mul_base, mul, add, st);
     case 4096: return ln_mod_launch<256, 4>(x, out, rows, D, eps, mul_base, mul, add, st);
     case 5120:
-      return rows <= FEW_ROWS
+      return rows <= few_rows
                  ? ln_mod_launch<256, 5, 1, true>(x, out, rows, D, eps, mul_base, mul, add, st)
                  : ln_mod_launch<256, 5>(x, out, rows, D, eps, mul_base, mul, add, st);
   }
@@ -540,7 +544,7 @@ cudaError_t ln_mod(const float* x, bf16* out, int rows, int D, float eps, float 
 
 cudaError_t qk_norm_rope(bf16* x, int rows, int ld, int D, int nseg, int dcol, const float* w0,
                          ptrdiff_t dw, float eps, const float2* rope, int tokens, int head_dim,
-                         cudaStream_t st) {
+                         int few_rows, cudaStream_t st) {
   if (rows == 0) return cudaSuccess;
 #define QKN(T, V, ...) \
   qkn_launch<T, V, ##__VA_ARGS__>(x, rows, ld, D, nseg, dcol, w0, dw, eps, rope, tokens, head_dim, st)
@@ -553,11 +557,11 @@ cudaError_t qk_norm_rope(bf16* x, int rows, int ld, int D, int nseg, int dcol, c
     // 16-candidate probe (24960 rows x 2 x 1536) 5.04 TB/s against 4.90 with two rows
     // per block and 4.60 with eight (at 49920 rows two rows per block gave 6.1 TB/s, one
     // row 5.4)
-    case 1536: return rows <= FEW_ROWS ? QKN(32, 12, 4, true) : QKN(32, 12, 4);
+    case 1536: return rows <= few_rows ? QKN(32, 12, 4, true) : QKN(32, 12, 4);
     case 2048: return QKN(128, 4);
     case 3072: return QKN(256, 3);
     case 4096: return QKN(256, 4);
-    case 5120: return rows <= FEW_ROWS ? QKN(256, 5, 1, true) : QKN(256, 5);
+    case 5120: return rows <= few_rows ? QKN(256, 5, 1, true) : QKN(256, 5);
   }
 #undef QKN
   return cudaErrorInvalidValue;
