@@ -725,8 +725,9 @@ fb_status analyse_plan(const fb_cfg& c, const float* sched, int S, const uint8_t
       for (int l = 0; l < L; ++l)
         if (!computed[l].empty()) last_use[{computed[l].back(), l}] = S;
     slot_of.clear();
-    std::vector<std::vector<int>> free_at(L);  // per layer and slot: the step after which it is free
-    for (const auto& e : last_use) {           // in step order
+    // per layer and slot: the step after which it is free
+    std::vector<std::vector<int>> free_at(L);
+    for (const auto& e : last_use) {  // in step order
       const int k = e.first.first;
       auto& pool = free_at[e.first.second];
       size_t i = 0;
@@ -736,7 +737,10 @@ fb_status analyse_plan(const fb_cfg& c, const float* sched, int S, const uint8_t
       slot_of[e.first] = (int)i;
     }
     out->n_slots = 0;
-    for (int l = 0; l < L; ++l) { slot_base[l] = out->n_slots; out->n_slots += (int)free_at[l].size(); }
+    for (int l = 0; l < L; ++l) {
+      slot_base[l] = out->n_slots;
+      out->n_slots += (int)free_at[l].size();
+    }
     return out->n_slots + 2 * out->n_sums;
   };
   // no more memory than contributions alone: if need be, sums go, the least useful half of the
@@ -771,7 +775,8 @@ fb_status analyse_plan(const fb_cfg& c, const float* sched, int S, const uint8_t
   for (int k = 0; k < S; ++k) {
     auto& acts = out->steps[k];
     auto proxy_action = [&]() -> Action& {
-      if (acts.empty() || acts.back().type != ACT_PROXY) acts.push_back(Action{ACT_PROXY, -1, -1, -1, {}, {}});
+      if (acts.empty() || acts.back().type != ACT_PROXY)
+        acts.push_back(Action{ACT_PROXY, -1, -1, -1, {}, {}});
       return acts.back();
     };
     int run_end = -1;  // last layer of the summed run being passed

@@ -234,7 +234,7 @@ __host__ __device__ __forceinline__ int c2_accs(int T) {
 }
 // Shared memory of a CTA: 2.5 KB less than an SM can give it, which lets two blocks of the
 // normalisation kernels that follow most GEMMs start beside it and wait there (1 KB each is
-// reserved by the system): one candidate's block 173.7 -> 172.3 us.
+// reserved by the system): one candidate's block 224.5 -> 221.9 us.
 constexpr int C2_SMEM_BYTES = 229888;
 // Epilogue tiles and operand ring per epilogue: each of the 8 epilogue warps owns NBUF tiles
 // of CHUNK tokens x 32 features, through which results leave by TMA store and (fp32 residual)
@@ -1104,11 +1104,12 @@ cudaError_t launch2(const GemmArgs& g, int* err, int num_sms, cudaStream_t st) {
   }
   bool use_sk = g.sk_mode == 2 || (g.sk_mode != 1 && sk_ok && sk_pays);
   // The model's own launches (sk_mode 3) take the faster of the two: a range of the split in
-  // the clocks of choose_tile and 15 % (full-width tiles stay short of the rate), then publishing, waiting for and summing the parts; a further
-  // accumulator about 1500. Measured (us, split / whole tiles): rows x 1536 x 8960, 32 rows
-  // 12.4 / 29.8, 256 18.6 / 31.0, 640 24.5 / 31.5, 1040 31.4 / 31.6, 1560 38.6 / 34.5; rows x
-  // 5120 x 5120, 100 rows 15.6 / 20.6, 256 22.2 / 22.4, 400 28.2 / 23.1. More than one round
-  // of tiles: whole (1040 x 5120 x 5120 50.3 / 44.7).
+  // the clocks of choose_tile and 15 % (full-width tiles stay short of the rate), then
+  // publishing, waiting for and summing the parts; a further accumulator about 1500. Measured
+  // (us, split / whole tiles): rows x 1536 x 8960, 32 rows 12.4 / 29.8, 256 18.6 / 31.0, 640
+  // 24.5 / 31.5, 1040 31.4 / 31.6, 1560 38.6 / 34.5; rows x 5120 x 5120, 100 rows 15.6 / 20.6,
+  // 256 22.2 / 22.4, 400 28.2 / 23.1. More than one round of tiles: whole (1040 x 5120 x 5120
+  // 50.3 / 44.7).
   if (g.sk_mode == 3 && use_sk) {
     const double range = (double)((tiles256 * nk + mc - 1) / mc);
     use_sk = rounds256 == 1 &&
