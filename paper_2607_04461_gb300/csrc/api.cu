@@ -675,6 +675,7 @@ fb_status analyse_plan(const fb_cfg& c, const float* sched, int S, const uint8_t
   const double launch_bytes = elems ? SUM_LAUNCH_BYTES / (double)elems : 0;
   std::vector<std::pair<double, int>> saved;  // anchor steps with sums, by what these save
   for (int s = 0; s < S; ++s) {
+    if (sums[s].empty()) continue;
     std::vector<char> alone(L), computed_at(L);
     for (int l = 0; l < L; ++l) {
       alone[l] = uses.count({s, l}) != 0;
@@ -751,8 +752,8 @@ fb_status analyse_plan(const fb_cfg& c, const float* sched, int S, const uint8_t
     for (size_t i = 0; i < drop; ++i)
       for (auto& e : sums[saved[i].second]) e.on = false;
     saved.erase(saved.begin(), saved.begin() + drop);
+    if (saved.empty()) assign_slots(false);
   }
-  if (saved.empty()) assign_slots(false);
   out->keep_slot.assign(keep ? L : 0, -1);
   out->keep_tau.assign(keep ? L : 0, std::nanf(""));
   if (keep)

@@ -353,7 +353,9 @@ __device__ __forceinline__ int sk_load(const int* ctr) {
 // waits (bounded) until `n` contributors are in
 __device__ __forceinline__ bool sk_wait(const int* ctr, int n, int* err) {
   const uint64_t t0 = fb_globaltimer();
+  uint32_t i = 0;
   for (int c; (c = sk_load(ctr)) < 0 || (c & SK_COUNT) != n;) {
+    if ((++i & 7u) != 0) continue;  // error word and clock now and then: short polls
     if (*(volatile int*)err != 0) return false;
     if (fb_globaltimer() - t0 > fb_wait_limit()) {
       fb_report(err, FB_DEVERR_WAIT_TIMEOUT);
@@ -370,12 +372,13 @@ __device__ __forceinline__ bool sk_wait(const int* ctr, int n, int* err) {
 enum { SK_GAVE_UP = 0, SK_SHARE, SK_HAND_OVER };
 __device__ __forceinline__ int sk_wait_all(int* ctr, int n, int* err) {
   const uint64_t t0 = fb_globaltimer();
-  while (true) {
+  for (uint32_t i = 1;; ++i) {
     const int c = sk_load(ctr);
     if (c >= 0) {
       if (c & SK_HANDOVER) return SK_HAND_OVER;
       if ((c & SK_COUNT) == n) return SK_SHARE;
     }
+    if ((i & 7u) != 0) continue;
     if (*(volatile int*)err != 0) return SK_GAVE_UP;
     const uint64_t waited = fb_globaltimer() - t0;
     if (waited > fb_wait_limit()) {
