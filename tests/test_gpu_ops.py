@@ -5,6 +5,7 @@ primitives on the same bf16 inputs."""
 import os
 import subprocess
 import sys
+import threading
 
 import numpy as np
 import pytest
@@ -197,6 +198,41 @@ def test_gemm_stream_k_handover(M, N, K, epi):
         assert torch.equal(out, outs[0][0])
         if epi == 3:
             assert torch.equal(delta, outs[0][1])
+
+
+def test_gemm_stream_k_on_several_streams():
+    """Models on streams of their own, each launch sized for the whole device: two tiles with 38
+    contributors each, so launches that run together can each hold part of a tile's pairs. Every
+    call ends (well inside the wait limit) with the result of a call alone, bit for bit."""
+    M, N, K, n = 200, 512, 9728, 4
+    A, W = randn((M, K), 67), randn((N, K), 68, scale=K ** -0.5)
+    models = [fb.Model(synth.TINY, synth.make_weights(synth.TINY)) for _ in range(n)]
+    outs = [torch.zeros((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(n + 1)]
+    call = lambda m, out: fb.fb_op_gemm(m.handle, M, N, K, A, W, None, 0, out, None, None,  # noqa: E731
+                                        None, None, 4)
+    call(models[0], outs[n])
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(i):
+        try:
+            fb.fb_set_op_repeat(models[i].handle, 40)
+            for _ in range(5):
+                call(models[i], outs[i])
+        except fb.FlashBonError as e:
+            errors.append(str(e))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(n)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for m in models:
+        m.close()
+    assert not errors
+    for out in outs[:n]:
+        assert torch.equal(out, outs[n])
 
 
 @pytest.mark.parametrize("M,N,K,twin", [
